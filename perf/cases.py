@@ -204,7 +204,7 @@ def work(case):
 
 def tolerance(case):
     # Probabilities are fp32 arithmetic on identical inputs whatever the storage type: against a softmax in
-    # 64 bits p, q and f differ by at most 2e-6 (relative, 2-norm).  A token or accepted length differs only
-    # where a uniform lies within a rounding error of an accept threshold or a boundary of the CDF: 0 to 3
-    # sequences in a thousand.
-    return {"rel": 1e-5, "max": 1e-4, "differ": 0.01}
+    # 64 bits p, q and f were seen to differ by up to 1.4e-7 (relative, 2-norm) and 7e-7 (largest).  A token or
+    # accepted length differs only where a uniform lies within a rounding error of an accept threshold or a
+    # boundary of the CDF: 0 to 3 sequences in a thousand, of which a small batch holds at most one.
+    return {"rel": 6e-7, "max": 3e-6, "differ": 0.01}
