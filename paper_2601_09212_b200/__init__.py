@@ -2,7 +2,8 @@
 
 Thin binding over the C ABI of ``libcsd.so`` (declared in ``include/csd.h``): the
 functions here have the ABI's names and only marshal arguments -- pointers of
-``torch`` tensors, sizes, the current CUDA stream.  Every step of the method
+``torch`` tensors, sizes, the current CUDA stream; for the calls a decoding loop
+makes every round, in C++ (``csrc/csd_bind.cpp``).  Every step of the method
 runs in the library's CUDA kernels.  There is no CPU fallback: if the library
 has not been built, or no CUDA device is present, calls raise.
 """
@@ -10,13 +11,14 @@ from __future__ import annotations
 
 import contextlib
 import ctypes as C
+import importlib.util
 import os
 from typing import Optional
 
 import numpy as np
 import torch
 
-from ._build import LIB_PATH
+from ._build import BIND_PATH, LIB_PATH
 
 CSD_F32, CSD_BF16 = 0, 1
 CSD_STATUS_BADROW, CSD_STATUS_BADTOKEN, CSD_STATUS_ZFALLBACK, CSD_STATUS_TIMEOUT = 1, 2, 4, 8
@@ -67,6 +69,31 @@ class csd_tree_params(C.Structure):
 
 
 _lib = None
+_bind = None        # the C++ marshalling module
+_addresses = {}     # of the loaded library's functions, by name
+
+
+def bind():
+    """The C++ marshalling module; raises if it has not been built."""
+    global _bind
+    if _bind is None:
+        if not os.path.exists(BIND_PATH):
+            raise RuntimeError(
+                f"{BIND_PATH} is missing: build it with `python -m paper_2601_09212_b200._build` "
+                "(there is no fallback path)")
+        spec = importlib.util.spec_from_file_location("_csd_bind", BIND_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _bind = mod
+    return _bind
+
+
+def _address(name: str) -> int:
+    """Address of a function of the library in use."""
+    a = _addresses.get(name)
+    if a is None:
+        a = _addresses[name] = C.cast(getattr(library(), name), C.c_void_p).value
+    return a
 
 
 def library() -> C.CDLL:
@@ -143,10 +170,12 @@ def checked_library():
         return tuple(rec)
 
     before, _lib = library(), lib
+    _addresses.clear()
     try:
         yield report
     finally:
         _lib = before
+        _addresses.clear()
 
 
 def error_string(code: int) -> str:
@@ -226,19 +255,8 @@ def _logit_dtype(t: torch.Tensor) -> int:
 def csd_verify(target_logits, draft_logits, draft_tokens, uniforms, relax_schedule, out_tokens,
                out_accept_len, stream=None) -> None:
     """Simple form: fp32 [B, gamma, V] logits; see ``csd_verify`` in csd.h."""
-    B, gamma, V = target_logits.shape
-    if draft_logits.shape != (B, gamma, V):
-        raise ValueError("target_logits and draft_logits must both be [B, gamma, V]")
-    rc = library().csd_verify(
-        _dev_ptr(target_logits, "target_logits", torch.float32),
-        _dev_ptr(draft_logits, "draft_logits", torch.float32),
-        _dev_ptr(draft_tokens, "draft_tokens", torch.int32),
-        _dev_ptr(uniforms, "uniforms", torch.float32),
-        _dev_ptr(relax_schedule, "relax_schedule", torch.float32),
-        B, gamma, V,
-        _dev_ptr(out_tokens, "out_tokens", torch.int32),
-        _dev_ptr(out_accept_len, "out_accept_len", torch.int32),
-        _stream_handle(stream))
+    rc = bind().verify(_address("csd_verify"), target_logits, draft_logits, draft_tokens, uniforms, relax_schedule,
+                       out_tokens, out_accept_len, stream)
     if rc != 0:
         raise CsdError(rc, "csd_verify")
 
@@ -250,19 +268,8 @@ def csd_verify_static(target_logits, draft_logits, draft_tokens, uniforms, relax
     and results, scratch taken from a fixed array inside the library, so nothing is allocated.
     Raises ``CsdError`` (code -8) when the problem needs more than ``CSD_STATIC_SCRATCH_BYTES``;
     calls on one device share that array and must not overlap on the GPU."""
-    B, gamma, V = target_logits.shape
-    if draft_logits.shape != (B, gamma, V):
-        raise ValueError("target_logits and draft_logits must both be [B, gamma, V]")
-    rc = library().csd_verify_static(
-        _dev_ptr(target_logits, "target_logits", torch.float32),
-        _dev_ptr(draft_logits, "draft_logits", torch.float32),
-        _dev_ptr(draft_tokens, "draft_tokens", torch.int32),
-        _dev_ptr(uniforms, "uniforms", torch.float32),
-        _dev_ptr(relax_schedule, "relax_schedule", torch.float32),
-        B, gamma, V,
-        _dev_ptr(out_tokens, "out_tokens", torch.int32),
-        _dev_ptr(out_accept_len, "out_accept_len", torch.int32),
-        _stream_handle(stream))
+    rc = bind().verify(_address("csd_verify_static"), target_logits, draft_logits, draft_tokens, uniforms, relax_schedule,
+                       out_tokens, out_accept_len, stream)
     if rc != 0:
         raise CsdError(rc, "csd_verify_static")
 
@@ -312,7 +319,7 @@ def make_params(target_logits, draft_logits, draft_tokens, uniforms, relax_sched
 
 
 def csd_verify_ex(params: csd_params) -> None:
-    rc = library().csd_verify_ex(C.byref(params))
+    rc = bind().call_block(_address("csd_verify_ex"), C.addressof(params))
     if rc != 0:
         raise CsdError(rc, "csd_verify_ex")
 
@@ -354,25 +361,11 @@ def csd_sample_rows(logits, uniforms, out_tokens, *, uncond=None, cfg_scale=1.0,
 
     ``logits`` (and ``uncond``, with the same strides) may be a view whose rows are contiguous but
     spaced apart, such as ``all_logits[:, -1]`` of a ``[B, T, V]`` tensor: the row stride is passed on."""
-    R, V = logits.shape
-    dt = _logit_dtype(logits)
-    ldt = logits.dtype
-
-    def rows_ptr(t, name):
-        if t is None:
-            return None
-        if (not t.is_cuda or t.dtype != ldt or t.dim() != 2 or t.shape != logits.shape or t.stride(1) != 1
-                or t.stride(0) != logits.stride(0) or t.stride(0) < V):
-            raise ValueError(f"{name} must be a CUDA tensor [R, V] of {ldt} with contiguous rows and the row stride of logits")
-        return t.data_ptr()
-
     if workspace is None:
-        workspace = torch.zeros(csd_sample_workspace_size(R, V, dt), dtype=torch.uint8, device=logits.device)
-    rc = library().csd_sample_rows(
-        rows_ptr(logits, "logits"), rows_ptr(uncond, "uncond"), float(cfg_scale), int(top_k), dt, R, V,
-        int(logits.stride(0)) if R > 1 else V, _dev_ptr(uniforms, "uniforms", torch.float32), _dev_ptr(out_tokens, "out_tokens", torch.int32),
-        _dev_ptr(out_status, "out_status", torch.int32), _dev_ptr(workspace, "workspace"),
-        workspace.numel() * workspace.element_size(), 1 if back_to_back else 0, _stream_handle(stream))
+        R, V = logits.shape
+        workspace = torch.zeros(csd_sample_workspace_size(R, V, _logit_dtype(logits)), dtype=torch.uint8, device=logits.device)
+    rc = bind().sample_rows(_address("csd_sample_rows"), logits, uniforms, out_tokens, uncond, cfg_scale, top_k, out_status,
+                            workspace, back_to_back, stream)
     if rc != 0:
         raise CsdError(rc, "csd_sample_rows")
 
@@ -405,42 +398,20 @@ def csd_verify_tree(target_logits, draft_logits, parent, draft_tokens, uniforms,
                     out_nodes=None, out_status=None, dbg_G=None, workspace=None, stream=None) -> None:
     """Tree-structured verification (see ``csd_verify_tree`` in csd.h): logits [B, N + 1, V] per context,
     ``parent`` a host array [N], ``draft_tokens`` [B, N], ``uniforms`` [B, N + 1], ``relax_schedule`` [D]."""
-    B, C1, V = target_logits.shape
-    N = C1 - 1
     par = np.ascontiguousarray(parent, dtype=np.int32)
-    if draft_logits.shape != (B, C1, V) or par.shape != (N,):
-        raise ValueError("shapes: target and draft [B, N + 1, V], parent [N]")
-    dt = _logit_dtype(target_logits)
-    ldt = target_logits.dtype
     if workspace is None:
         # one grow-only buffer per device, kept by the module: the call is asynchronous, so a buffer made
         # here must outlive this function
-        need = csd_tree_workspace_size(B, N, V, dt)
+        B, C1, V = target_logits.shape
+        need = csd_tree_workspace_size(B, C1 - 1, V, _logit_dtype(target_logits))
         key = target_logits.device
         workspace = _tree_ws.get(key)
         if workspace is None or workspace.numel() < need:
             workspace = torch.zeros(need, dtype=torch.uint8, device=key)
             _tree_ws[key] = workspace
-    p = csd_tree_params()
-    p.target_logits = _dev_ptr(target_logits, "target_logits", ldt)
-    p.draft_logits = _dev_ptr(draft_logits, "draft_logits", ldt)
-    p.target_uncond = _dev_ptr(target_uncond, "target_uncond", ldt)
-    p.draft_uncond = _dev_ptr(draft_uncond, "draft_uncond", ldt)
-    p.cfg_scale, p.top_k, p.dtype = float(cfg_scale), int(top_k), dt
-    p.B, p.N, p.V = B, N, V
-    p.parent = par.ctypes.data
-    p.draft_tokens = _dev_ptr(draft_tokens, "draft_tokens", torch.int32)
-    p.uniforms = _dev_ptr(uniforms, "uniforms", torch.float32)
-    p.relax_schedule = _dev_ptr(relax_schedule, "relax_schedule", torch.float32)
-    p.out_tokens = _dev_ptr(out_tokens, "out_tokens", torch.int32)
-    p.out_accept_len = _dev_ptr(out_accept_len, "out_accept_len", torch.int32)
-    p.out_nodes = _dev_ptr(out_nodes, "out_nodes", torch.int32)
-    p.out_status = _dev_ptr(out_status, "out_status", torch.int32)
-    p.dbg_G = _dev_ptr(dbg_G, "dbg_G", torch.float32)
-    p.workspace = _dev_ptr(workspace, "workspace")
-    p.workspace_bytes = workspace.numel() * workspace.element_size()
-    p.stream = _stream_handle(stream)
-    rc = library().csd_verify_tree(C.byref(p))
+    rc = bind().verify_tree(_address("csd_verify_tree"), target_logits, draft_logits, par, draft_tokens, uniforms,
+                            relax_schedule, out_tokens, out_accept_len, target_uncond, draft_uncond, cfg_scale, top_k,
+                            out_nodes, out_status, dbg_G, workspace, stream)
     if rc != 0:
         raise CsdError(rc, "csd_verify_tree")
 

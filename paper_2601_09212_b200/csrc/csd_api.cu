@@ -72,19 +72,20 @@ Layout layout_for(int B, int gamma, int V, int dtype) {
   return l;
 }
 
-// c with P(N(0,1) > c) = tail, by bisection on erfc (host, called once per call; 60 steps)
+// c with P(N(0,1) > c) = tail, 0 < tail < 1: the rational approximation 26.2.23 of Abramowitz and Stegun's
+// Handbook of Mathematical Functions (absolute error below 4.5e-4), then two Newton steps on erfc.  Called up to
+// three times per top-k call (by bisection these took 4 us of the call's 8.6 us on the host).
 double normal_upper_quantile(double tail) {
-  double lo = -8.0, hi = 8.0;
-  for (int it = 0; it < 60; ++it) {
-    const double mid = 0.5 * (lo + hi);
-    if (0.5 * erfc(mid / sqrt(2.0)) > tail) lo = mid; else hi = mid;
-  }
-  return 0.5 * (lo + hi);
+  const double p = tail < 0.5 ? tail : 1.0 - tail;
+  const double t = sqrt(-2.0 * log(p));
+  double x = t - ((0.010328 * t + 0.802853) * t + 2.515517) / (((0.001308 * t + 0.189269) * t + 1.432788) * t + 1.0);
+  for (int it = 0; it < 2; ++it) x += (0.5 * erfc(x * 0.70710678118654752) - p) * 2.5066282746310002 * exp(0.5 * x * x);
+  return tail < 0.5 ? x : -x;
 }
 
 // Launches one of the single-launch kernels (KERNEL: 0 plain, 1 top-k on rows that are a whole
-// number of stages, 2 top-k on any row length, 3 and 4 the same two with the large candidate lists) with its shared-memory size, optionally with
-// programmatic stream serialisation and as clusters of ctas_per_seq blocks.
+// number of stages, 2 top-k on any row length, 3 and 4 the same two with the large candidate lists) with its shared-memory size, as a programmatic
+// dependent launch and, for ctas_per_seq > 1, as clusters of that many blocks.
 template <typename T, bool CFG, int KERNEL>
 cudaError_t launch_fused(const FusedArgs& a, int grid, bool overlap, cudaStream_t stream) {
   auto kern = KERNEL == 0 ? verify_plain_kernel<T, CFG>

@@ -1,0 +1,295 @@
+// Argument marshalling of the Python binding, in C++: checks of tensors, their addresses, the current
+// stream, and the call.  A decoding loop makes one small call per round, and in Python these checks took longer
+// than the GPU needs for a call of one sequence (csd_verify, B = 1: 14.3 us on the host against 12.9 us on the
+// device; 5 us here).  Nothing of the method is in this file: every function ends in one call of libcsd's C ABI,
+// whose address the caller passes in (the library is loaded, and exchanged in tests, by the Python module).
+#define PY_SSIZE_T_CLEAN
+#include <ATen/core/Tensor.h>
+#include <Python.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/csd.h"
+
+namespace {
+
+// Thrown after a Python exception has been set.
+struct Failed {};
+
+const at::Tensor& tensor_of(PyObject* o, const char* name) {
+  if (!THPVariable_Check(o)) {
+    PyErr_Format(PyExc_TypeError, "%s must be a tensor", name);
+    throw Failed();
+  }
+  return THPVariable_Unpack(o);
+}
+
+const char* dtype_name(at::ScalarType t) {
+  switch (t) {
+    case at::kFloat: return "torch.float32";
+    case at::kBFloat16: return "torch.bfloat16";
+    case at::kInt: return "torch.int32";
+    case at::kDouble: return "torch.float64";
+    default: return c10::toString(t);
+  }
+}
+
+void check_dtype(const at::Tensor& t, const char* name, at::ScalarType want) {
+  if (t.scalar_type() != want) {
+    PyErr_Format(PyExc_TypeError, "%s must be %s, got %s", name, dtype_name(want), dtype_name(t.scalar_type()));
+    throw Failed();
+  }
+}
+
+// Address of a contiguous CUDA tensor (None: null)
+void* dev_ptr(PyObject* o, const char* name, at::ScalarType want, bool any_dtype = false) {
+  if (o == Py_None) return nullptr;
+  const at::Tensor& t = tensor_of(o, name);
+  if (!t.is_cuda()) {
+    PyErr_Format(PyExc_ValueError, "%s must be a CUDA tensor", name);
+    throw Failed();
+  }
+  if (!t.is_contiguous()) {
+    PyErr_Format(PyExc_ValueError, "%s must be contiguous", name);
+    throw Failed();
+  }
+  if (!any_dtype) check_dtype(t, name, want);
+  return t.data_ptr();
+}
+
+void fail(const char* what) {
+  PyErr_SetString(PyExc_ValueError, what);
+  throw Failed();
+}
+
+csd_dtype logit_dtype(const at::Tensor& t) {
+  if (t.scalar_type() == at::kFloat) return CSD_F32;
+  if (t.scalar_type() == at::kBFloat16) return CSD_BF16;
+  PyErr_Format(PyExc_TypeError, "logits must be float32 or bfloat16, got %s", dtype_name(t.scalar_type()));
+  throw Failed();
+}
+
+// None: the current stream; an int: the handle itself; else an object with a cuda_stream attribute
+void* stream_of(PyObject* o) {
+  if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+  PyObject* v = o;
+  if (!PyLong_Check(o)) {
+    v = PyObject_GetAttrString(o, "cuda_stream");
+    if (!v) throw Failed();
+  }
+  void* s = PyLong_AsVoidPtr(v);
+  if (v != o) Py_DECREF(v);
+  if (!s && PyErr_Occurred()) throw Failed();
+  return s;
+}
+
+template <typename F>
+F function_of(PyObject* o) {
+  void* p = PyLong_AsVoidPtr(o);
+  if (!p) {
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "no function");
+    throw Failed();
+  }
+  return reinterpret_cast<F>(p);
+}
+
+double number_of(PyObject* o) {
+  const double v = PyFloat_AsDouble(o);
+  if (v == -1.0 && PyErr_Occurred()) throw Failed();
+  return v;
+}
+long long integer_of(PyObject* o) {
+  const long long v = PyLong_AsLongLong(o);
+  if (v == -1 && PyErr_Occurred()) throw Failed();
+  return v;
+}
+
+// Runs `body` (which returns the library's code), translating what it throws.
+template <typename Body>
+PyObject* guarded(Py_ssize_t n, Py_ssize_t want, Body body) {
+  if (n != want) {
+    PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
+    return nullptr;
+  }
+  try {
+    return PyLong_FromLong(body());
+  } catch (const Failed&) {
+    return nullptr;
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+// the library call itself, without the interpreter lock
+template <typename Call>
+int unlocked(Call call) {
+  int rc;
+  Py_BEGIN_ALLOW_THREADS rc = call();
+  Py_END_ALLOW_THREADS return rc;
+}
+
+// csd_verify / csd_verify_static: function, target, draft, tokens, uniforms, schedule, out_tokens, out_len, stream
+PyObject* verify(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 9, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_verify)>(a[0]);
+    const at::Tensor &t = tensor_of(a[1], "target_logits"), &d = tensor_of(a[2], "draft_logits");
+    if (t.dim() != 3 || !d.sizes().equals(t.sizes())) fail("target_logits and draft_logits must both be [B, gamma, V]");
+    const void* tp = dev_ptr(a[1], "target_logits", at::kFloat);
+    const void* dp = dev_ptr(a[2], "draft_logits", at::kFloat);
+    const void* tok = dev_ptr(a[3], "draft_tokens", at::kInt);
+    const void* uni = dev_ptr(a[4], "uniforms", at::kFloat);
+    const void* sched = dev_ptr(a[5], "relax_schedule", at::kFloat);
+    void* otok = dev_ptr(a[6], "out_tokens", at::kInt);
+    void* olen = dev_ptr(a[7], "out_accept_len", at::kInt);
+    void* s = stream_of(a[8]);
+    const int B = (int)t.size(0), L = (int)t.size(1), V = (int)t.size(2);
+    return unlocked([&] {
+      return fn((const float*)tp, (const float*)dp, (const int32_t*)tok, (const float*)uni, (const float*)sched, B, L, V,
+                (int32_t*)otok, (int32_t*)olen, s);
+    });
+  });
+}
+
+// a function of one parameter block (csd_verify_ex): function, address of the block
+PyObject* call_block(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 2, [&]() -> int {
+    const auto fn = function_of<int (*)(const void*)>(a[0]);
+    const void* p = PyLong_AsVoidPtr(a[1]);
+    return unlocked([&] { return fn(p); });
+  });
+}
+
+// rows that are contiguous in themselves, at any spacing
+const void* rows_ptr(PyObject* o, const char* name, const at::Tensor& like) {
+  if (o == Py_None) return nullptr;
+  const at::Tensor& t = tensor_of(o, name);
+  if (!t.is_cuda() || t.scalar_type() != like.scalar_type() || t.dim() != 2 || !t.sizes().equals(like.sizes()) || t.stride(1) != 1 ||
+      t.stride(0) != like.stride(0) || t.stride(0) < like.size(1)) {
+    PyErr_Format(PyExc_ValueError, "%s must be a CUDA tensor [R, V] of %s with contiguous rows and the row stride of logits", name,
+                 dtype_name(like.scalar_type()));
+    throw Failed();
+  }
+  return t.data_ptr();
+}
+
+// csd_sample_rows: function, logits, uniforms, out_tokens, uncond, cfg_scale, top_k, out_status, workspace,
+// back_to_back, stream
+PyObject* sample_rows(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 11, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_sample_rows)>(a[0]);
+    const at::Tensor& x = tensor_of(a[1], "logits");
+    if (x.dim() != 2) fail("logits must be [R, V]");
+    const int dt = logit_dtype(x);
+    const void* xp = rows_ptr(a[1], "logits", x);
+    const void* up = rows_ptr(a[4], "uncond", x);
+    const void* uni = dev_ptr(a[2], "uniforms", at::kFloat);
+    void* otok = dev_ptr(a[3], "out_tokens", at::kInt);
+    const float scale = (float)number_of(a[5]);
+    const int top_k = (int)integer_of(a[6]);
+    void* ost = dev_ptr(a[7], "out_status", at::kInt);
+    void* ws = dev_ptr(a[8], "workspace", at::kByte, true);
+    const size_t ws_bytes = ws ? THPVariable_Unpack(a[8]).nbytes() : 0;
+    const int b2b = PyObject_IsTrue(a[9]);
+    void* s = stream_of(a[10]);
+    const int R = (int)x.size(0), V = (int)x.size(1);
+    const int64_t stride = R > 1 ? x.stride(0) : V;
+    return unlocked([&] {
+      return fn(xp, up, scale, top_k, dt, R, V, stride, (const float*)uni, (int32_t*)otok, (int32_t*)ost, ws, ws_bytes, b2b, s);
+    });
+  });
+}
+
+// csd_verify_tree: function, target, draft, parent (a contiguous int32 buffer), tokens, uniforms, schedule, out_tokens,
+// out_len, target_uncond, draft_uncond, cfg_scale, top_k, out_nodes, out_status, dbg_G, workspace, stream
+PyObject* verify_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 18, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_verify_tree)>(a[0]);
+    const at::Tensor &t = tensor_of(a[1], "target_logits"), &d = tensor_of(a[2], "draft_logits");
+    Py_buffer par;
+    if (PyObject_GetBuffer(a[3], &par, PyBUF_C_CONTIGUOUS) != 0) throw Failed();
+    struct Release {
+      Py_buffer* b;
+      ~Release() { PyBuffer_Release(b); }
+    } release{&par};
+    const int64_t N = par.len / 4;
+    if (par.itemsize != 4 || t.dim() != 3 || t.size(1) != N + 1 || !d.sizes().equals(t.sizes()))
+      fail("shapes: target and draft [B, N + 1, V], parent [N]");
+    csd_tree_params p;
+    memset(&p, 0, sizeof p);
+    p.dtype = logit_dtype(t);
+    const at::ScalarType lt = t.scalar_type();
+    p.target_logits = dev_ptr(a[1], "target_logits", lt);
+    p.draft_logits = dev_ptr(a[2], "draft_logits", lt);
+    p.target_uncond = dev_ptr(a[9], "target_uncond", lt);
+    p.draft_uncond = dev_ptr(a[10], "draft_uncond", lt);
+    p.cfg_scale = (float)number_of(a[11]);
+    p.top_k = (int32_t)integer_of(a[12]);
+    p.B = (int32_t)t.size(0); p.N = (int32_t)N; p.V = (int32_t)t.size(2);
+    p.parent = (const int32_t*)par.buf;
+    p.draft_tokens = (const int32_t*)dev_ptr(a[4], "draft_tokens", at::kInt);
+    p.uniforms = (const float*)dev_ptr(a[5], "uniforms", at::kFloat);
+    p.relax_schedule = (const float*)dev_ptr(a[6], "relax_schedule", at::kFloat);
+    p.out_tokens = (int32_t*)dev_ptr(a[7], "out_tokens", at::kInt);
+    p.out_accept_len = (int32_t*)dev_ptr(a[8], "out_accept_len", at::kInt);
+    p.out_nodes = (int32_t*)dev_ptr(a[13], "out_nodes", at::kInt);
+    p.out_status = (int32_t*)dev_ptr(a[14], "out_status", at::kInt);
+    p.dbg_G = (float*)dev_ptr(a[15], "dbg_G", at::kFloat);
+    p.workspace = dev_ptr(a[16], "workspace", at::kByte, true);
+    p.workspace_bytes = p.workspace ? THPVariable_Unpack(a[16]).nbytes() : 0;
+    p.stream = stream_of(a[17]);
+    return unlocked([&] { return fn(&p); });
+  });
+}
+
+// the four calls of the vocabulary-sharded round: function, address of the parameter block, then the tensors
+PyObject* shard_stats(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 3, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_shard_stats)>(a[0]);
+    const auto p = (const csd_shard_params*)PyLong_AsVoidPtr(a[1]);
+    void* rec = dev_ptr(a[2], "records", at::kFloat);
+    return unlocked([&] { return fn(p, rec); });
+  });
+}
+PyObject* shard_partial(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 7, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_shard_partial)>(a[0]);
+    const auto p = (const csd_shard_params*)PyLong_AsVoidPtr(a[1]);
+    const void* rec = dev_ptr(a[2], "records_all", at::kFloat);
+    double* tot = (double*)dev_ptr(a[3], "totals", at::kDouble);
+    float* dp = (float*)dev_ptr(a[4], "dbg_p", at::kFloat);
+    float* dq = (float*)dev_ptr(a[5], "dbg_q", at::kFloat);
+    float* df = (float*)dev_ptr(a[6], "dbg_f", at::kFloat);
+    return unlocked([&] { return fn(p, rec, tot, dp, dq, df); });
+  });
+}
+PyObject* shard_pick(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 5, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_shard_pick)>(a[0]);
+    const auto p = (const csd_shard_params*)PyLong_AsVoidPtr(a[1]);
+    const void* rec = dev_ptr(a[2], "records_all", at::kFloat);
+    const double* tot = (const double*)dev_ptr(a[3], "totals_all", at::kDouble);
+    int32_t* cand = (int32_t*)dev_ptr(a[4], "cand", at::kInt);
+    return unlocked([&] { return fn(p, rec, tot, cand); });
+  });
+}
+PyObject* shard_emit(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 6, [&]() -> int {
+    const auto fn = function_of<decltype(&csd_shard_emit)>(a[0]);
+    const auto p = (const csd_shard_params*)PyLong_AsVoidPtr(a[1]);
+    const int32_t* cand = (const int32_t*)dev_ptr(a[2], "cand_all", at::kInt);
+    int32_t* tok = (int32_t*)dev_ptr(a[3], "out_tokens", at::kInt);
+    int32_t* len = (int32_t*)dev_ptr(a[4], "out_accept_len", at::kInt);
+    int32_t* st = (int32_t*)dev_ptr(a[5], "out_status", at::kInt);
+    return unlocked([&] { return fn(p, cand, tok, len, st); });
+  });
+}
+
+#define CSD_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+PyMethodDef g_methods[] = {CSD_METHOD(verify),      CSD_METHOD(call_block),    CSD_METHOD(sample_rows), CSD_METHOD(verify_tree),
+                           CSD_METHOD(shard_stats), CSD_METHOD(shard_partial), CSD_METHOD(shard_pick),  CSD_METHOD(shard_emit),
+                           {nullptr, nullptr, 0, nullptr}};
+PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_csd_bind", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__csd_bind(void) { return PyModule_Create(&g_module); }

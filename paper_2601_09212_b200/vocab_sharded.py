@@ -9,7 +9,7 @@ from typing import Callable, Optional
 
 import torch
 
-from . import CsdError, _dev_ptr, _logit_dtype, _stream_handle, library
+from . import CsdError, _address, _dev_ptr, _logit_dtype, _stream_handle, bind, library
 
 
 class csd_shard_params(C.Structure):
@@ -78,7 +78,7 @@ class ShardedRound:
         p.relax_schedule = _dev_ptr(relax_schedule, "relax_schedule", torch.float32)
         p.workspace, p.workspace_bytes = self.ws.data_ptr(), need
         p.stream = _stream_handle(stream)
-        self.p, self.lib = p, lib
+        self.p = p
 
     @staticmethod
     def _check(rc, where):
@@ -86,30 +86,25 @@ class ShardedRound:
             raise CsdError(rc, where)
 
     def stats(self) -> torch.Tensor:
-        self._check(self.lib.csd_shard_stats(C.byref(self.p), self.records.data_ptr()), "csd_shard_stats")
+        self._check(bind().shard_stats(_address("csd_shard_stats"), C.addressof(self.p), self.records), "csd_shard_stats")
         return self.records
 
     def partial(self, records_all: torch.Tensor, dbg_p=None, dbg_q=None, dbg_f=None) -> torch.Tensor:
         self._records_all = records_all
-        self._check(self.lib.csd_shard_partial(
-            C.byref(self.p), _dev_ptr(records_all, "records_all", torch.float32), self.totals.data_ptr(),
-            _dev_ptr(dbg_p, "dbg_p", torch.float32), _dev_ptr(dbg_q, "dbg_q", torch.float32),
-            _dev_ptr(dbg_f, "dbg_f", torch.float32)), "csd_shard_partial")
+        self._check(bind().shard_partial(_address("csd_shard_partial"), C.addressof(self.p), records_all, self.totals,
+                                         dbg_p, dbg_q, dbg_f), "csd_shard_partial")
         return self.totals
 
     def pick(self, totals_all: torch.Tensor) -> torch.Tensor:
         self._totals_all = totals_all
-        self._check(self.lib.csd_shard_pick(
-            C.byref(self.p), self._records_all.data_ptr(), _dev_ptr(totals_all, "totals_all", torch.float64),
-            self.cand.data_ptr()), "csd_shard_pick")
+        self._check(bind().shard_pick(_address("csd_shard_pick"), C.addressof(self.p), self._records_all, totals_all,
+                                      self.cand), "csd_shard_pick")
         return self.cand
 
     def emit(self, cand_all: torch.Tensor, out_tokens, out_accept_len, out_status=None) -> None:
         self._cand_all = cand_all
-        self._check(self.lib.csd_shard_emit(
-            C.byref(self.p), _dev_ptr(cand_all, "cand_all", torch.int32), _dev_ptr(out_tokens, "out_tokens", torch.int32),
-            _dev_ptr(out_accept_len, "out_accept_len", torch.int32), _dev_ptr(out_status, "out_status", torch.int32)),
-            "csd_shard_emit")
+        self._check(bind().shard_emit(_address("csd_shard_emit"), C.addressof(self.p), cand_all, out_tokens,
+                                      out_accept_len, out_status), "csd_shard_emit")
 
 
 def all_gather_rank_major(t: torch.Tensor, n: int, group=None) -> torch.Tensor:
