@@ -87,7 +87,7 @@ double normal_upper_quantile(double tail) {
 // number of stages, 2 top-k on any row length, 3 and 4 the same two with the large candidate lists) with its shared-memory size, as a programmatic
 // dependent launch and, for ctas_per_seq > 1, as clusters of that many blocks.
 template <typename T, bool CFG, int KERNEL>
-cudaError_t launch_fused(const FusedArgs& a, int grid, bool overlap, cudaStream_t stream) {
+cudaError_t launch_fused(const FusedArgs& a, int grid, cudaStream_t stream) {
   auto kern = KERNEL == 0 ? verify_plain_kernel<T, CFG>
               : KERNEL == 1 ? verify_topk_kernel<T, CFG, false, kWarpList>
               : KERNEL == 2 ? verify_topk_kernel<T, CFG, true, kWarpList>
@@ -112,11 +112,10 @@ cudaError_t launch_fused(const FusedArgs& a, int grid, bool overlap, cudaStream_
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
-  if (overlap) {   // the call may start while the operation before it on the stream is still running
-    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
-    ++n_attr;
-  }
+  // the blocks may become resident while the operation before this one on the stream is still running
+  attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+  ++n_attr;
   if (a.ctas_per_seq > 1) {   // the blocks of a sequence are one cluster
     attr[n_attr].id = cudaLaunchAttributeClusterDimension;
     attr[n_attr].val.clusterDim.x = (unsigned)a.ctas_per_seq;
@@ -130,12 +129,30 @@ cudaError_t launch_fused(const FusedArgs& a, int grid, bool overlap, cudaStream_
 }
 
 template <typename T, bool CFG>
-cudaError_t launch_fused_t(const FusedArgs& a, bool topk, int grid, bool overlap, cudaStream_t stream) {
-  if (!topk) return launch_fused<T, CFG, 0>(a, grid, overlap, stream);
+cudaError_t launch_fused_t(const FusedArgs& a, bool topk, int grid, cudaStream_t stream) {
+  if (!topk) return launch_fused<T, CFG, 0>(a, grid, stream);
   constexpr int kStageElems = kTkStageBytes / ((int)sizeof(T) * (CFG ? 2 : 1));
   const bool whole = a.fin.V % kStageElems == 0;
-  if (a.large_lists) return whole ? launch_fused<T, CFG, 3>(a, grid, overlap, stream) : launch_fused<T, CFG, 4>(a, grid, overlap, stream);
-  return whole ? launch_fused<T, CFG, 1>(a, grid, overlap, stream) : launch_fused<T, CFG, 2>(a, grid, overlap, stream);
+  if (a.large_lists) return whole ? launch_fused<T, CFG, 3>(a, grid, stream) : launch_fused<T, CFG, 4>(a, grid, stream);
+  return whole ? launch_fused<T, CFG, 1>(a, grid, stream) : launch_fused<T, CFG, 2>(a, grid, stream);
+}
+
+// A kernel that begins with griddepcontrol.wait, as a programmatic dependent launch: its blocks are resident
+// and set up when the operation before it completes.
+template <typename K, typename A>
+cudaError_t launch_after(K kern, const A& a, unsigned grid, unsigned block, size_t smem, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
 template <typename T, bool CFG, int U, bool TOPK>
@@ -151,8 +168,7 @@ cudaError_t launch_stats(const StatsArgs& a, int sms, cudaStream_t stream) {
   }
   long long grid = (long long)sms * per_sm;
   if (grid > a.n_items) grid = a.n_items;
-  kern<<<(unsigned)grid, kStatsThreads, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_after(kern, a, (unsigned)grid, kStatsThreads, 0, stream);
 }
 
 template <typename T, bool CFG>
@@ -173,8 +189,7 @@ cudaError_t launch_select(const SelectArgs& a, int sms, cudaStream_t stream) {
   const long long rows = (long long)a.B * (a.T + a.gamma);
   long long grid = 2LL * sms;
   if (grid > rows) grid = rows;
-  topk_threshold_kernel<T, CFG><<<(unsigned)grid, kSelectThreads, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_after(topk_threshold_kernel<T, CFG>, a, (unsigned)grid, kSelectThreads, 0, stream);
 }
 
 template <typename T, bool CFG>
@@ -194,18 +209,7 @@ cudaError_t launch_finish(const FinishArgs& a_in, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3((unsigned)a.B);
-  cfg.blockDim = dim3(kFinishThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return launch_after(kern, a, (unsigned)a.B, kFinishThreads, smem, stream);
 }
 
 // Test aids (csd_test_hooks): process-wide, read at every launch of the single-launch path.
@@ -328,13 +332,18 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     ua.ctas_per_seq = (int)c;
     ua.seqs_per_cta = (int)spc;
     cudaError_t fe;
-    const bool overlap = in.back_to_back != 0;
+    ua.ordered = in.back_to_back ? 0 : 1;
+    // In stream order the next call's blocks may come in early where this grid has at most one block per SM:
+    // with more, they would fill the SMs that happen to have room and end up unevenly spread (256 sequences of 16
+    // positions, 256 blocks: 67.6 us a call without the early signal, 85.8 with it).  A stats-only call is
+    // followed by its finishing kernel, whose large blocks would only sit on SMs this kernel needs.
+    ua.signal = (in.stats_out == nullptr && (in.back_to_back || grid <= sms)) ? 1 : 0;
     if (in.dtype == CSD_F32)
-      fe = cfg ? launch_fused_t<float, true>(ua, topk, (int)grid, overlap, stream)
-               : launch_fused_t<float, false>(ua, topk, (int)grid, overlap, stream);
+      fe = cfg ? launch_fused_t<float, true>(ua, topk, (int)grid, stream)
+               : launch_fused_t<float, false>(ua, topk, (int)grid, stream);
     else
-      fe = cfg ? launch_fused_t<__nv_bfloat16, true>(ua, topk, (int)grid, overlap, stream)
-               : launch_fused_t<__nv_bfloat16, false>(ua, topk, (int)grid, overlap, stream);
+      fe = cfg ? launch_fused_t<__nv_bfloat16, true>(ua, topk, (int)grid, stream)
+               : launch_fused_t<__nv_bfloat16, false>(ua, topk, (int)grid, stream);
     return fe;
   }
 }
@@ -615,18 +624,7 @@ cudaError_t launch_tree_finish(const TreeArgs& a_in, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3((unsigned)a.fin.B);
-  cfg.blockDim = dim3(kFinishThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  return launch_after(kern, a, (unsigned)a.fin.B, kFinishThreads, smem, stream);
 }
 
 // Depth of the tree (the root's children are level 1), or a negative csd_error for a malformed one:
@@ -848,21 +846,6 @@ void shard_args(const csd_shard_params& p, int sms, ShardArgs& sa, StatsArgs& st
   st.partials = reinterpret_cast<float2*>(ws + lay.partials_off);
   st.thresholds = nullptr;
 }
-
-template <typename K>
-cudaError_t launch_after(K kern, const ShardArgs& a, unsigned grid, unsigned block, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
-}
 }  // namespace
 extern "C" {
 
@@ -890,14 +873,14 @@ int csd_shard_stats(const csd_shard_params* pp, void* out_records) {
   if (p.dtype == CSD_F32) {
     e = cfg ? launch_stats_u<float, true>(st, U, false, sms, stream) : launch_stats_u<float, false>(st, U, false, sms, stream);
     if (e == cudaSuccess)
-      e = cfg ? launch_after(shard_merge_kernel<float, true>, sa, grid, 256, stream)
-              : launch_after(shard_merge_kernel<float, false>, sa, grid, 256, stream);
+      e = cfg ? launch_after(shard_merge_kernel<float, true>, sa, grid, 256, 0, stream)
+              : launch_after(shard_merge_kernel<float, false>, sa, grid, 256, 0, stream);
   } else {
     e = cfg ? launch_stats_u<__nv_bfloat16, true>(st, U, false, sms, stream)
             : launch_stats_u<__nv_bfloat16, false>(st, U, false, sms, stream);
     if (e == cudaSuccess)
-      e = cfg ? launch_after(shard_merge_kernel<__nv_bfloat16, true>, sa, grid, 256, stream)
-              : launch_after(shard_merge_kernel<__nv_bfloat16, false>, sa, grid, 256, stream);
+      e = cfg ? launch_after(shard_merge_kernel<__nv_bfloat16, true>, sa, grid, 256, 0, stream)
+              : launch_after(shard_merge_kernel<__nv_bfloat16, false>, sa, grid, 256, 0, stream);
   }
   return e == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
 }
@@ -915,14 +898,14 @@ int csd_shard_partial(const csd_shard_params* pp, const void* records_all, doubl
   sa.fin.dbg_p = dbg_p; sa.fin.dbg_q = dbg_q; sa.fin.dbg_f = dbg_f;
   const bool cfg = p.target_uncond != nullptr;
   cudaStream_t stream = (cudaStream_t)p.stream;
-  if (p.dtype == CSD_F32) {
-    if (cfg) shard_partial_kernel<float, true><<<p.B, kFinishThreads, 0, stream>>>(sa);
-    else shard_partial_kernel<float, false><<<p.B, kFinishThreads, 0, stream>>>(sa);
-  } else {
-    if (cfg) shard_partial_kernel<__nv_bfloat16, true><<<p.B, kFinishThreads, 0, stream>>>(sa);
-    else shard_partial_kernel<__nv_bfloat16, false><<<p.B, kFinishThreads, 0, stream>>>(sa);
-  }
-  return cudaGetLastError() == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+  cudaError_t e;
+  if (p.dtype == CSD_F32)
+    e = cfg ? launch_after(shard_partial_kernel<float, true>, sa, p.B, kFinishThreads, 0, stream)
+            : launch_after(shard_partial_kernel<float, false>, sa, p.B, kFinishThreads, 0, stream);
+  else
+    e = cfg ? launch_after(shard_partial_kernel<__nv_bfloat16, true>, sa, p.B, kFinishThreads, 0, stream)
+            : launch_after(shard_partial_kernel<__nv_bfloat16, false>, sa, p.B, kFinishThreads, 0, stream);
+  return e == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
 }
 
 int csd_shard_pick(const csd_shard_params* pp, const void* records_all, const double* totals_all, int32_t* out_candidates) {
@@ -937,14 +920,14 @@ int csd_shard_pick(const csd_shard_params* pp, const void* records_all, const do
   sa.cand_local = out_candidates;
   const bool cfg = p.target_uncond != nullptr;
   cudaStream_t stream = (cudaStream_t)p.stream;
-  if (p.dtype == CSD_F32) {
-    if (cfg) shard_pick_kernel<float, true><<<p.B, kFinishThreads, 0, stream>>>(sa);
-    else shard_pick_kernel<float, false><<<p.B, kFinishThreads, 0, stream>>>(sa);
-  } else {
-    if (cfg) shard_pick_kernel<__nv_bfloat16, true><<<p.B, kFinishThreads, 0, stream>>>(sa);
-    else shard_pick_kernel<__nv_bfloat16, false><<<p.B, kFinishThreads, 0, stream>>>(sa);
-  }
-  return cudaGetLastError() == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+  cudaError_t e;
+  if (p.dtype == CSD_F32)
+    e = cfg ? launch_after(shard_pick_kernel<float, true>, sa, p.B, kFinishThreads, 0, stream)
+            : launch_after(shard_pick_kernel<float, false>, sa, p.B, kFinishThreads, 0, stream);
+  else
+    e = cfg ? launch_after(shard_pick_kernel<__nv_bfloat16, true>, sa, p.B, kFinishThreads, 0, stream)
+            : launch_after(shard_pick_kernel<__nv_bfloat16, false>, sa, p.B, kFinishThreads, 0, stream);
+  return e == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
 }
 
 int csd_shard_emit(const csd_shard_params* pp, const int32_t* candidates_all, int32_t* out_tokens, int32_t* out_accept_len,
@@ -957,8 +940,7 @@ int csd_shard_emit(const csd_shard_params* pp, const int32_t* candidates_all, in
   shard_args(p, device_sms(nullptr), sa, st);
   sa.cand_all = candidates_all;
   sa.fin.out_tokens = out_tokens; sa.fin.out_accept_len = out_accept_len; sa.fin.out_status = out_status;
-  shard_emit_kernel<<<p.B, 64, 0, (cudaStream_t)p.stream>>>(sa);
-  return cudaGetLastError() == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+  return launch_after(shard_emit_kernel, sa, p.B, 64, 0, (cudaStream_t)p.stream) == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
 }
 
 // ---- allocation-free form -------------------------------------------------------------

@@ -116,19 +116,21 @@ __device__ __forceinline__ bool checked_ok(int idx, int width, int n, int site) 
 #endif
 
 // ---- element access -----------------------------------------------------------
+// Global loads go past the L1 (ld.global.cg): a kernel that became resident while the operation before it was
+// still running must not meet a line that L1 held from then, and no path reads a logit often enough to gain.
 template <typename T> struct Elem;
 template <> struct Elem<float> {
   static constexpr int kVec = 4;
   __device__ static __forceinline__ void load_vec(const float* p, float (&out)[4]) {
-    float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    float4 v = __ldcg(reinterpret_cast<const float4*>(p));
     out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
   }
-  __device__ static __forceinline__ float load_one(const float* p) { return __ldg(p); }
+  __device__ static __forceinline__ float load_one(const float* p) { return __ldcg(p); }
 };
 template <> struct Elem<__nv_bfloat16> {
   static constexpr int kVec = 8;
   __device__ static __forceinline__ void load_vec(const __nv_bfloat16* p, float (&out)[8]) {
-    uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+    uint4 v = __ldcg(reinterpret_cast<const uint4*>(p));
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -137,7 +139,7 @@ template <> struct Elem<__nv_bfloat16> {
     }
   }
   __device__ static __forceinline__ float load_one(const __nv_bfloat16* p) {
-    return __uint_as_float(((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p))) << 16);
+    return __uint_as_float(((uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(p))) << 16);
   }
 };
 
@@ -258,6 +260,7 @@ __global__ void __launch_bounds__(kStatsThreads) row_stats_kernel(const StatsArg
   constexpr int VEC = Elem<T>::kVec;
   __shared__ float sh_m[2][kStatsThreads / 32];
   __shared__ float sh_s[2][kStatsThreads / 32];
+  pdl_wait();               // the logits, and with top-k the thresholds, are complete
   pdl_launch_dependents();  // the finishing kernel may become resident as soon as blocks retire
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -411,6 +414,7 @@ __global__ void __launch_bounds__(kSelectThreads) topk_threshold_kernel(const Se
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rows_per_seq = a.T + a.gamma;
   const int n_rows = a.B * rows_per_seq;
+  pdl_wait();
   for (int row_id = blockIdx.x; row_id < n_rows; row_id += gridDim.x) {
     const int b = row_id / rows_per_seq;
     const int r = row_id - b * rows_per_seq;
@@ -741,9 +745,9 @@ __device__ void finish_sequence(const FinishArgs& a, const int b, const int tid,
       sm.valid[0][i] = t_ok; sm.valid[1][i] = d_ok;
       int flag = 0;
       if (i < L) {
-        const int tok = a.tokens[(int64_t)b * L + i];
+        const int tok = __ldcg(&a.tokens[(int64_t)b * L + i]);
         const bool tok_ok = tok >= 0 && tok < V;
-        float omega = a.schedule[i];
+        float omega = __ldcg(&a.schedule[i]);
         omega = omega >= 0.0f ? omega : 0.0f;
         float f = 0.0f, p = __int_as_float(0x7fc00000), q = p;
         if (!t_ok || !d_ok) flag = 1;
@@ -765,7 +769,7 @@ __device__ void finish_sequence(const FinishArgs& a, const int b, const int tid,
           else if (dt == CSD_NEG_INF) f = 0.0f;    // p = 0 < q
           else f = fminf(1.0f, omega * grow * ex2f((dt - dd) * kLog2e) * ((1.0f + S[1]) / (1.0f + S[0])));
         }
-        const float r = a.uniforms[(int64_t)b * (L + 1) + i];
+        const float r = __ldcg(&a.uniforms[(int64_t)b * (L + 1) + i]);
         sm.acc[i] = (r <= f) ? 1 : 0;
         if (a.dbg_p) a.dbg_p[(int64_t)b * L + i] = p;
         if (a.dbg_q) a.dbg_q[(int64_t)b * L + i] = q;
@@ -804,13 +808,13 @@ __device__ void finish_sequence(const FinishArgs& a, const int b, const int tid,
     ctx.Md = j < L ? sm.M[1][j] : 0.0f; ctx.Sd = j < L ? sm.S[1][j] : 0.0f;
     ctx.inv_t = 1.0f / (1.0f + ctx.St);
     ctx.inv_den = ctx.inv_t / (1.0f + ctx.Sd);
-    float omega = j < L ? a.schedule[j] : 0.0f;
+    float omega = j < L ? __ldcg(&a.schedule[j]) : 0.0f;
     omega = omega >= 0.0f ? omega : 0.0f;
     ctx.one_minus_omega = 1.0f - omega;
     Row<T, CFG> rt{tgt + (int64_t)j * V, CFG ? tgt_u + (int64_t)j * V : nullptr, a.cfg_scale, sm.thr[0][j] CSD_ROW_LEN(V)};
     Row<T, CFG> rd = rt;
     if (j < L) rd = Row<T, CFG>{dft + (int64_t)j * V, CFG ? dft_u + (int64_t)j * V : nullptr, a.cfg_scale, sm.thr[1][j] CSD_ROW_LEN(V)};
-    const float u = a.uniforms[(int64_t)b * (L + 1) + L];
+    const float u = __ldcg(&a.uniforms[(int64_t)b * (L + 1) + L]);
     // (omega >= 1: the aggregated mass only raises f above f_van, and Eq. opt_G is the vanilla residual)
     const bool similar = a.nbr != nullptr && j < L && omega < 1.0f && ctx.mode == 0;
     // Every candidate with target mass then needs the mass of up to k neighbours: where the block's shared
@@ -925,7 +929,7 @@ __device__ void finish_sequence(const FinishArgs& a, const int b, const int tid,
   // ---- 8. emit x_{1:tau+1} ---------------------------------------------------------
   if (tid <= L) {
     int v = -1;
-    if (tid < tau) v = a.tokens[(int64_t)b * L + tid];
+    if (tid < tau) v = __ldcg(&a.tokens[(int64_t)b * L + tid]);
     else if (tid == tau) v = token;
     a.out_tokens[(int64_t)b * (L + 1) + tid] = v;
   }
@@ -943,7 +947,7 @@ __device__ void finish_sequence(const FinishArgs& a, const int b, const int tid,
         TermsCtx tc;
         tc.Mt = sm.M[0][i]; tc.Md = sm.M[1][i];
         tc.inv_t = 1.0f / (1.0f + sm.S[0][i]); tc.inv_d = 1.0f / (1.0f + sm.S[1][i]);
-        const float om = a.schedule[i];
+        const float om = __ldcg(&a.schedule[i]);
         tc.omega = om >= 0.0f ? om : 0.0f;
         const Row<T, CFG> rt{tgt + (int64_t)i * V, CFG ? tgt_u + (int64_t)i * V : nullptr, a.cfg_scale, sm.thr[0][i] CSD_ROW_LEN(V)};
         const Row<T, CFG> rd{dft + (int64_t)i * V, CFG ? dft_u + (int64_t)i * V : nullptr, a.cfg_scale, sm.thr[1][i] CSD_ROW_LEN(V)};

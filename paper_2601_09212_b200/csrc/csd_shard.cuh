@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) shard_merge_kernel(const ShardArgs a) {
     const int which = r < f.T ? 0 : 1, i = r < f.T ? r : r - f.T;
     float tokz = CSD_NEG_INF;
     if (i < f.gamma) {
-      const int loc = f.tokens[(int64_t)b * f.gamma + i] - a.v_offset;
+      const int loc = __ldcg(&f.tokens[(int64_t)b * f.gamma + i]) - a.v_offset;
       if (loc >= 0 && loc < f.V) {
         const T* base = reinterpret_cast<const T*>(which == 0 ? f.target : f.draft);
         const T* ubase = CFG ? reinterpret_cast<const T*>(which == 0 ? f.target_uncond : f.draft_uncond) : nullptr;
@@ -105,9 +105,9 @@ __device__ __forceinline__ int shard_accept(const ShardArgs& a, const int b, Sha
   if (tid < L) {
     const int i = tid;
     const bool t_ok = sm.valid[0][i], d_ok = sm.valid[1][i];
-    const int tok = f.tokens[(int64_t)b * L + i];
+    const int tok = __ldcg(&f.tokens[(int64_t)b * L + i]);
     const bool tok_ok = tok >= 0 && tok < a.V_total;
-    float omega = f.schedule[i];
+    float omega = __ldcg(&f.schedule[i]);
     omega = omega >= 0.0f ? omega : 0.0f;
     float fa = 0.0f, p = __int_as_float(0x7fc00000), q = p;
     int flag = 0;
@@ -121,7 +121,7 @@ __device__ __forceinline__ int shard_accept(const ShardArgs& a, const int b, Sha
       else if (dt == CSD_NEG_INF) fa = 0.0f;    // p = 0 < q
       else fa = fminf(1.0f, omega * ex2f((dt - dd) * kLog2e) * ((1.0f + sm.S[1][i]) / (1.0f + sm.S[0][i])));
     }
-    sm.acc[i] = (f.uniforms[(int64_t)b * (L + 1) + i] <= fa) ? 1 : 0;
+    sm.acc[i] = (__ldcg(&f.uniforms[(int64_t)b * (L + 1) + i]) <= fa) ? 1 : 0;
     sm.flag[i] = flag;
     if (dbg_row) { dbg_row[0] = p; dbg_row[1] = q; dbg_row[2] = fa; }
   }
@@ -184,6 +184,7 @@ template <typename T, bool CFG>
 __global__ void __launch_bounds__(kFinishThreads, 1) shard_partial_kernel(const ShardArgs a) {
   __shared__ ShardSmem sm;
   const FinishArgs& f = a.fin;
+  pdl_wait();
   constexpr int TILE = 32 * Elem<T>::kVec;
   const int tid = threadIdx.x, b = blockIdx.x, L = f.gamma;
   const int ntiles = (f.V + TILE - 1) / TILE;
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_partial_kernel(const 
   pc.Md = j < L ? sm.M[1][j] : 0.0f; pc.Sd = j < L ? sm.S[1][j] : 0.0f;
   pc.inv_t = 1.0f / (1.0f + pc.St);
   pc.inv_den = pc.inv_t / (1.0f + pc.Sd);
-  float omega = j < L ? f.schedule[j] : 0.0f;
+  float omega = j < L ? __ldcg(&f.schedule[j]) : 0.0f;
   omega = omega >= 0.0f ? omega : 0.0f;
   pc.one_minus_omega = 1.0f - omega;
   pc.mode = mode == 0 ? 0 : 1;
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_partial_kernel(const 
     ShardDraw d;
     d.Mt = pc.Mt; d.St = pc.St; d.Md = pc.Md; d.Sd = pc.Sd;
     d.one_minus_omega = pc.one_minus_omega;
-    d.u = f.uniforms[(int64_t)b * (L + 1) + L];
+    d.u = __ldcg(&f.uniforms[(int64_t)b * (L + 1) + L]);
     d.j = j; d.mode = mode; d.tau = tau; d.status = status;
     for (int k = 0; k < 6; ++k) d.pad[k] = 0;
     const float4* src = reinterpret_cast<const float4*>(&d);
@@ -248,6 +249,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_pick_kernel(const Sha
   __shared__ FinishSmem sm;
   __shared__ double sh_target, sh_pre;
   __shared__ int sh_owner, sh_fallback;
+  pdl_wait();
   const FinishArgs& f = a.fin;
   constexpr int VEC = Elem<T>::kVec;
   constexpr int TILE = 32 * VEC;
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_pick_kernel(const Sha
   ShardDraw d;
   {
     float4* dst = reinterpret_cast<float4*>(&d);
-    for (int k = 0; k < 4; ++k) dst[k] = a.ctx[4 * b + k];
+    for (int k = 0; k < 4; ++k) dst[k] = __ldcg(&a.ctx[4 * b + k]);
   }
   int status = d.status, token = -1;
   if (d.mode >= 0) {
@@ -269,12 +271,12 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_pick_kernel(const Sha
     if (tid == 0) {
       // totals of all slices, in vocabulary order; an empty positive part falls back to P_j
       double Z = 0.0;
-      for (int k = 0; k < a.n_shards; ++k) Z += a.z_all[((int64_t)k * f.B + b) * 2];
+      for (int k = 0; k < a.n_shards; ++k) Z += __ldcg(&a.z_all[((int64_t)k * f.B + b) * 2]);
       int which = 0;
       if (d.mode == 0 && !(Z > 0.0 && Z < (double)CSD_POS_INF)) {
         which = 1;
         Z = 0.0;
-        for (int k = 0; k < a.n_shards; ++k) Z += a.z_all[((int64_t)k * f.B + b) * 2 + 1];
+        for (int k = 0; k < a.n_shards; ++k) Z += __ldcg(&a.z_all[((int64_t)k * f.B + b) * 2 + 1]);
       }
       const double target = (double)d.u * Z;
       // the first slice whose running total passes the target owns the token; if none does (u >= 1,
@@ -283,7 +285,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) shard_pick_kernel(const Sha
       int owner = -1, last = -1;
       double pre_last = 0.0;
       for (int k = 0; k < a.n_shards; ++k) {
-        const double zk = a.z_all[((int64_t)k * f.B + b) * 2 + which];
+        const double zk = __ldcg(&a.z_all[((int64_t)k * f.B + b) * 2 + which]);
         if (zk > 0.0) { last = k; pre_last = c; }
         if (owner < 0 && zk > 0.0 && c + zk > target) { owner = k; pre = c; }
         c += zk;
@@ -334,20 +336,21 @@ __global__ void shard_emit_kernel(const ShardArgs a) {
   const FinishArgs& f = a.fin;
   const int b = blockIdx.x, tid = threadIdx.x, L = f.gamma;
   __shared__ int sh_tok, sh_status;
+  pdl_wait();
   if (tid == 0) {
     int tok = -1, status = 0;
     for (int k = 0; k < a.n_shards; ++k) {
-      tok = max(tok, a.cand_all[((int64_t)k * f.B + b) * 2]);
-      status |= a.cand_all[((int64_t)k * f.B + b) * 2 + 1];
+      tok = max(tok, __ldcg(&a.cand_all[((int64_t)k * f.B + b) * 2]));
+      status |= __ldcg(&a.cand_all[((int64_t)k * f.B + b) * 2 + 1]);
     }
     sh_tok = tok; sh_status = status;
   }
   __syncthreads();
   const ShardDraw* d = reinterpret_cast<const ShardDraw*>(a.ctx + 4 * b);
-  const int tau = d->tau;
+  const int tau = __ldcg(&d->tau);
   if (tid <= L) {
     int v = -1;
-    if (tid < tau) v = f.tokens[(int64_t)b * L + tid];
+    if (tid < tau) v = __ldcg(&f.tokens[(int64_t)b * L + tid]);
     else if (tid == tau) v = sh_tok;
     f.out_tokens[(int64_t)b * (L + 1) + tid] = v;
   }

@@ -112,9 +112,9 @@ __global__ void __launch_bounds__(kFinishThreads, 1) tree_finish_kernel(const Tr
 
   if (tid < N) {
     const int n = tid, c = a.parent[n] + 1;
-    const int tok = f.tokens[(int64_t)b * N + n];
+    const int tok = __ldcg(&f.tokens[(int64_t)b * N + n]);
     sm.tok[n] = tok;
-    sm.uni[n] = f.uniforms[(int64_t)b * (N + 1) + n];
+    sm.uni[n] = __ldcg(&f.uniforms[(int64_t)b * (N + 1) + n]);
     float zt = 0.0f, zd = 0.0f;
     if (tok >= 0 && tok < V && sm.valid[0][c] && sm.valid[1][c]) {
       const Row<T, CFG> qt{tgt + (int64_t)c * V, CFG ? tgt_u + (int64_t)c * V : nullptr, f.cfg_scale, sm.thr[0][c] CSD_ROW_LEN(V)};
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) tree_finish_kernel(const Tr
   __syncthreads();
 
   // ---- the walk (every thread follows it; thread 0 takes the accept decisions) ---------------
-  const float u = f.uniforms[(int64_t)b * (N + 1) + N];
+  const float u = __ldcg(&f.uniforms[(int64_t)b * (N + 1) + N]);
   int status = 0, level = 0, ctx = 0, token = -1;
   int k = 0;                // rejections in the final context (depth of the residual drawn from)
   bool drew = false;
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) tree_finish_kernel(const Tr
     pc.mode = d_ok ? 0 : 1;
     pc.Md = d_ok ? sm.M[1][ctx] : 0.0f; pc.Sd = d_ok ? sm.S[1][ctx] : 0.0f;
     pc.inv_den = pc.inv_t / (1.0f + pc.Sd);
-    omega = f.schedule[level];
+    omega = __ldcg(&f.schedule[level]);
     omega = omega >= 0.0f ? omega : 0.0f;
     pc.one_minus_omega = 1.0f - omega;
     int accepted = -1;
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kFinishThreads, 1) tree_finish_kernel(const Tr
     }
     if (accepted >= 0) {
       if (tid == 0) {
-        sm.path_tok[level] = f.tokens[(int64_t)b * N + accepted];
+        sm.path_tok[level] = __ldcg(&f.tokens[(int64_t)b * N + accepted]);
         sm.path_node[level] = accepted;
       }
       ++level;
