@@ -2,15 +2,18 @@
 // Every step of the method runs in the kernels of csd_kernels.cuh; nothing here
 // touches logits.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "../../include/csd.h"
 #include "csd_kernels.cuh"
 #include "csd_fused.cuh"
+#include "csd_slice.cuh"
 #include "csd_tree.cuh"
 #include "csd_shard.cuh"
 
@@ -215,6 +218,154 @@ cudaError_t launch_finish(const FinishArgs& a_in, cudaStream_t stream) {
 // Test aids (csd_test_hooks): process-wide, read at every launch of the single-launch path.
 long long g_wait_limit = kWaitCycles;
 int g_drop_first_copy = 0;
+
+// ---- the vocabulary-sliced kernel (csd_slice.cuh) ------------------------------------------------------------
+constexpr size_t kSliceSmem[2] = {113 * 1024, 226 * 1024};   // two blocks per SM, one block per SM
+
+void slice_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int grid, int c, size_t smem, cudaStream_t stream) {
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kSliceThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)c;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+}
+
+// Sequences in clusters of 2^log2c blocks that the GPU holds at once, for each of the two shared-memory sizes; asked
+// once per kernel and device.
+template <typename K>
+int slice_capacity(K kern, std::atomic<int> (&known)[kMaxDevices][5][2], int dev, int log2c, int cls) {
+  int k = known[dev][log2c][cls].load(std::memory_order_acquire);   // 0: not asked yet; -1: none
+  if (k == 0) {
+    int clusters = 0;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    slice_config(cfg, attr, 1 << log2c, 1 << log2c, kSliceSmem[cls], 0);
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceSmem[1]);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); clusters = 0; }
+    k = clusters > 0 ? clusters : -1;
+    known[dev][log2c][cls].store(k, std::memory_order_release);
+  }
+  return k;
+}
+
+// Shared-memory layout of a call split over c blocks; false if it does not fit `room` bytes.
+template <typename T, bool CFG>
+bool slice_layout(const SliceArgs& a, int R, int c, size_t room, SliceGeo& g, size_t& bytes) {
+  constexpr int ES = (int)sizeof(T), ARR = CFG ? 2 : 1, TILE = 32 * Elem<T>::kVec;
+  const int ntiles = (a.f.fin.V + TILE - 1) / TILE;
+  const int tiles = (ntiles + c - 1) / c, n = tiles * TILE, upr = (n + kSliceUnit - 1) / kSliceUnit;
+  g = a.g;
+  g.slot_bytes = (n * ES + (g.vec_ok ? 0 : 16)) * ARR;
+  g.wpr_log2 = 0;
+  while (g.wpr_log2 < 4 && (1 << g.wpr_log2) < upr) ++g.wpr_log2;
+  g.direct = (c << g.wpr_log2) <= 32 ? 1 : 0;
+  size_t off = kSliceHeader;
+  auto take = [&](size_t want) { const size_t o = off; off += (want + 127) / 128 * 128; return (int)o; };
+  g.rec_off = take((size_t)R * (g.direct ? c << g.wpr_log2 : c) * sizeof(float2));
+  g.tile_off = take((size_t)tiles * sizeof(double));
+  g.stash_off = take(g.direct ? 0 : ((size_t)R << g.wpr_log2) * sizeof(float2));
+  g.arena_off = (int)off;
+  if (off >= room) return false;
+  const size_t slots = (room - off) / g.slot_bytes;
+  g.slots = slots > (size_t)R ? R : (int)slots;
+  bytes = off + (size_t)g.slots * g.slot_bytes;
+  return g.slots >= (R < 4 ? R : 4);
+}
+
+// Launches the sliced kernel if it suits the call; *launched says whether it did (with `dry`, whether it would).
+// The split is the one with the fewest logits for the busiest SM to go through; where rows are aligned it has to leave
+// at most three quarters of what `other_work` says that the position split would give it.  That is where the lines lie
+// (us per call, sliced / position split): 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3 (0.71 of the
+// work), B=16 17.6 / 15.2 (1.4); 64 K bf16 B=4 18.0 / 23.2 (0.35), fp32 gamma=16 B=1 31.9 / 41.5 (0.41), B=8 48 / 42 (0.83).
+template <typename T, bool CFG>
+cudaError_t try_slice(SliceArgs& a, long long other_work, bool dry, cudaStream_t stream, bool* launched) {
+  constexpr int TILE = 32 * Elem<T>::kVec;
+  static std::atomic<int> known[kMaxDevices][5][2];
+  auto kern = verify_slice_kernel<T, CFG>;
+  const FinishArgs& f = a.f.fin;
+  const int R = f.T + f.gamma, ntiles = (f.V + TILE - 1) / TILE;
+  *launched = false;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (R > kSliceRows) return cudaSuccess;
+  long long best = a.g.vec_ok ? other_work * 3 / 4 + 1 : LLONG_MAX;
+  SliceGeo geo;
+  size_t bytes = 0;
+  int best_c = 0;
+  for (int log2c = 4; log2c >= 0; --log2c) {
+    const int c = 1 << log2c;
+    if (c > ntiles || (c > 1 && f.V / c < kSliceUnit)) continue;
+    const long long n = (long long)((ntiles + c - 1) / c) * TILE;
+    if (n * R >= best) continue;
+    // a block to an SM where the clusters fit so, with room for more rows at once; else two
+    const int cap1 = slice_capacity(kern, known, dev, log2c, 1), cap2 = slice_capacity(kern, known, dev, log2c, 0);
+    if (cap1 <= 0 || cap2 <= 0) continue;
+    const long long work = n * R * (f.B <= cap1 ? 1 : 2LL * ((f.B + cap2 - 1) / cap2));
+    if (best_c == 0 ? work >= best : work * 8 >= best * 7) continue;   // (more blocks if it is nearly as good: 24 unaligned
+                                                                       // rows of bf16, eight blocks 24.4, four 26.8)
+    SliceGeo g;
+    size_t need;
+    bool fits = slice_layout<T, CFG>(a, R, c, kSliceSmem[0], g, need);
+    if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG>(a, R, c, kSliceSmem[1], g, need);
+    if (!fits) continue;
+    best = work;
+    best_c = c;
+    geo = g;
+    bytes = need;
+  }
+  if (best_c == 0) return cudaSuccess;
+  *launched = true;
+  if (dry) return cudaSuccess;
+  a.g = geo;
+  a.f.ctas_per_seq = best_c;
+  a.f.signal = 1;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  slice_config(cfg, attr, f.B * best_c, best_c, bytes, stream);
+  return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// A call as the sliced kernel sees it, and its launch.
+struct SliceCall {
+  FinishArgs fa;
+  int dtype;
+  bool cfg;
+  int* error_flag;
+  int sms;
+};
+cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool* launched) {
+  *launched = false;
+  // The position split's work for its busiest SM (see plan_and_launch_fused).  Once it fills the GPU it streams better
+  // than slices do (fp32 B=32: 16.9 us, sliced 21.1).
+  const int B = in.fa.B, gamma = in.fa.gamma;
+  int pos = 1;
+  while (2 * pos <= 2 * in.sms / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
+  if (in.fa.vec_ok && (long long)B * pos > in.sms) return cudaSuccess;
+  const long long rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
+  const long long other_work = rows * in.fa.V;
+  SliceArgs a;
+  memset(&a, 0, sizeof a);
+  a.f.fin = in.fa;
+  a.f.error_flag = in.error_flag;
+  a.f.wait_limit = g_wait_limit;
+  a.f.drop_first_copy = g_drop_first_copy;
+  a.f.ordered = 1;
+  a.g.vec_ok = in.fa.vec_ok;
+  if (in.dtype == CSD_F32)
+    return in.cfg ? try_slice<float, true>(a, other_work, dry, stream, launched) : try_slice<float, false>(a, other_work, dry, stream, launched);
+  return in.cfg ? try_slice<__nv_bfloat16, true>(a, other_work, dry, stream, launched) : try_slice<__nv_bfloat16, false>(a, other_work, dry, stream, launched);
+}
 
 // The single-launch path's partition and launch (see the comments inside).  With stats_out set the
 // kernels stop after their streaming phase and write every row's (m, s) -- and, with top-k, its exact
@@ -453,8 +604,19 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
   // statistics still come from the streaming kernels (one launch, every logit read once)
   const bool stream_stats = !fused && similar.nbr != nullptr && !no_workspace && vec_ok && (size_t)p.V * es >= 512 &&
                             (p.V + 32 * vw - 1) / (32 * vw) <= kFinTiles;
+  // ---- stream order, few sequences or unaligned rows: the vocabulary-sliced kernel -----------------------------
+  bool sliced = false;
+  if (similar.nbr == nullptr && !topk && !p.diag_accept_mass && !p.diag_bound_term && (!fused || !p.back_to_back) && p.V >= 512) {
+    SliceCall sc;
+    sc.fa = fa;
+    sc.dtype = p.dtype; sc.cfg = cfg; sc.sms = sms;
+    sc.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
+    const cudaError_t e = slice_call(sc, plan_only != nullptr, stream, &sliced);
+    if (e != cudaSuccess) return CSD_ERR_LAUNCH;
+    if (sliced && !plan_only) return CSD_OK;
+  }
   if (plan_only) {  // number of kernels this call would enqueue
-    *plan_only = fused ? 1 : (stream_stats ? 2 : (topk ? 3 : 2));
+    *plan_only = (fused || sliced) ? 1 : (stream_stats ? 2 : (topk ? 3 : 2));
     return CSD_OK;
   }
   if (fused) {

@@ -1,0 +1,80 @@
+"""The vocabulary-sliced kernel at the edges of its layout: slices of one unit and just beside it, every cluster size,
+rows that do not all fit a block's shared memory at once, parts of a row that are merged before they are exchanged, and
+rows at every offset from a 16-byte boundary.  Tolerances are those of the other parity tests (tests/gpu_util.py)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2601_09212_b200 as csd
+from paper_2601_09212_b200 import workloads as W
+from gpu_util import check, run_gpu
+
+DEV = "cuda"
+
+
+def _make(kw, seed=5):
+    L = kw["gamma"]
+    return W.make("t", schedule=csd.csd_make_schedule(1, 1.2, 0.6, L), seed=seed, device=DEV, **kw)
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=1, gamma=1, V=512),                                            # one unit, one block
+    dict(B=1, gamma=2, V=1020, dtype=W.F32), dict(B=2, gamma=3, V=1024),  # a ragged second block / two whole ones
+    dict(B=3, gamma=4, V=8192), dict(B=3, gamma=4, V=8188, bonus_row=True),   # sixteen blocks of one unit / ragged
+    dict(B=2, gamma=5, V=8200, dtype=W.BF16, bonus_row=True),             # a block with one short tile more
+    dict(B=14, gamma=8, V=16384, bonus_row=True), dict(B=15, gamma=8, V=16384, bonus_row=True),   # sixteen / eight blocks
+    dict(B=1, gamma=16, V=65536, bonus_row=True),                         # rows in turns through the slots
+    dict(B=1, gamma=32, V=32768, dtype=W.BF16, bonus_row=True),           # 65 rows
+    dict(B=2, gamma=4, V=131072, dtype=W.BF16),                           # parts merged before the exchange
+    dict(B=4, gamma=3, V=20000, cfg=True, cfg_scale=3.0, bonus_row=True),
+    dict(B=4, gamma=6, V=65536, dtype=W.BF16, cfg=True, cfg_scale=3.0),
+])
+def test_layout_edges(kw):
+    w = _make(kw)
+    rep, got, _ = check(w, want_dbg=kw["B"] * kw["V"] <= 300000)
+    assert rep.ok and rep.tau_mismatch_near + rep.token_mismatch_near <= 1, rep.summary()
+    other = run_gpu(w, want_dbg=False, back_to_back=True)   # the same round on the position split
+    same = (got["tokens"] == other["tokens"]).all(axis=1) & (got["accept_len"] == other["accept_len"])
+    assert (~same).sum() <= 1, kw   # (two summation orders: one sequence may sit on a boundary)
+
+
+@pytest.mark.parametrize("shift", range(8))
+@pytest.mark.parametrize("dtype,cfg", [(W.F32, False), (W.BF16, False), (W.BF16, True)])
+def test_every_alignment(shift, dtype, cfg):
+    """Rows of odd length, arrays beginning `shift` elements past a 16-byte boundary (the drafter's and the unconditional
+    ones at other offsets): the same results as the aligned copy's oracle."""
+    w = _make(dict(B=3, gamma=4, V=2051, dtype=dtype, bonus_row=True, cfg=cfg), seed=7 + shift)
+
+    def moved(t, by):
+        if t is None:
+            return None
+        buf = torch.empty(t.numel() + 16, dtype=t.dtype, device=DEV)
+        buf[by:by + t.numel()] = t.reshape(-1)
+        return buf[by:by + t.numel()].view(t.shape)
+
+    w.target_logits, w.draft_logits = moved(w.target_logits, shift), moved(w.draft_logits, (shift + 3) % 8)
+    w.target_uncond, w.draft_uncond = moved(w.target_uncond, (shift + 5) % 8), moved(w.draft_uncond, (shift + 6) % 8)
+    rep, _, _ = check(w)
+    assert rep.ok and rep.tau_mismatch_near + rep.token_mismatch_near <= 1, rep.summary()
+
+
+@pytest.mark.parametrize("R,V", [(1, 512), (64, 16384), (70, 16387), (148, 4096), (300, 3001)])
+def test_drafting_draws(R, V):
+    """One token per row: slices and the whole-row blocks draw the same tokens."""
+    w = _make(dict(B=R, gamma=1, V=V, dtype=W.BF16, cfg=True), seed=3)
+    rows, unc, u = w.draft_logits[:, 0].contiguous(), w.draft_uncond[:, 0].contiguous(), w.uniforms[:, 0].contiguous()
+    outs = []
+    for b2b in (False, True):
+        out = torch.empty(R, dtype=torch.int32, device=DEV)
+        csd.csd_sample_rows(rows, u, out, uncond=unc, cfg_scale=w.cfg_scale, back_to_back=b2b)
+        outs.append(out.cpu().numpy())
+    z = torch.addcmul(unc.float(), rows.float() - unc.float(), torch.tensor(w.cfg_scale, device=DEV)).double()
+    cdf = torch.softmax(z, -1).cumsum(-1)
+    want = (cdf <= (u.double() * cdf[:, -1])[:, None]).sum(-1).cpu().numpy()
+    for out in outs:
+        assert (out != want).sum() <= 1
