@@ -86,6 +86,25 @@ double normal_upper_quantile(double tail) {
   return tail < 0.5 ? x : -x;
 }
 
+// Top-k: the streaming selection's levels, from k and V alone.  `lo` expects `tail` V values at or above it, a little more
+// than k; `hi` is its mirror image, a level with, almost surely, fewer than k values above it (NaN where k is too
+// small for one).  False if too large a share of the row would lie above lo.
+struct TopkGuess {
+  double tail;
+  float lo_sigmas, lo_delta, hi_delta;
+};
+bool topk_guess(double k, double v, TopkGuess& g) {
+  g.tail = 1.25 * k / v + 4.0 * sqrt(k) / v + 16.0 / v;
+  g.lo_sigmas = g.hi_delta = nanf("");
+  g.lo_delta = 0.0f;
+  if (g.tail >= 0.45) return false;
+  g.lo_sigmas = (float)normal_upper_quantile(g.tail);
+  g.lo_delta = g.lo_sigmas - (float)normal_upper_quantile(k / v);
+  const double tail_hi = 0.75 * k / v - 4.0 * sqrt(k) / v - 16.0 / v;
+  if (tail_hi * v >= 8.0) g.hi_delta = (float)normal_upper_quantile(tail_hi) - g.lo_sigmas;
+  return true;
+}
+
 // Launches one of the single-launch kernels (KERNEL: 0 plain, 1 top-k on rows that are a whole
 // number of stages, 2 top-k on any row length, 3 and 4 the same two with the large candidate lists) with its shared-memory size, as a programmatic
 // dependent launch and, for ctas_per_seq > 1, as clusters of that many blocks.
@@ -260,8 +279,9 @@ int slice_capacity(K kern, std::atomic<int> (&known)[kMaxDevices][5][2], int dev
 }
 
 // Shared-memory layout of a call split over c blocks; false if it does not fit `room` bytes.
-template <typename T, bool CFG>
-bool slice_layout(const SliceArgs& a, int R, int c, size_t room, SliceGeo& g, size_t& bytes) {
+// `tail`: the share of a row that the top-k lists expect.
+template <typename T, bool CFG, bool TOPK>
+bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, SliceGeo& g, size_t& bytes) {
   constexpr int ES = (int)sizeof(T), ARR = CFG ? 2 : 1, TILE = 32 * Elem<T>::kVec;
   const int ntiles = (a.f.fin.V + TILE - 1) / TILE;
   const int tiles = (ntiles + c - 1) / c, n = tiles * TILE, upr = (n + kSliceUnit - 1) / kSliceUnit;
@@ -272,9 +292,17 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, SliceGeo& g, si
   g.direct = (c << g.wpr_log2) <= 32 ? 1 : 0;
   size_t off = kSliceHeader;
   auto take = [&](size_t want) { const size_t o = off; off += (want + 127) / 128 * 128; return (int)o; };
-  g.rec_off = take((size_t)R * (g.direct ? c << g.wpr_log2 : c) * sizeof(float2));
+  const size_t owned = (size_t)(R + c - 1) / c;   // top-k: rows whose lists a block receives
+  g.rec_off = take((size_t)R * (TOPK ? (size_t)c * sizeof(float4) : (size_t)(g.direct ? c << g.wpr_log2 : c) * sizeof(float2)));
   g.tile_off = take((size_t)tiles * sizeof(double));
-  g.stash_off = take(g.direct ? 0 : ((size_t)R << g.wpr_log2) * sizeof(float2));
+  g.stash_off = take(TOPK ? owned * c * sizeof(int) : (g.direct ? 0 : ((size_t)R << g.wpr_log2) * sizeof(float2)));
+  if (TOPK) {
+    const double e = tail * n;   // values a slice's list expects
+    g.list_cap = ((int)(1.25 * e + 6.0 * sqrt(e) + 24.0) + 3) / 4 * 4;
+    if (g.list_cap > n) g.list_cap = n;
+    g.list_off = take(sizeof(SliceTopk) + (size_t)R * g.list_cap * sizeof(float));
+    g.own_off = take(owned * c * g.list_cap * sizeof(float));
+  }
   g.arena_off = (int)off;
   if (off >= room) return false;
   const size_t slots = (room - off) / g.slot_bytes;
@@ -287,12 +315,12 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, SliceGeo& g, si
 // The split is the one with the fewest logits for the busiest SM to go through; where rows are aligned it has to leave
 // at most three quarters of what `other_work` says that the position split would give it.  That is where the lines lie
 // (us per call, sliced / position split): 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3 (0.71 of the
-// work), B=16 17.6 / 15.2 (1.4); 64 K bf16 B=4 18.0 / 23.2 (0.35), fp32 gamma=16 B=1 31.9 / 41.5 (0.41), B=8 48 / 42 (0.83).
-template <typename T, bool CFG>
-cudaError_t try_slice(SliceArgs& a, long long other_work, bool dry, cudaStream_t stream, bool* launched) {
+// work), B=16 17.6 / 15.2 (1.4); guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; 64 K bf16 B=4 18.0 / 23.2 (0.35), fp32 gamma=16 B=1 31.9 / 41.5 (0.41), B=8 48 / 42 (0.83).
+template <typename T, bool CFG, bool TOPK>
+cudaError_t try_slice(SliceArgs& a, long long other_work, double tail, bool dry, cudaStream_t stream, bool* launched) {
   constexpr int TILE = 32 * Elem<T>::kVec;
   static std::atomic<int> known[kMaxDevices][5][2];
-  auto kern = verify_slice_kernel<T, CFG>;
+  auto kern = verify_slice_kernel<T, CFG, TOPK>;
   const FinishArgs& f = a.f.fin;
   const int R = f.T + f.gamma, ntiles = (f.V + TILE - 1) / TILE;
   *launched = false;
@@ -313,11 +341,11 @@ cudaError_t try_slice(SliceArgs& a, long long other_work, bool dry, cudaStream_t
     if (cap1 <= 0 || cap2 <= 0) continue;
     const long long work = n * R * (f.B <= cap1 ? 1 : 2LL * ((f.B + cap2 - 1) / cap2));
     if (best_c == 0 ? work >= best : work * 8 >= best * 7) continue;   // (more blocks if it is nearly as good: 24 unaligned
-                                                                       // rows of bf16, eight blocks 24.4, four 26.8)
+                                                                       // sequences, bf16: eight blocks 24.4, four 26.8)
     SliceGeo g;
     size_t need;
-    bool fits = slice_layout<T, CFG>(a, R, c, kSliceSmem[0], g, need);
-    if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG>(a, R, c, kSliceSmem[1], g, need);
+    bool fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[0], tail, g, need);
+    if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[1], tail, g, need);
     if (!fits) continue;
     best = work;
     best_c = c;
@@ -339,8 +367,8 @@ cudaError_t try_slice(SliceArgs& a, long long other_work, bool dry, cudaStream_t
 // A call as the sliced kernel sees it, and its launch.
 struct SliceCall {
   FinishArgs fa;
-  int dtype;
-  bool cfg;
+  int dtype, top_k;
+  bool cfg, topk, exact;   // exact: every row's exact threshold is wanted
   int* error_flag;
   int sms;
 };
@@ -350,10 +378,14 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   // than slices do (fp32 B=32: 16.9 us, sliced 21.1).
   const int B = in.fa.B, gamma = in.fa.gamma;
   int pos = 1;
-  while (2 * pos <= 2 * in.sms / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
+  const int split_below = (in.topk ? 4 : 2) * in.sms;
+  while (2 * pos <= split_below / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
   if (in.fa.vec_ok && (long long)B * pos > in.sms) return cudaSuccess;
   const long long rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
   const long long other_work = rows * in.fa.V;
+  // (with top-k the two exchanges before the accept tests want something to save: a row of 16 K a block, the drafting
+  // stage's, takes 13.6 us whole and 15.1 sliced; three rows 23.6 and 18.0)
+  if (in.topk && in.fa.vec_ok && other_work < 24 * 1024) return cudaSuccess;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;
@@ -362,9 +394,23 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   a.f.drop_first_copy = g_drop_first_copy;
   a.f.ordered = 1;
   a.g.vec_ok = in.fa.vec_ok;
-  if (in.dtype == CSD_F32)
-    return in.cfg ? try_slice<float, true>(a, other_work, dry, stream, launched) : try_slice<float, false>(a, other_work, dry, stream, launched);
-  return in.cfg ? try_slice<__nv_bfloat16, true>(a, other_work, dry, stream, launched) : try_slice<__nv_bfloat16, false>(a, other_work, dry, stream, launched);
+  a.g.exact = in.exact ? 1 : 0;
+  TopkGuess guess;
+  guess.tail = 0.0;
+  if (in.topk) {
+    if (!topk_guess(in.top_k, in.fa.V, guess)) return cudaSuccess;
+    a.f.top_k = in.top_k;
+    a.f.lo_sigmas = guess.lo_sigmas;
+    a.f.hi_delta = guess.hi_delta;
+  }
+#define CSD_SLICE(T, CFG, TOPK) try_slice<T, CFG, TOPK>(a, other_work, guess.tail, dry, stream, launched)
+  if (in.dtype == CSD_F32) {
+    if (in.cfg) return in.topk ? CSD_SLICE(float, true, true) : CSD_SLICE(float, true, false);
+    return in.topk ? CSD_SLICE(float, false, true) : CSD_SLICE(float, false, false);
+  }
+  if (in.cfg) return in.topk ? CSD_SLICE(__nv_bfloat16, true, true) : CSD_SLICE(__nv_bfloat16, true, false);
+  return in.topk ? CSD_SLICE(__nv_bfloat16, false, true) : CSD_SLICE(__nv_bfloat16, false, false);
+#undef CSD_SLICE
 }
 
 // The single-launch path's partition and launch (see the comments inside).  With stats_out set the
@@ -409,8 +455,9 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     // until the GPU is full.
     const long long merge_above = 8LL * sms;   // beyond this many sequences a block takes several
     // (measured: the top-k kernel, with its longer per-row work, gains from the finer split)
-    const double tk_k = in.top_k, tk_v = in.V;
-    const double tk_tail = 1.25 * tk_k / tk_v + 4.0 * sqrt(tk_k) / tk_v + 16.0 / tk_v;
+    TopkGuess guess;
+    const bool guessed = topk && topk_guess(in.top_k, in.V, guess);
+    const double tk_v = in.V, tk_tail = topk ? guess.tail : 0.0;
     const bool tk_large = topk && tk_tail * tk_v >= 0.8 * (kTopkWarps * kWarpList);
     const long long split_below = in.back_to_back ? 16 : (topk ? 4LL : 2LL) * sms;
     long long c = 1, spc = 1;
@@ -423,20 +470,16 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     if (topk) {
       ua.chunks_per_part = 0;
       ua.parts_per_row = 1;
-      const double k = tk_k, v = tk_v, tail = tk_tail;
       // the candidates must fit the per-warp lists with room to spare: the small lists (four blocks per SM)
       // where they do, else the large ones (three blocks per SM), else every row is selected exactly
       ua.large_lists = tk_large ? 1 : 0;
-      if (tail < 0.45 && tail * v < 0.8 * (kTopkWarps * kWarpListLarge)) {
-        ua.lo_sigmas = (float)normal_upper_quantile(tail);
-        ua.lo_delta = ua.lo_sigmas - (float)normal_upper_quantile(k / v);
-        // a level with, almost surely, fewer than k values above it: the mirror image of the guess.
-        // The short cut it serves keeps lo as the row's threshold, which the diagnostic outputs that
+      if (guessed && tk_tail * tk_v < 0.8 * (kTopkWarps * kWarpListLarge)) {
+        // The short cut that hi serves keeps lo as the row's threshold, which the diagnostic outputs that
         // evaluate every token (the distribution drawn from, the monitors) would show in their last
         // digits: with them requested every row gets its exact threshold.
-        const double tail_hi = 0.75 * k / v - 4.0 * sqrt(k) / v - 16.0 / v;
-        if (tail_hi * v >= 8.0 && in.allow_short_cut)
-          ua.hi_delta = (float)normal_upper_quantile(tail_hi) - ua.lo_sigmas;
+        ua.lo_sigmas = guess.lo_sigmas;
+        ua.lo_delta = guess.lo_delta;
+        if (in.allow_short_cut) ua.hi_delta = guess.hi_delta;
       }
     } else {
       // warp-wide items: parts of rows, sized so that every warp of the grid gets several
@@ -606,10 +649,11 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
                             (p.V + 32 * vw - 1) / (32 * vw) <= kFinTiles;
   // ---- stream order, few sequences or unaligned rows: the vocabulary-sliced kernel -----------------------------
   bool sliced = false;
-  if (similar.nbr == nullptr && !topk && !p.diag_accept_mass && !p.diag_bound_term && (!fused || !p.back_to_back) && p.V >= 512) {
+  if (similar.nbr == nullptr && !p.diag_accept_mass && !p.diag_bound_term && (!fused || !p.back_to_back) && p.V >= 512) {
     SliceCall sc;
     sc.fa = fa;
-    sc.dtype = p.dtype; sc.cfg = cfg; sc.sms = sms;
+    sc.dtype = p.dtype; sc.top_k = p.top_k; sc.cfg = cfg; sc.topk = topk; sc.exact = p.dbg_G != nullptr;
+    sc.sms = sms;
     sc.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
     const cudaError_t e = slice_call(sc, plan_only != nullptr, stream, &sliced);
     if (e != cudaSuccess) return CSD_ERR_LAUNCH;

@@ -7,7 +7,8 @@
 // slice of all rows fits the block's shared memory each logit is fetched once:
 //   1. every row's slice comes in by one bulk copy per array, as many rows at once as fit (the rest follow as slots
 //      free up);
-//   2. each warp takes units of 512 logits and leaves (m, s) of its part of each row;
+//   2. each warp takes units of 512 logits and leaves (m, s) of its part of each row; with top-k the values not below a
+//      guessed level are gathered and sent to the block that owns the row, which settles it;
 //   3. the parts go into every block of the cluster (distributed shared memory); one cluster barrier later every
 //      block knows all rows' normalisers, so every warp runs all accept tests itself and nothing further is exchanged
 //      to agree on the first rejection;
@@ -23,6 +24,9 @@ constexpr int kSliceWarps = kSliceThreads / 32;
 constexpr int kSliceCluster = 16;       // blocks of a sequence (above 8: a non-portable cluster size)
 constexpr int kSliceRows = 128;
 constexpr int kSliceUnit = 512;         // logits of a warp's unit of work: 16 per lane
+constexpr int kSliceSample = 4096;      // top-k: logits of a row that the moments are taken from, over all blocks
+constexpr int kSliceBins = 128;         // per row being settled: histogram of the values between the two levels
+constexpr int kSliceCand = 64;          // per row being settled: values of the bin that holds the threshold
 static_assert(kSliceRows <= kBlockRows, "a block's row results live in RowStats");
 
 // How a call is laid out; chosen by the host.
@@ -31,7 +35,10 @@ struct SliceGeo {
   int vec_ok;              // rows are whole 16-byte vectors at 16-byte aligned addresses
   int wpr_log2;            // 2^this warps work on a row at once
   int direct;              // the warps' parts of a row go to the other blocks as they are (else merged first)
-  int rec_off, stash_off, tile_off, arena_off;   // dynamic shared memory after SliceSmem: offsets in bytes
+  int list_cap;            // top-k: values a row's list holds
+  int exact;               // top-k: every row's exact threshold is wanted
+  // dynamic shared memory after SliceSmem: offsets in bytes
+  int rec_off, stash_off, tile_off, list_off, own_off, arena_off;
 };
 struct SliceArgs {
   FusedArgs f;
@@ -50,6 +57,19 @@ struct SliceSmem {
   FinishSmem fin;
   FinishStage fst;
 };
+// ... and what top-k needs beside it (at list_off's head)
+struct SliceTopk {
+  alignas(16) float4 res[kSliceRows];   // (m, s, threshold, 1: the filter drops the drafted token), from the row's owner
+  float2 level[kSliceRows];  // (lo, hi)
+  int cnt[kSliceRows];       // length of the row's list (may run past its capacity)
+  unsigned need[kSliceRows / 32];       // rows of this block to be read again
+  float4 red[kSliceWarps][kSliceWarps];
+  float wmax[kSliceWarps][kSliceWarps];
+  int hist[kSliceWarps][kSliceBins];    // (rows read again use it as one)
+  float cand[kSliceWarps][kSliceCand];
+  int n_cand[kSliceWarps];
+  alignas(16) int bc_i[2];
+};
 constexpr int kSliceHeader = (int)((sizeof(SliceSmem) + 127) / 128 * 128);
 
 __device__ __forceinline__ uint32_t cluster_map(const void* local, uint32_t rank) {
@@ -59,6 +79,12 @@ __device__ __forceinline__ uint32_t cluster_map(const void* local, uint32_t rank
 }
 __device__ __forceinline__ void cluster_store_f2(float2* local, uint32_t rank, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(cluster_map(local, rank)), "f"(v.x), "f"(v.y) : "memory");
+}
+
+__device__ __forceinline__ void cluster_store_f4(void* local, uint32_t rank, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_map(local, rank)), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
 }
 
 // ---- the block's place -----------------------------------------------------------------------------------------
@@ -390,6 +416,381 @@ __device__ __forceinline__ bool slice_rows_plain(const Slice<T, CFG>& k) {
   return ok;
 }
 
+// ---- phase 1, top-k: every row's list of values not below its level, sent to the row's owner -----------------------
+// The moments of a sample of every row (about 4096 logits, from all blocks) give a level `lo` a little below the k-th
+// largest (the guess of verify_topk_kernel); the values not below it are gathered into the block's lists, and each row's
+// lists go to the block that owns the row.  Rows are taken in groups of as many as there are slots.  `late` puts the
+// drafted tokens' logits into shared memory.
+template <typename T, bool CFG, typename Late>
+__device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late late) {
+  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.list_off);
+  const FusedArgs& a = k.a.f;
+  const int slots = k.a.g.slots, R = k.R, cap = k.a.g.list_cap, lane = k.lane, c = k.c;
+  const int wl = k.a.g.wpr_log2, part = k.warp & ((1 << wl) - 1);
+  float4* const mom = reinterpret_cast<float4*>(k.base + k.a.g.rec_off);   // [c][R]: sum, sum of |deviations|, values
+  float* const lists = reinterpret_cast<float*>(k.base + k.a.g.list_off + sizeof(SliceTopk));
+  const int groups = (R + slots - 1) / slots, G = (R + groups - 1) / groups;
+  const uint32_t lanemask_lt = (1u << lane) - 1u;
+  // units of a row's slice in the sample: one warp takes them one after the other
+  const int su = min(k.upr, (kSliceSample / kSliceUnit + c - 1) / c);
+  bool ok = true, peers = c == 1;
+  for (int g0 = 0; g0 < R; g0 += G) {
+    const int g1 = min(R, g0 + G);
+    // ---- moments of the sample: its sum, and the sum of absolute deviations from each unit's mean --------------------
+    for (int r = g0 + k.warp; r < g1; r += kSliceWarps) {
+      if (ok && !k.wait_row(r)) ok = false;
+      const unsigned char *p, *pu;
+      k.slice_at(r, p, pu);
+      float s1 = 0.0f, s2 = 0.0f, cnt = 0.0f;
+      for (int u = 0; u < su; ++u) {
+        const int valid = min(kSliceUnit, k.n - u * kSliceUnit);
+        if (valid < kSliceUnit && u > 0) break;
+        float z[16];
+        k.unit(p, pu, u, z);
+        if (valid < kSliceUnit) {   // a slice of less than a unit: what lies beyond it does not count
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            if (k.unit_index(e) >= valid) z[e] = 0.0f;
+        }
+        uint64_t s1p = pack2(0.0f, 0.0f);
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) s1p = add2(s1p, pack2(z[e], z[e + 1]));
+        float x0, x1;
+        unpack2(s1p, x0, x1);
+        float us = x0 + x1;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) us += __shfl_xor_sync(0xffffffffu, us, off);
+        const float wm = us * rcp_approx((float)valid);
+        const uint64_t nwm = pack2(-wm, -wm);
+        float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+          unpack2(add2(pack2(z[e], z[e + 1]), nwm), x0, x1);
+          if (valid < kSliceUnit) {
+            if (k.unit_index(e) >= valid) x0 = 0.0f;
+            if (k.unit_index(e + 1) >= valid) x1 = 0.0f;
+          }
+          d0 += fabsf(x0);
+          d1 += fabsf(x1);
+        }
+        s1 += us;
+        s2 += d0 + d1;
+        cnt += (float)valid;
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+      if (!peers) { cluster_wait(); peers = true; }   // every peer is running
+      if (lane < c) cluster_store_f4(&mom[k.me * R + r], (uint32_t)lane, make_float4(s1, s2, cnt, 0.0f));
+    }
+    if (!peers) { cluster_wait(); peers = true; }
+    if (c > 1) { cluster_arrive(); cluster_wait(); }
+    else __syncthreads();
+    if (k.tid < g1 - g0) {
+      const int r = g0 + k.tid;
+      float s1 = 0.0f, s2 = 0.0f, cnt = 0.0f;
+      for (int q = 0; q < c; ++q) {
+        const float4 v = mom[q * R + r];
+        s1 += v.x; s2 += v.y; cnt += v.z;
+      }
+      const float inv = 1.0f / cnt;
+      const float dev = 1.2533141f * (s2 * inv);   // (the standard deviation, were the row Gaussian)
+      const float lo = s1 * inv + a.lo_sigmas * dev;
+      tk.level[r] = make_float2(lo, lo + a.hi_delta * dev);
+      tk.cnt[r] = 0;
+    }
+    __syncthreads();
+    // ---- gather (by the sign of z - lo, so that a NaN lands in the list; see verify_topk_kernel) -------------------
+    for (int r = g0 + (k.warp >> wl); r < g1; r += kSliceWarps >> wl) {
+      if (ok && !k.wait_row(r)) ok = false;
+      const unsigned char *p, *pu;
+      k.slice_at(r, p, pu);
+      const float lo = tk.level[r].x;
+      const uint64_t nlo2 = pack2(-lo, -lo);
+      const uint32_t list = smem_addr(lists + r * cap);
+      for (int u = part; u < k.upr; u += 1 << wl) {
+        float z[16];
+        k.unit(p, pu, u, z);
+        uint32_t below_lo = 0;
+#pragma unroll
+        for (int e = 14; e >= 0; e -= 2) {
+          float d0, d1;
+          unpack2(add2(pack2(z[e], z[e + 1]), nlo2), d0, d1);
+          below_lo = __funnelshift_l(__float_as_uint(d1), below_lo, 1);
+          below_lo = __funnelshift_l(__float_as_uint(d0), below_lo, 1);
+        }
+        const uint32_t mask = ~below_lo & 0xffffu;
+        const uint32_t cnt = (uint32_t)__popc(mask);
+        const uint32_t tot = __reduce_add_sync(0xffffffffu, cnt);
+        uint32_t start = 0;
+        if (lane == 0) start = (uint32_t)atom_add_shared(&tk.cnt[r], (int)tot);
+        uint32_t before = 0;
+#pragma unroll
+        for (int bit = 0; bit < 5; ++bit) {
+          const uint32_t bal = __ballot_sync(0xffffffffu, (cnt >> bit) & 1u);
+          before += (uint32_t)__popc(bal & lanemask_lt) << bit;
+        }
+        start = __shfl_sync(0xffffffffu, start, 0) + before;
+        if (start + cnt <= (uint32_t)cap) {
+          uint32_t addr = list + 4u * start;
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            if (mask & (1u << e)) {
+              asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(z[e]) : "memory");
+              addr += 4u;
+            }
+          }
+        }
+      }
+      k.release_row(r, ok);
+    }
+  }
+  late();
+  __syncthreads();
+  // ---- the lists go to the rows' owners: row r to block r % c --------------------------------------------------------
+  float* const own = reinterpret_cast<float*>(k.base + k.a.g.own_off);   // [rows owned][c][cap]
+  int* const own_cnt = reinterpret_cast<int*>(k.base + k.a.g.stash_off); // [rows owned][c]
+  for (int r = k.warp; r < R; r += kSliceWarps) {
+    const int len = min(tk.cnt[r], cap), oi = r / c, at = oi * c + k.me;
+    const uint32_t owner = (uint32_t)(r - oi * c);
+    for (int i = 4 * lane; i < len; i += 128) {
+      const float4 v = *reinterpret_cast<const float4*>(lists + r * cap + i);
+      cluster_store_f4(own + at * cap + i, owner, v);
+    }
+    if (lane == 0) cluster_store(&own_cnt[at], owner, (uint32_t)tk.cnt[r]);
+  }
+  return ok;
+}
+
+// Exact threshold and filtered statistics of one row read again from global memory, by radix (see
+// exact_row_from_global): for rows whose lists cannot be used.  Valid in every thread.
+template <typename T, bool CFG>
+__device__ __noinline__ float4 slice_exact_row(const Row<T, CFG> row, const int V, int kk, const int vec_ok, SliceTopk& tk) {
+  constexpr int VEC = Elem<T>::kVec;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int* const hist = &tk.hist[0][0];
+  uint32_t prefix = 0, mask = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 24 - 8 * pass;
+    __syncthreads();
+    if (tid < 256) hist[tid] = 0;
+    __syncthreads();
+    for (int x0 = tid * VEC; x0 < V; x0 += kSliceThreads * VEC) {
+      float z[VEC];
+      row.load_tile(x0, V, vec_ok != 0, z);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        const uint32_t key = order_key(z[e]);
+        if (x0 + e < V && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int above;
+      const int bin = select_bin_from_top(hist, 256, kk, lane, &above);
+      if (lane == 0) { tk.bc_i[0] = (int)(prefix | ((uint32_t)bin << shift)); tk.bc_i[1] = kk - above; }
+    }
+    __syncthreads();
+    prefix = (uint32_t)tk.bc_i[0];
+    kk = tk.bc_i[1];
+    mask |= 255u << shift;
+  }
+  const float thr = order_value(prefix);
+  float m = CSD_NEG_INF, s = -1.0f;
+  for (int x0 = tid * VEC; x0 < V; x0 += kSliceThreads * VEC) {
+    float z[VEC];
+    row.load_tile(x0, V, vec_ok != 0, z);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) z[e] = z[e] < thr ? CSD_NEG_INF : z[e];
+    float m1, s1;
+    stat_of_values(z, m1, s1);
+    stat_merge(m, s, m1, s1);
+  }
+  stat_warp_allreduce(m, s);
+  __syncthreads();
+  if (lane == 0) tk.red[0][warp] = make_float4(m, s, 0.0f, 0.0f);
+  __syncthreads();
+  m = tk.red[0][0].x; s = tk.red[0][0].y;
+#pragma unroll 1
+  for (int w = 1; w < kSliceWarps; ++w) stat_merge(m, s, tk.red[0][w].x, tk.red[0][w].y);
+  return make_float4(m, s, thr, 0.0f);
+}
+
+// The warps of a block that settle one row together: G of them, numbered w, with a barrier of their own.
+struct RowGroup {
+  int id, G, w, lane;
+  __device__ __forceinline__ void sync() const {
+    if (G == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "r"(32 * G) : "memory");
+  }
+};
+
+// One row from its gathered values, by one group of its owner's warps.  `each(f)` calls f(value) for the lane's share
+// of them (and may be called repeatedly).  Two ways:
+// - the short cut of verify_topk_kernel: fewer than k values lie above the upper level, so the k-th largest lies
+//   between the levels, and what the filter would drop among the gathered values, at most (n_lo - k) exp(hi - m), is
+//   below 2^-26 of the normaliser: nothing that fp32 can see.  The row's (m, s) is that of everything gathered and
+//   `lo` serves as its threshold; the drafted token is dropped if k gathered values lie above its logit;
+// - the exact threshold: a histogram of the values between the levels finds the bin of the k-th largest, its rank among
+//   the bin's few values the value.
+// False if neither can be had (the lists do not hold the k largest, a crowded bin): the row is read again.  The group's
+// results are the same in all its threads.
+// (By one warp a row took 6 us with the short cut and up to 30 without, 16 K and 64 K vocabularies; by the block's warps 1 - 3.)
+template <typename Each>
+__device__ __forceinline__ bool slice_settle(SliceTopk& tk, const RowGroup& g, const int n_lo, const int k_top, const bool exact,
+                                             const float lo, float hi, const float ztok, Each each, float4& out) {
+  const int lane = g.lane;
+  int* const hist = tk.hist[g.id];
+  float* const cand = tk.cand[g.id];
+  float4* const red = tk.red[g.id];   // one per warp of the group; written between barriers
+  float m = CSD_NEG_INF;
+  each([&](const float v) { m = max_nan(m, v); });
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if (lane == 0) tk.wmax[g.id][g.w] = m;
+  for (int i = g.w * 32 + lane; i < kSliceBins; i += 32 * g.G) hist[i] = 0;
+  if (g.w == 0 && lane == 0) tk.n_cand[g.id] = 0;
+  g.sync();
+  if (lane < g.G) m = tk.wmax[g.id][lane];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if (!(n_lo >= k_top && m > lo && m < CSD_POS_INF)) return false;   // (NaN and +inf rows, constant rows, a missed guess)
+  if (!(hi > lo && hi < m)) hi = m;   // (no upper level)
+  // four sums over the group's values (all but the first are whole numbers below 2^24)
+  auto group_sum = [&](float a0, int i1, int i2, int i3) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, off);
+    i1 = __reduce_add_sync(0xffffffffu, i1);
+    i2 = __reduce_add_sync(0xffffffffu, i2);
+    i3 = __reduce_add_sync(0xffffffffu, i3);
+    if (lane == 0) red[g.w] = make_float4(a0, (float)i1, (float)i2, (float)i3);
+    g.sync();
+    float4 v = lane < g.G ? red[lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+      v.z += __shfl_xor_sync(0xffffffffu, v.z, off);
+      v.w += __shfl_xor_sync(0xffffffffu, v.w, off);
+    }
+    v.x = __shfl_sync(0xffffffffu, v.x, 0); v.y = __shfl_sync(0xffffffffu, v.y, 0);
+    v.z = __shfl_sync(0xffffffffu, v.z, 0); v.w = __shfl_sync(0xffffffffu, v.w, 0);
+    return v;
+  };
+  float acc = 0.0f;
+  int cmax = 0, above_hi = 0, rank = 0;
+  each([&](const float v) {
+    const float ev = ex2f((v - m) * kLog2e);
+    if (v == m) ++cmax; else acc += ev;
+    above_hi += (v > hi) ? 1 : 0;
+    rank += (v > ztok) ? 1 : 0;
+  });
+  const float4 all = group_sum(acc, cmax, above_hi, rank);
+  int n_hi = (int)all.z;
+  if (n_hi >= k_top) { hi = m; n_hi = 0; }   // (the upper level was a bad guess)
+  if (!exact && (float)(n_lo - k_top) * ex2f((hi - m) * kLog2e) <= 1.4901161e-8f) {
+    out = make_float4(m, all.x + (all.y - 1.0f), lo, (int)all.w >= k_top ? 1.0f : 0.0f);
+    return true;
+  }
+  int kk = k_top - n_hi;   // rank of the answer among the values in [lo, hi]
+  const float scale = (float)kSliceBins * rcp_approx(hi - lo);
+  if (!(scale < CSD_POS_INF)) return false;
+  auto bin_of = [&](const float v) { return min(kSliceBins - 1, (int)__fmul_rn(__fsub_rn(v, lo), scale)); };
+  each([&](const float v) { if (!(v > hi)) atomicAdd(&hist[bin_of(v)], 1); });
+  g.sync();
+  int above;
+  const int bin = select_bin_from_top(hist, kSliceBins, kk, lane, &above);
+  kk -= above;
+  each([&](const float v) {
+    if (!(v > hi) && bin_of(v) == bin) {
+      const int at = atomicAdd(&tk.n_cand[g.id], 1);
+      if (at < kSliceCand) cand[at] = v;
+    }
+  });
+  g.sync();
+  const int nc = tk.n_cand[g.id];
+  if (nc > kSliceCand) return false;
+  const float v0 = lane < nc ? cand[lane] : CSD_NEG_INF, v1 = lane + 32 < nc ? cand[lane + 32] : CSD_NEG_INF;
+  int gt0 = 0, ge0 = 0, gt1 = 0, ge1 = 0;
+  for (int i = 0; i < nc; ++i) {
+    const float w = cand[i];
+    gt0 += (w > v0) ? 1 : 0; ge0 += (w >= v0) ? 1 : 0;
+    gt1 += (w > v1) ? 1 : 0; ge1 += (w >= v1) ? 1 : 0;
+  }
+  const unsigned b0 = __ballot_sync(0xffffffffu, lane < nc && gt0 < kk && kk <= ge0);
+  const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < nc && gt1 < kk && kk <= ge1);
+  if ((b0 | b1) == 0u) return false;
+  const float thr = b0 ? __shfl_sync(0xffffffffu, v0, __ffs(b0) - 1) : __shfl_sync(0xffffffffu, v1, __ffs(b1) - 1);
+  acc = 0.0f;
+  cmax = 0;
+  each([&](const float v) {
+    if (v >= thr) { if (v == m) ++cmax; else acc += ex2f((v - m) * kLog2e); }
+  });
+  const float4 kept = group_sum(acc, cmax, 0, 0);   // (every warp has read the first sums before the barriers in between)
+  out = make_float4(m, kept.x + (kept.y - 1.0f), thr, 0.0f);
+  return true;
+}
+
+// The rows this block owns are settled, several at once by as many groups of warps, and their results go into every block.
+template <typename T, bool CFG>
+__device__ __forceinline__ void slice_settle_rows(const Slice<T, CFG>& k) {
+  SliceSmem& sm = k.sm;
+  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.list_off);
+  const float* const own = reinterpret_cast<const float*>(k.base + k.a.g.own_off);
+  const int* const own_cnt = reinterpret_cast<const int*>(k.base + k.a.g.stash_off);
+  const int c = k.c, R = k.R, lane = k.lane, cap = k.a.g.list_cap, k_top = k.a.f.top_k;
+  const int rows = (R - k.me + c - 1) / c;   // rows this block owns
+  int gl = 0;                                // 2^gl groups
+  while (gl < 4 && (1 << gl) < rows) ++gl;
+  RowGroup g;
+  g.G = kSliceWarps >> gl;
+  g.id = k.warp / g.G;
+  g.w = k.warp - g.id * g.G;
+  g.lane = lane;
+  for (int oi = g.id; oi < rows; oi += 1 << gl) {
+    const int r = oi * c + k.me;
+    const int nq = lane < c ? own_cnt[oi * c + lane] : 0;
+    const bool over = __any_sync(0xffffffffu, nq > cap);
+    const int n_lo = __reduce_add_sync(0xffffffffu, nq);
+    const float2 lv = tk.level[r];
+    const float* const list = own + oi * c * cap;
+    auto each = [&](auto f) {   // the lists are dealt out over the group's warps
+      for (int q = g.w; q < c; q += g.G) {
+        const int len = __shfl_sync(0xffffffffu, nq, q);
+        const float* const l = list + q * cap;
+#pragma unroll 4
+        for (int i = lane; i < len; i += 32) f(l[i]);
+      }
+    };
+    float4 v;
+    const bool done = !over && slice_settle(tk, g, n_lo, k_top, k.a.g.exact != 0, lv.x, lv.y, sm.rs.tokz[r], each, v);
+    if (g.w == 0) {
+      if (done) {
+        if (lane < c) cluster_store_f4(&tk.res[r], (uint32_t)lane, v);
+      } else if (lane == 0) {
+        atomicOr(&tk.need[r >> 5], 1u << (r & 31));
+      }
+    }
+    g.sync();   // (the group's scratch is used again)
+  }
+  __syncthreads();
+  for (int w = 0; w < kSliceRows / 32; ++w) {
+    for (unsigned bits = tk.need[w]; bits; bits &= bits - 1u) {   // (the same in every thread; nobody adds to it any more)
+      const int r = 32 * w + __ffs(bits) - 1;
+      const float4 v = slice_exact_row<T, CFG>(k.row(r), k.a.f.fin.V, k_top, k.a.g.vec_ok, tk);
+      if (k.tid < c) cluster_store_f4(&tk.res[r], (uint32_t)k.tid, v);
+    }
+  }
+  if (c > 1) { cluster_arrive(); cluster_wait(); }
+  else __syncthreads();
+  for (int r = k.tid; r < R; r += kSliceThreads) {
+    const float4 v = tk.res[r];
+    sm.rs.ms[r] = make_float2(v.x, v.y);
+    sm.rs.thr[r] = v.z;
+    if (v.w != 0.0f) sm.rs.tokz[r] = CSD_NEG_INF;   // the exact filter drops the drafted token
+  }
+}
+
 // Per tile of the slice, the sum of what `weight(xo)` returns for the lane's VEC values from element xo on.
 template <typename T, bool CFG, typename W>
 __device__ __forceinline__ void slice_tiles(const Slice<T, CFG>& k, double* tile_sums, W weight) {
@@ -554,7 +955,7 @@ __device__ __forceinline__ void slice_finish_chain(const Slice<T, CFG>& k, int s
   }
 }
 
-template <typename T, bool CFG>
+template <typename T, bool CFG, bool TOPK>
 __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const SliceArgs a) {
   extern __shared__ __align__(128) unsigned char fused_smem_raw[];
   SliceSmem& sm = *reinterpret_cast<SliceSmem*>(fused_smem_raw);
@@ -564,6 +965,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
 
   if (tid < slots) { mbar_init(&sm.full[tid], 1); sm.left[tid] = 1 << a.g.wpr_log2; sm.issued[tid] = 0; sm.cur[tid] = -1; }
   if (tid == 0) sm.abort = 0;
+  if (TOPK && tid < kSliceRows / 32) reinterpret_cast<SliceTopk*>(fused_smem_raw + a.g.list_off)->need[tid] = 0u;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
   if (c > 1) cluster_arrive();   // first half; waited for before the first store to a peer
@@ -583,15 +985,23 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
     tok = __ldcg(&f.tokens[(int64_t)k.b * L + (tid >> 1)]);
     if (tok >= 0 && tok < f.V) ztok = k.row(tid).load_one(tok);
   }
-  bool ok = slice_rows_plain<T, CFG>(k);
-  if (tid <= L) sm.fst.uni[tid] = uni;
-  if (tid < L) sm.fst.omega[tid] = omega >= 0.0f ? omega : 0.0f;
-  if (tid < 2 * L && !(tid & 1)) sm.fst.tok[tid >> 1] = tok;
-  if (tid < R) sm.rs.tokz[tid] = ztok;
+  auto late = [&]() {
+    if (tid <= L) sm.fst.uni[tid] = uni;
+    if (tid < L) sm.fst.omega[tid] = omega >= 0.0f ? omega : 0.0f;
+    if (tid < 2 * L && !(tid & 1)) sm.fst.tok[tid >> 1] = tok;
+    if (tid < R) sm.rs.tokz[tid] = ztok;   // (+inf for a token out of range: it has no rank)
+  };
+  bool ok;
+  if (TOPK) {
+    ok = slice_rows_topk<T, CFG>(k, late);
+  } else {
+    ok = slice_rows_plain<T, CFG>(k);
+    late();
+  }
   if (!ok) *(volatile int*)&sm.abort = 1;
   const int wl = a.g.wpr_log2;
   float2* const xs = reinterpret_cast<float2*>(fused_smem_raw + a.g.rec_off);   // [c][parts][R]
-  if (!a.g.direct) {   // the warps' parts of a row are merged before they go to the other blocks
+  if (!TOPK && !a.g.direct) {   // the warps' parts of a row are merged before they go to the other blocks
     __syncthreads();
     const float2* const stash = reinterpret_cast<const float2*>(fused_smem_raw + a.g.stash_off);
     for (int r0 = 2 * k.warp; r0 < R; r0 += 2 * kSliceWarps) {
@@ -612,9 +1022,11 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   if (c > 1) { cluster_arrive(); cluster_wait(); }
   else __syncthreads();
 
-  // ---- every row's statistics over the whole vocabulary ----------------------------------------------------------
+  // ---- every row's statistics over the whole vocabulary (top-k: of what the filter keeps) ----------------------------------------------------------
   const int np = a.g.direct ? c << wl : c;   // parts of a row, at most 32
-  if (np <= 16) {
+  if (TOPK) {
+    slice_settle_rows<T, CFG>(k);
+  } else if (np <= 16) {
     for (int r0 = 2 * k.warp; r0 < R; r0 += 2 * kSliceWarps) {
       const int r = r0 + (lane >> 4), q = lane & 15;
       const float2 v = merge_parts((q < np && r < R) ? xs[q * R + r] : make_float2(CSD_NEG_INF, -1.0f), lane, 16);
@@ -630,7 +1042,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   for (int q = 0; q < c; ++q) status_any |= sm.xflag[q] ? 8 : 0;
   if (a.f.error_flag && __ldcg(a.f.error_flag)) status_any |= 8;
   __syncthreads();
-  slice_finish_chain<T, CFG, false>(k, status_any);
+  slice_finish_chain<T, CFG, TOPK>(k, status_any);
 }
 
 }  // namespace csd

@@ -78,3 +78,40 @@ def test_drafting_draws(R, V):
     want = (cdf <= (u.double() * cdf[:, -1])[:, None]).sum(-1).cpu().numpy()
     for out in outs:
         assert (out != want).sum() <= 1
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=4, gamma=8, V=16384, dtype=W.BF16, cfg=True, cfg_scale=4.0, top_k=1000, bonus_row=True),   # the short cut
+    dict(B=4, gamma=8, V=16384, dtype=W.BF16, top_k=1000, bonus_row=True),       # exact thresholds, duplicates
+    dict(B=14, gamma=8, V=16384, dtype=W.F32, top_k=1000),                       # eight blocks, two rows to a block
+    dict(B=2, gamma=16, V=8192, dtype=W.F32, top_k=3),                           # no upper level
+    dict(B=2, gamma=16, V=8192, dtype=W.F32, top_k=1), dict(B=2, gamma=9, V=8192, top_k=2500),
+    dict(B=1, gamma=32, V=16384, dtype=W.BF16, top_k=200, bonus_row=True),       # 65 rows: five to a block
+    dict(B=2, gamma=8, V=65536, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=2000, bonus_row=True),   # rows in turns
+    dict(B=3, gamma=8, V=16384, dtype=W.BF16, law="student3", rho=0.85, top_k=500),
+    dict(B=3, gamma=8, V=16387, dtype=W.BF16, top_k=500, bonus_row=True), dict(B=3, gamma=8, V=16387, dtype=W.F32, cfg=True, top_k=40),
+])
+@pytest.mark.parametrize("want_dbg", [False, True])
+def test_topk_slices(kw, want_dbg):
+    """want_dbg asks for the distribution drawn from: every row then gets its exact threshold."""
+    rep, _, _ = check(_make(kw), want_dbg=want_dbg)
+    assert rep.ok and rep.tau_mismatch_near + rep.token_mismatch_near <= 1, rep.summary()
+
+
+@pytest.mark.parametrize("kind", ["masked", "ties", "two_levels", "nan"])
+def test_topk_slices_on_rows_the_guess_misses(kind):
+    """Rows whose lists cannot be used (the guess is far off, a crowded histogram bin, NaN) are read again."""
+    w = _make(dict(B=3, gamma=8, V=16384, dtype=W.F32, top_k=300, bonus_row=True))
+    for t in (w.target_logits, w.draft_logits):
+        keep = torch.zeros(t.shape[-1], dtype=torch.bool, device=DEV)
+        keep[::7] = True
+        if kind == "masked":
+            t[:, ::2, ~keep] = float("-inf")
+        elif kind == "ties":
+            t.copy_((t * 2).round() / 2)
+        elif kind == "two_levels":
+            t[:, 1::2, ~keep] -= 200.0
+        else:
+            t[1, 2, 777] = float("nan")
+    rep, _, _ = check(w)
+    assert rep.ok, rep.summary()
