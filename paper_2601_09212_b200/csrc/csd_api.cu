@@ -2,7 +2,6 @@
 // Every step of the method runs in the kernels of csd_kernels.cuh; nothing here
 // touches logits.
 #include <cuda_runtime.h>
-#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -312,12 +311,15 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
 }
 
 // Launches the sliced kernel if it suits the call; *launched says whether it did (with `dry`, whether it would).
-// The split is the one with the fewest logits for the busiest SM to go through; where rows are aligned it has to leave
-// at most three quarters of what `other_work` says that the position split would give it.  That is where the lines lie
-// (us per call, sliced / position split): 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3 (0.71 of the
-// work), B=16 17.6 / 15.2 (1.4); guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; 64 K bf16 B=4 18.0 / 23.2 (0.35), fp32 gamma=16 B=1 31.9 / 41.5 (0.41), B=8 48 / 42 (0.83).
+// The split is the one with the least expected time, which where rows are aligned has to be below `other_ns`, what the
+// position split should take.  Expected times are a fixed part for each wave of clusters and a rate over the logits that
+// the busiest SM goes through, fitted to (us per call, sliced / position split):
+//   no top-k: 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3, B=16 17.6 / 15.2; 64 K bf16 B=4 18.0 / 23.2, fp32
+//   gamma=16 B=1 31.9 / 41.5, B=8 48 / 42; drafting calls of 64 guided rows of 16 K 8.7 / 11.5, 25 of 23 K 8.3 / 13.3;
+//   top-k: guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; drafting calls of 64
+//   rows of 16 K 15.1 / 13.6, 20 of 30 K 13.9 / 20.5; guided 33 K top-k 1823 gamma=13 B=8 (five turns) 73.7 / 63.6.
 template <typename T, bool CFG, bool TOPK>
-cudaError_t try_slice(SliceArgs& a, long long other_work, double tail, bool dry, cudaStream_t stream, bool* launched) {
+cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cudaStream_t stream, bool* launched) {
   constexpr int TILE = 32 * Elem<T>::kVec;
   static std::atomic<int> known[kMaxDevices][5][2];
   auto kern = verify_slice_kernel<T, CFG, TOPK>;
@@ -327,27 +329,33 @@ cudaError_t try_slice(SliceArgs& a, long long other_work, double tail, bool dry,
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (R > kSliceRows) return cudaSuccess;
-  long long best = a.g.vec_ok ? other_work * 3 / 4 + 1 : LLONG_MAX;
+  double best = a.g.vec_ok ? other_ns : 1e30;
   SliceGeo geo;
   size_t bytes = 0;
   int best_c = 0;
   for (int log2c = 4; log2c >= 0; --log2c) {
     const int c = 1 << log2c;
     if (c > ntiles || (c > 1 && f.V / c < kSliceUnit)) continue;
-    const long long n = (long long)((ntiles + c - 1) / c) * TILE;
-    if (n * R >= best) continue;
+    const double logits = (double)((ntiles + c - 1) / c) * TILE * R;   // a block's
+    auto expect = [&](int waves, double per_sm) { return TOPK ? 14e3 * waves + 0.30 * per_sm : 7e3 * waves + 0.15 * per_sm; };
+    if (expect(1, logits) >= best) continue;
     // a block to an SM where the clusters fit so, with room for more rows at once; else two
     const int cap1 = slice_capacity(kern, known, dev, log2c, 1), cap2 = slice_capacity(kern, known, dev, log2c, 0);
     if (cap1 <= 0 || cap2 <= 0) continue;
-    const long long work = n * R * (f.B <= cap1 ? 1 : 2LL * ((f.B + cap2 - 1) / cap2));
-    if (best_c == 0 ? work >= best : work * 8 >= best * 7) continue;   // (more blocks if it is nearly as good: 24 unaligned
-                                                                       // sequences, bf16: eight blocks 24.4, four 26.8)
+    const int waves = (f.B + cap2 - 1) / cap2;
+    double ns = expect(waves, f.B <= cap1 ? logits : 2.0 * waves * logits);
+    // (more blocks if that is nearly as good: 24 unaligned sequences, bf16: eight blocks each 23.1 us, four 25.9)
+    if (best_c == 0 ? ns >= best : ns * 8 >= best * 7) continue;
     SliceGeo g;
     size_t need;
     bool fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[0], tail, g, need);
     if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[1], tail, g, need);
     if (!fits) continue;
-    best = work;
+    if (TOPK) {   // rows that do not fit at once go in turns, each with an exchange of moments
+      ns += 6e3 * waves * ((R - 1) / g.slots);
+      if (ns >= best) continue;
+    }
+    best = ns;
     best_c = c;
     geo = g;
     bytes = need;
@@ -374,18 +382,16 @@ struct SliceCall {
 };
 cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool* launched) {
   *launched = false;
-  // The position split's work for its busiest SM (see plan_and_launch_fused).  Once it fills the GPU it streams better
-  // than slices do (fp32 B=32: 16.9 us, sliced 21.1).
+  // What the position split should take, from its busiest block (see plan_and_launch_fused).  Once it fills the GPU it
+  // streams better than slices do (fp32 B=32: 16.9 us, sliced 21.1).
   const int B = in.fa.B, gamma = in.fa.gamma;
   int pos = 1;
   const int split_below = (in.topk ? 4 : 2) * in.sms;
   while (2 * pos <= split_below / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
   if (in.fa.vec_ok && (long long)B * pos > in.sms) return cudaSuccess;
-  const long long rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
-  const long long other_work = rows * in.fa.V;
-  // (with top-k the two exchanges before the accept tests want something to save: a row of 16 K a block, the drafting
-  // stage's, takes 13.6 us whole and 15.1 sliced; three rows 23.6 and 18.0)
-  if (in.topk && in.fa.vec_ok && other_work < 24 * 1024) return cudaSuccess;
+  const int rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
+  const double logits = (double)rows * in.fa.V;
+  const double other_ns = in.topk ? 5e3 + 0.39 * logits : 9e3 + 0.09 * logits;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;
@@ -403,7 +409,7 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
     a.f.lo_sigmas = guess.lo_sigmas;
     a.f.hi_delta = guess.hi_delta;
   }
-#define CSD_SLICE(T, CFG, TOPK) try_slice<T, CFG, TOPK>(a, other_work, guess.tail, dry, stream, launched)
+#define CSD_SLICE(T, CFG, TOPK) try_slice<T, CFG, TOPK>(a, other_ns, guess.tail, dry, stream, launched)
   if (in.dtype == CSD_F32) {
     if (in.cfg) return in.topk ? CSD_SLICE(float, true, true) : CSD_SLICE(float, true, false);
     return in.topk ? CSD_SLICE(float, false, true) : CSD_SLICE(float, false, false);
