@@ -256,57 +256,84 @@ void slice_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int g
   cfg.numAttrs = 2;
 }
 
-// Sequences in clusters of 2^log2c blocks that the GPU holds at once, for each of the two shared-memory sizes; asked
+// Sequences in clusters of c blocks that the GPU holds at once, for each of the two shared-memory sizes; asked
 // once per kernel and device.
 template <typename K>
-int slice_capacity(K kern, std::atomic<int> (&known)[kMaxDevices][5][2], int dev, int log2c, int cls) {
-  int k = known[dev][log2c][cls].load(std::memory_order_acquire);   // 0: not asked yet; -1: none
+int slice_capacity(K kern, std::atomic<int> (&known)[kMaxDevices][kSliceCluster + 1][2], int dev, int c, int cls) {
+  int k = known[dev][c][cls].load(std::memory_order_acquire);   // 0: not asked yet; -1: none
   if (k == 0) {
     int clusters = 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    slice_config(cfg, attr, 1 << log2c, 1 << log2c, kSliceSmem[cls], 0);
+    slice_config(cfg, attr, c, c, kSliceSmem[cls], 0);
     cfg.numAttrs = 1;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceSmem[1]);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
     if (e != cudaSuccess) { (void)cudaGetLastError(); clusters = 0; }
     k = clusters > 0 ? clusters : -1;
-    known[dev][log2c][cls].store(k, std::memory_order_release);
+    known[dev][c][cls].store(k, std::memory_order_release);
   }
   return k;
 }
 
+// Into how many parts a row's slice of `upr` units is cut so that the busiest of the block's warps has the least to do (a
+// part costs its units and about a third of one); returns that warp's units.
+int slice_rounds(int R, int upr, int& parts, int& upp) {
+  double best = 0.0;
+  int units = 0;
+  for (int np = 1; np <= 16 && np <= upr; ++np) {
+    const int per = (upr + np - 1) / np, n = (upr + per - 1) / per;
+    if (n != np) continue;   // (the same cut as a smaller np)
+    const int turns = (R * n + kSliceWarps - 1) / kSliceWarps;
+    const double load = turns * (per + 0.33);
+    if (units == 0 || load < best) { best = load; units = turns * per; parts = n; upp = per; }
+  }
+  return units;
+}
+
 // Shared-memory layout of a call split over c blocks; false if it does not fit `room` bytes.
 // `tail`: the share of a row that the top-k lists expect.
-template <typename T, bool CFG, bool TOPK>
+template <typename T, bool CFG, bool TOPK, bool TREE>
 bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, SliceGeo& g, size_t& bytes) {
   constexpr int ES = (int)sizeof(T), ARR = CFG ? 2 : 1, TILE = 32 * Elem<T>::kVec;
   const int ntiles = (a.f.fin.V + TILE - 1) / TILE;
   const int tiles = (ntiles + c - 1) / c, n = tiles * TILE, upr = (n + kSliceUnit - 1) / kSliceUnit;
   g = a.g;
   g.slot_bytes = (n * ES + (g.vec_ok ? 0 : 16)) * ARR;
-  g.wpr_log2 = 0;
-  while (g.wpr_log2 < 4 && (1 << g.wpr_log2) < upr) ++g.wpr_log2;
-  g.direct = (c << g.wpr_log2) <= 32 ? 1 : 0;
+  slice_rounds(R, upr, g.parts, g.upp);
+  g.direct = c * g.parts <= 32 ? 1 : 0;
   size_t off = kSliceHeader;
   auto take = [&](size_t want) { const size_t o = off; off += (want + 127) / 128 * 128; return (int)o; };
   const size_t owned = (size_t)(R + c - 1) / c;   // top-k: rows whose lists a block receives
-  g.rec_off = take((size_t)R * (TOPK ? (size_t)c * sizeof(float4) : (size_t)(g.direct ? c << g.wpr_log2 : c) * sizeof(float2)));
+  g.rec_off = take((size_t)R * (TOPK ? (size_t)c * sizeof(float4) : (size_t)(g.direct ? c * g.parts : c) * sizeof(float2)));
   g.tile_off = take((size_t)tiles * sizeof(double));
-  g.stash_off = take(TOPK ? owned * c * sizeof(int) : (g.direct ? 0 : ((size_t)R << g.wpr_log2) * sizeof(float2)));
+  g.stash_off = take(TOPK ? owned * c * sizeof(int) : (g.direct ? 0 : (size_t)R * g.parts * sizeof(float2)));
+  g.tree_off = take(TREE ? sizeof(SliceTree) : 0);
+  const size_t tables = TREE ? 2 * (size_t)(n + 4) * sizeof(float) : 0;
+  const size_t scratch = TOPK ? sizeof(SliceSettle) : 0;
   if (TOPK) {
     const double e = tail * n;   // values a slice's list expects
     g.list_cap = ((int)(1.25 * e + 6.0 * sqrt(e) + 24.0) + 3) / 4 * 4;
     if (g.list_cap > n) g.list_cap = n;
-    g.list_off = take(sizeof(SliceTopk) + (size_t)R * g.list_cap * sizeof(float));
-    g.own_off = take(owned * c * g.list_cap * sizeof(float));
+    g.topk_off = take(sizeof(SliceTopk));
+    const size_t lists = owned * c * g.list_cap * sizeof(float);
+    g.own_off = take(lists > tables ? lists : tables);
+    g.tab_off = g.own_off;   // (a tree's walk begins when the lists are done with)
+  } else {
+    g.tab_off = take(tables);
   }
-  g.arena_off = (int)off;
-  if (off >= room) return false;
-  const size_t slots = (room - off) / g.slot_bytes;
-  g.slots = slots > (size_t)R ? R : (int)slots;
-  bytes = off + (size_t)g.slots * g.slot_bytes;
+  // slots, and with top-k a list for each (in whose place rows are settled later)
+  for (g.slots = R; g.slots > 0; --g.slots) {
+    size_t region = (size_t)g.slots * g.list_cap * sizeof(float);
+    if (TOPK && region < scratch) region = scratch;
+    region = (region + 127) / 128 * 128;
+    bytes = off + region + (size_t)g.slots * g.slot_bytes;
+    if (bytes > room) continue;
+    g.list_off = (int)off;
+    g.arena_off = (int)(off + region);
+    break;
+  }
   return g.slots >= (R < 4 ? R : 4);
 }
 
@@ -318,11 +345,11 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
 //   gamma=16 B=1 31.9 / 41.5, B=8 48 / 42; drafting calls of 64 guided rows of 16 K 8.7 / 11.5, 25 of 23 K 8.3 / 13.3;
 //   top-k: guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; drafting calls of 64
 //   rows of 16 K 15.1 / 13.6, 20 of 30 K 13.9 / 20.5; guided 33 K top-k 1823 gamma=13 B=8 (five turns) 73.7 / 63.6.
-template <typename T, bool CFG, bool TOPK>
+template <typename T, bool CFG, bool TOPK, bool TREE>
 cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cudaStream_t stream, bool* launched) {
   constexpr int TILE = 32 * Elem<T>::kVec;
-  static std::atomic<int> known[kMaxDevices][5][2];
-  auto kern = verify_slice_kernel<T, CFG, TOPK>;
+  static std::atomic<int> known[kMaxDevices][kSliceCluster + 1][2];
+  auto kern = verify_slice_kernel<T, CFG, TOPK, TREE>;
   const FinishArgs& f = a.f.fin;
   const int R = f.T + f.gamma, ntiles = (f.V + TILE - 1) / TILE;
   *launched = false;
@@ -333,26 +360,28 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
   SliceGeo geo;
   size_t bytes = 0;
   int best_c = 0;
-  for (int log2c = 4; log2c >= 0; --log2c) {
-    const int c = 1 << log2c;
+  for (int c = kSliceCluster; c >= 1; --c) {
     if (c > ntiles || (c > 1 && f.V / c < kSliceUnit)) continue;
-    const double logits = (double)((ntiles + c - 1) / c) * TILE * R;   // a block's
-    auto expect = [&](int waves, double per_sm) { return TOPK ? 14e3 * waves + 0.30 * per_sm : 7e3 * waves + 0.15 * per_sm; };
+    int np, upp;   // the work of a block: its busiest warp's, times its warps
+    const double logits = (double)slice_rounds(R, (((ntiles + c - 1) / c) * TILE + kSliceUnit - 1) / kSliceUnit, np, upp) * kSliceUnit * kSliceWarps;
+    auto expect = [&](int waves, double per_sm) {
+      return waves * ((TOPK ? 11e3 : 7e3) + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
+    };
     if (expect(1, logits) >= best) continue;
     // a block to an SM where the clusters fit so, with room for more rows at once; else two
-    const int cap1 = slice_capacity(kern, known, dev, log2c, 1), cap2 = slice_capacity(kern, known, dev, log2c, 0);
+    const int cap1 = slice_capacity(kern, known, dev, c, 1), cap2 = slice_capacity(kern, known, dev, c, 0);
     if (cap1 <= 0 || cap2 <= 0) continue;
     const int waves = (f.B + cap2 - 1) / cap2;
-    double ns = expect(waves, f.B <= cap1 ? logits : 2.0 * waves * logits);
+    double ns = expect(waves, f.B <= cap1 ? logits : 1.7 * waves * logits);
     // (more blocks if that is nearly as good: 24 unaligned sequences, bf16: eight blocks each 23.1 us, four 25.9)
     if (best_c == 0 ? ns >= best : ns * 8 >= best * 7) continue;
     SliceGeo g;
     size_t need;
-    bool fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[0], tail, g, need);
-    if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG, TOPK>(a, R, c, kSliceSmem[1], tail, g, need);
+    bool fits = slice_layout<T, CFG, TOPK, TREE>(a, R, c, kSliceSmem[0], tail, g, need);
+    if (f.B <= cap1 && (!fits || g.slots < R)) fits = slice_layout<T, CFG, TOPK, TREE>(a, R, c, kSliceSmem[1], tail, g, need);
     if (!fits) continue;
     if (TOPK) {   // rows that do not fit at once go in turns, each with an exchange of moments
-      ns += 6e3 * waves * ((R - 1) / g.slots);
+      ns += 5e3 * waves * ((R - 1) / g.slots);
       if (ns >= best) continue;
     }
     best = ns;
@@ -379,19 +408,25 @@ struct SliceCall {
   bool cfg, topk, exact;   // exact: every row's exact threshold is wanted
   int* error_flag;
   int sms;
+  int N = 0, D = 0;        // N > 0: a tree (fa: gamma = T = N + 1 contexts)
+  int32_t* out_nodes = nullptr;
+  const int32_t* parent = nullptr;
 };
 cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool* launched) {
   *launched = false;
   // What the position split should take, from its busiest block (see plan_and_launch_fused).  Once it fills the GPU it
   // streams better than slices do (fp32 B=32: 16.9 us, sliced 21.1).
   const int B = in.fa.B, gamma = in.fa.gamma;
+  const bool tree = in.N > 0;
   int pos = 1;
   const int split_below = (in.topk ? 4 : 2) * in.sms;
   while (2 * pos <= split_below / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
-  if (in.fa.vec_ok && (long long)B * pos > in.sms) return cudaSuccess;
+  if (in.fa.vec_ok && !tree && (long long)B * pos > in.sms) return cudaSuccess;
   const int rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
   const double logits = (double)rows * in.fa.V;
-  const double other_ns = in.topk ? 5e3 + 0.39 * logits : 9e3 + 0.09 * logits;
+  // (a tree: the statistics of all rows, then the walk by one block per sequence)
+  const double other_ns = tree ? ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms)
+                          : in.topk ? 5e3 + 0.39 * logits : 9e3 + 0.09 * logits;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;
@@ -409,7 +444,12 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
     a.f.lo_sigmas = guess.lo_sigmas;
     a.f.hi_delta = guess.hi_delta;
   }
-#define CSD_SLICE(T, CFG, TOPK) try_slice<T, CFG, TOPK>(a, other_ns, guess.tail, dry, stream, launched)
+  a.N = in.N; a.D = in.D;
+  a.out_nodes = in.out_nodes;
+  for (int n = 0; n < in.N; ++n) a.parent[n] = (signed char)in.parent[n];
+#define CSD_SLICE(T, CFG, TOPK) \
+  (tree ? try_slice<T, CFG, TOPK, true>(a, other_ns, guess.tail, dry, stream, launched) \
+        : try_slice<T, CFG, TOPK, false>(a, other_ns, guess.tail, dry, stream, launched))
   if (in.dtype == CSD_F32) {
     if (in.cfg) return in.topk ? CSD_SLICE(float, true, true) : CSD_SLICE(float, true, false);
     return in.topk ? CSD_SLICE(float, false, true) : CSD_SLICE(float, false, false);
@@ -943,6 +983,20 @@ int csd_verify_tree(const csd_tree_params* pp) {
   for (int n = 0; n < p.N; ++n) ta.parent[n] = (signed char)p.parent[n];
 
   cudaError_t e = cudaSuccess;
+  if (p.V >= 512) {   // the walk shared by a cluster of blocks
+    SliceCall sc;
+    sc.fa = fa;
+    sc.dtype = p.dtype; sc.top_k = p.top_k; sc.cfg = cfg; sc.topk = topk;
+    sc.exact = true;   // a residual after several rejections has little mass left: the filter is taken exactly
+    sc.sms = sms;
+    sc.error_flag = reinterpret_cast<int*>(ws + lay.header_off);
+    sc.N = p.N; sc.D = D;
+    sc.out_nodes = p.out_nodes;
+    sc.parent = p.parent;
+    bool sliced = false;
+    e = slice_call(sc, false, stream, &sliced);
+    if (sliced || e != cudaSuccess) return e == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+  }
   // Row statistics (and thresholds) of all 2 C rows: by the streaming kernels of the single-launch path
   // where the rows qualify for them (aligned, at least 512 bytes, within the draw's tile table), one
   // launch that reads every logit once; otherwise by the select and statistics kernels.

@@ -1,4 +1,4 @@
-// Calls in stream order with few sequences or unaligned rows (sm_100a): a sequence's rows are split over the
+// Calls in stream order with few sequences or unaligned rows, and draft trees (sm_100a): a sequence's rows are split over the
 // VOCABULARY, one slice of every row per block, and the blocks of a sequence form one thread-block cluster of up to 16.
 //
 // Such a call is bound by latency, not by bandwidth.  The position split of csd_fused.cuh gives a block two rows
@@ -16,13 +16,14 @@
 //      block; one cluster barrier later the block whose slice holds the crossing C(x) > u Z picks the token and emits.
 #pragma once
 #include "csd_fused.cuh"
+#include "csd_tree.cuh"
 
 namespace csd {
 
 constexpr int kSliceThreads = 512;      // two blocks per SM
 constexpr int kSliceWarps = kSliceThreads / 32;
 constexpr int kSliceCluster = 16;       // blocks of a sequence (above 8: a non-portable cluster size)
-constexpr int kSliceRows = 128;
+constexpr int kSliceRows = 2 * (kMaxTreeNodes + 1);
 constexpr int kSliceUnit = 512;         // logits of a warp's unit of work: 16 per lane
 constexpr int kSliceSample = 4096;      // top-k: logits of a row that the moments are taken from, over all blocks
 constexpr int kSliceBins = 128;         // per row being settled: histogram of the values between the two levels
@@ -33,21 +34,32 @@ static_assert(kSliceRows <= kBlockRows, "a block's row results live in RowStats"
 struct SliceGeo {
   int slots, slot_bytes;   // rows whose slices the block holds at once; bytes of one (all arrays)
   int vec_ok;              // rows are whole 16-byte vectors at 16-byte aligned addresses
-  int wpr_log2;            // 2^this warps work on a row at once
+  int parts, upp;          // a row's slice is dealt out to the warps in this many parts, of this many units each
   int direct;              // the warps' parts of a row go to the other blocks as they are (else merged first)
   int list_cap;            // top-k: values a row's list holds
   int exact;               // top-k: every row's exact threshold is wanted
   // dynamic shared memory after SliceSmem: offsets in bytes
-  int rec_off, stash_off, tile_off, list_off, own_off, arena_off;
+  int rec_off, stash_off, tile_off, tree_off, topk_off, list_off, own_off, tab_off, arena_off;
 };
 struct SliceArgs {
   FusedArgs f;
   SliceGeo g;
+  int N, D;                // a tree: nodes, levels (f.fin: gamma = T = N + 1 contexts)
+  int32_t* out_nodes;
+  signed char parent[kMaxTreeNodes + 1];
+};
+// ... and a tree's small inputs, in shared memory, with what its walk keeps
+struct SliceTree {
+  float inv_z[kMaxSiblings];   // 1 / Z_k of the rejections so far in the current context
+  int keep[kMaxSiblings];      // the k-th update found an empty positive part and kept the residual
+  int path_tok[kMaxTreeDepth + 1], path_node[kMaxTreeDepth];
+  int tok[kMaxTreeNodes];
+  float tokz[2][kMaxTreeNodes], uni[kMaxTreeNodes], omega[kMaxTreeDepth], u;
 };
 
 struct SliceSmem {
   alignas(8) uint64_t full[kSliceRows];
-  int left[kSliceRows];      // warps that have yet to read the slot's row
+  int left[kSliceRows];      // parts of the slot's row not yet read
   int issued[kSliceRows];    // rows announced to the slot's barrier so far
   int cur[kSliceRows];       // the latest of them
   uint32_t xflag[kSliceCluster];        // a bounded wait gave up in that block
@@ -57,18 +69,21 @@ struct SliceSmem {
   FinishSmem fin;
   FinishStage fst;
 };
-// ... and what top-k needs beside it (at list_off's head)
+// ... and what top-k needs beside it (at topk_off)
 struct SliceTopk {
   alignas(16) float4 res[kSliceRows];   // (m, s, threshold, 1: the filter drops the drafted token), from the row's owner
   float2 level[kSliceRows];  // (lo, hi)
   int cnt[kSliceRows];       // length of the row's list (may run past its capacity)
   unsigned need[kSliceRows / 32];       // rows of this block to be read again
-  float4 red[kSliceWarps][kSliceWarps];
+};
+// Scratch of the rows being settled (in the lists' place: those have been sent by then).
+struct SliceSettle {
+  alignas(16) float4 red[kSliceWarps][kSliceWarps];
   float wmax[kSliceWarps][kSliceWarps];
   int hist[kSliceWarps][kSliceBins];    // (rows read again use it as one)
   float cand[kSliceWarps][kSliceCand];
   int n_cand[kSliceWarps];
-  alignas(16) int bc_i[2];
+  int bc_i[2];
 };
 constexpr int kSliceHeader = (int)((sizeof(SliceSmem) + 127) / 128 * 128);
 
@@ -182,7 +197,7 @@ struct Slice {
     __syncwarp();
     return mbar_wait(&sm.full[s], (uint32_t)(r / a.g.slots) & 1u, a.f.wait_limit);
   }
-  // This warp has read its units of row r: the row's last reader hands the slot to the row that follows in it.
+  // This warp has read its part of row r: the row's last reader hands the slot to the row that follows in it.
   __device__ __forceinline__ void release_row(const int r, const bool ok) const {
     if (a.g.slots >= R) return;
     __syncwarp();
@@ -191,7 +206,7 @@ struct Slice {
       if (!ok) *(volatile int*)&sm.abort = 1;
       __threadfence_block();
       if (atom_add_shared(&sm.left[s], -1) == 1) {
-        sm.left[s] = 1 << a.g.wpr_log2;
+        sm.left[s] = a.g.parts;
         __threadfence_block();
         if (r + a.g.slots < R && *(volatile int*)&sm.abort == 0) {
           fence_before_bulk();
@@ -390,15 +405,17 @@ __device__ __forceinline__ float2 merge_parts(const float2 v, const int lane, co
 template <typename T, bool CFG>
 __device__ __forceinline__ bool slice_rows_plain(const Slice<T, CFG>& k) {
   float2* const parts = reinterpret_cast<float2*>(k.base + (k.a.g.direct ? k.a.g.rec_off : k.a.g.stash_off));
-  const int wl = k.a.g.wpr_log2, part = k.warp & ((1 << wl) - 1), R = k.R;
+  const int R = k.R, np = k.a.g.parts, upp = k.a.g.upp;
   bool ok = true, peers = k.c == 1;
-  for (int r = k.warp >> wl; r < R; r += kSliceWarps >> wl) {
+  int r = k.warp / np, part = k.warp - r * np;
+  while (r < R) {
     if (ok && !k.wait_row(r)) ok = false;
     const unsigned char *p, *pu;
     k.slice_at(r, p, pu);
     UnitStats st;
     st.begin();
-    for (int u = part; u < k.upr; u += 1 << wl) {
+    const int u1 = min(k.upr, (part + 1) * upp);
+    for (int u = part * upp; u < u1; ++u) {
       float z[16];
       k.unit(p, pu, u, z);
       st.add(z);
@@ -407,10 +424,12 @@ __device__ __forceinline__ bool slice_rows_plain(const Slice<T, CFG>& k) {
     const float2 v = st.end();
     if (k.a.g.direct) {   // into every block
       if (!peers) { cluster_wait(); peers = true; }   // every peer is running
-      if (k.lane < k.c) cluster_store_f2(&parts[((k.me << wl) + part) * R + r], (uint32_t)k.lane, v);
+      if (k.lane < k.c) cluster_store_f2(&parts[(k.me * np + part) * R + r], (uint32_t)k.lane, v);
     } else if (k.lane == 0) {
-      parts[(r << wl) + part] = v;
+      parts[r * np + part] = v;
     }
+    part += kSliceWarps;
+    while (part >= np) { part -= np; ++r; }
   }
   if (!peers) cluster_wait();
   return ok;
@@ -423,12 +442,14 @@ __device__ __forceinline__ bool slice_rows_plain(const Slice<T, CFG>& k) {
 // drafted tokens' logits into shared memory.
 template <typename T, bool CFG, typename Late>
 __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late late) {
-  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.list_off);
+  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.topk_off);
   const FusedArgs& a = k.a.f;
   const int slots = k.a.g.slots, R = k.R, cap = k.a.g.list_cap, lane = k.lane, c = k.c;
-  const int wl = k.a.g.wpr_log2, part = k.warp & ((1 << wl) - 1);
+  const int np = k.a.g.parts, upp = k.a.g.upp;
   float4* const mom = reinterpret_cast<float4*>(k.base + k.a.g.rec_off);   // [c][R]: sum, sum of |deviations|, values
-  float* const lists = reinterpret_cast<float*>(k.base + k.a.g.list_off + sizeof(SliceTopk));
+  float* const lists = reinterpret_cast<float*>(k.base + k.a.g.list_off);   // of the group's rows
+  float* const own = reinterpret_cast<float*>(k.base + k.a.g.own_off);     // [rows owned][c][cap]
+  int* const own_cnt = reinterpret_cast<int*>(k.base + k.a.g.stash_off);   // [rows owned][c]
   const int groups = (R + slots - 1) / slots, G = (R + groups - 1) / groups;
   const uint32_t lanemask_lt = (1u << lane) - 1u;
   // units of a row's slice in the sample: one warp takes them one after the other
@@ -500,14 +521,16 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
     }
     __syncthreads();
     // ---- gather (by the sign of z - lo, so that a NaN lands in the list; see verify_topk_kernel) -------------------
-    for (int r = g0 + (k.warp >> wl); r < g1; r += kSliceWarps >> wl) {
+    int r = g0 + k.warp / np, part = k.warp % np;
+    while (r < g1) {
       if (ok && !k.wait_row(r)) ok = false;
       const unsigned char *p, *pu;
       k.slice_at(r, p, pu);
       const float lo = tk.level[r].x;
       const uint64_t nlo2 = pack2(-lo, -lo);
-      const uint32_t list = smem_addr(lists + r * cap);
-      for (int u = part; u < k.upr; u += 1 << wl) {
+      const uint32_t list = smem_addr(lists + (r - g0) * cap);
+      const int u1 = min(k.upr, (part + 1) * upp);
+      for (int u = part * upp; u < u1; ++u) {
         float z[16];
         k.unit(p, pu, u, z);
         uint32_t below_lo = 0;
@@ -542,21 +565,19 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
         }
       }
       k.release_row(r, ok);
+      part += kSliceWarps;
+      while (part >= np) { part -= np; ++r; }
     }
-  }
-  late();
-  __syncthreads();
-  // ---- the lists go to the rows' owners: row r to block r % c --------------------------------------------------------
-  float* const own = reinterpret_cast<float*>(k.base + k.a.g.own_off);   // [rows owned][c][cap]
-  int* const own_cnt = reinterpret_cast<int*>(k.base + k.a.g.stash_off); // [rows owned][c]
-  for (int r = k.warp; r < R; r += kSliceWarps) {
-    const int len = min(tk.cnt[r], cap), oi = r / c, at = oi * c + k.me;
-    const uint32_t owner = (uint32_t)(r - oi * c);
-    for (int i = 4 * lane; i < len; i += 128) {
-      const float4 v = *reinterpret_cast<const float4*>(lists + r * cap + i);
-      cluster_store_f4(own + at * cap + i, owner, v);
+    // ---- the lists go to the rows' owners: row r to block r % c ------------------------------------------------------
+    if (g1 == R) late();
+    __syncthreads();
+    for (r = g0 + k.warp; r < g1; r += kSliceWarps) {
+      const int len = min(tk.cnt[r], cap), oi = r / c, at = oi * c + k.me;
+      const uint32_t owner = (uint32_t)(r - oi * c);
+      for (int i = 4 * lane; i < len; i += 128)
+        cluster_store_f4(own + at * cap + i, owner, *reinterpret_cast<const float4*>(lists + (r - g0) * cap + i));
+      if (lane == 0) cluster_store(&own_cnt[at], owner, (uint32_t)tk.cnt[r]);
     }
-    if (lane == 0) cluster_store(&own_cnt[at], owner, (uint32_t)tk.cnt[r]);
   }
   return ok;
 }
@@ -564,7 +585,7 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
 // Exact threshold and filtered statistics of one row read again from global memory, by radix (see
 // exact_row_from_global): for rows whose lists cannot be used.  Valid in every thread.
 template <typename T, bool CFG>
-__device__ __noinline__ float4 slice_exact_row(const Row<T, CFG> row, const int V, int kk, const int vec_ok, SliceTopk& tk) {
+__device__ __noinline__ float4 slice_exact_row(const Row<T, CFG> row, const int V, int kk, const int vec_ok, SliceSettle& tk) {
   constexpr int VEC = Elem<T>::kVec;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int* const hist = &tk.hist[0][0];
@@ -637,7 +658,7 @@ struct RowGroup {
 // results are the same in all its threads.
 // (By one warp a row took 6 us with the short cut and up to 30 without, 16 K and 64 K vocabularies; by the block's warps 1 - 3.)
 template <typename Each>
-__device__ __forceinline__ bool slice_settle(SliceTopk& tk, const RowGroup& g, const int n_lo, const int k_top, const bool exact,
+__device__ __forceinline__ bool slice_settle(SliceSettle& tk, const RowGroup& g, const int n_lo, const int k_top, const bool exact,
                                              const float lo, float hi, const float ztok, Each each, float4& out) {
   const int lane = g.lane;
   int* const hist = tk.hist[g.id];
@@ -735,7 +756,8 @@ __device__ __forceinline__ bool slice_settle(SliceTopk& tk, const RowGroup& g, c
 template <typename T, bool CFG>
 __device__ __forceinline__ void slice_settle_rows(const Slice<T, CFG>& k) {
   SliceSmem& sm = k.sm;
-  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.list_off);
+  SliceTopk& tk = *reinterpret_cast<SliceTopk*>(k.base + k.a.g.topk_off);
+  SliceSettle& scratch = *reinterpret_cast<SliceSettle*>(k.base + k.a.g.list_off);
   const float* const own = reinterpret_cast<const float*>(k.base + k.a.g.own_off);
   const int* const own_cnt = reinterpret_cast<const int*>(k.base + k.a.g.stash_off);
   const int c = k.c, R = k.R, lane = k.lane, cap = k.a.g.list_cap, k_top = k.a.f.top_k;
@@ -763,7 +785,7 @@ __device__ __forceinline__ void slice_settle_rows(const Slice<T, CFG>& k) {
       }
     };
     float4 v;
-    const bool done = !over && slice_settle(tk, g, n_lo, k_top, k.a.g.exact != 0, lv.x, lv.y, sm.rs.tokz[r], each, v);
+    const bool done = !over && slice_settle(scratch, g, n_lo, k_top, k.a.g.exact != 0, lv.x, lv.y, sm.rs.tokz[r], each, v);
     if (g.w == 0) {
       if (done) {
         if (lane < c) cluster_store_f4(&tk.res[r], (uint32_t)lane, v);
@@ -777,7 +799,7 @@ __device__ __forceinline__ void slice_settle_rows(const Slice<T, CFG>& k) {
   for (int w = 0; w < kSliceRows / 32; ++w) {
     for (unsigned bits = tk.need[w]; bits; bits &= bits - 1u) {   // (the same in every thread; nobody adds to it any more)
       const int r = 32 * w + __ffs(bits) - 1;
-      const float4 v = slice_exact_row<T, CFG>(k.row(r), k.a.f.fin.V, k_top, k.a.g.vec_ok, tk);
+      const float4 v = slice_exact_row<T, CFG>(k.row(r), k.a.f.fin.V, k_top, k.a.g.vec_ok, scratch);
       if (k.tid < c) cluster_store_f4(&tk.res[r], (uint32_t)k.tid, v);
     }
   }
@@ -955,7 +977,249 @@ __device__ __forceinline__ void slice_finish_chain(const Slice<T, CFG>& k, int s
   }
 }
 
+// ---- trees: the walk of tree_finish_kernel, every block on its slice -----------------------------------------------
+// Rows 2 c and 2 c + 1 are context c's.  Every thread of every block follows the walk and takes the accept decisions; a
+// rejection costs one pass over the slices of the context's two rows and one cluster barrier.  The current context's
+// residual and the drafter's Q over the slice stay in two tables, so that later rejections there update them in place.
 template <typename T, bool CFG, bool TOPK>
+__device__ __forceinline__ void slice_finish_tree(const Slice<T, CFG>& k, int status_any) {
+  constexpr int VEC = Elem<T>::kVec;
+  SliceSmem& sm = k.sm;
+  SliceTree& tr = *reinterpret_cast<SliceTree*>(k.base + k.a.g.tree_off);
+  const FinishArgs& f = k.a.f.fin;
+  const int N = k.a.N, D = k.a.D, tid = k.tid, lane = k.lane, warp = k.warp, b = k.b, n = k.n;
+  double* const tile_sums = reinterpret_cast<double*>(k.base + k.a.g.tile_off);
+  float* const tabG = reinterpret_cast<float*>(k.base + k.a.g.tab_off);
+  float* const tabQ = tabG + (n + 3) / 4 * 4;
+  auto valid = [&](const int r) {
+    const float2 v = sm.rs.ms[r];
+    return v.x > CSD_NEG_INF && v.x < CSD_POS_INF && v.y >= 0.0f && v.y < CSD_POS_INF;
+  };
+  if (TOPK && tid < N) {
+    const int cx = k.a.parent[tid] + 1;
+    if (tr.tokz[0][tid] < sm.rs.thr[2 * cx]) tr.tokz[0][tid] = CSD_NEG_INF;
+    if (tr.tokz[1][tid] < sm.rs.thr[2 * cx + 1]) tr.tokz[1][tid] = CSD_NEG_INF;
+  }
+  __syncthreads();
+  const float u = tr.u;
+  int status = 0, level = 0, cx = 0, token = -1, passes = 0, owner = 0;
+  int kr = 0;              // rejections in the current context
+  double Z = 0.0, zk = 0.0, incl = 0.0;
+  bool drew = false;
+  PairCtx pc;
+  Row<T, CFG> ft, fd;      // (their filters)
+  const unsigned char *pt = nullptr, *ptu = nullptr, *pd = nullptr, *pdu = nullptr;
+  float omega = 0.0f;
+  auto open = [&](const int r, const unsigned char*& p, const unsigned char*& pu) {
+    if (k.a.g.slots < k.R && !k.need(r)) status_any |= 8;
+    k.slice_at(r, p, pu);
+  };
+  auto load = [&](const int xo, const bool both, float (&zt)[VEC], float (&zd)[VEC]) {
+    k.vec_at(pt, ptu, xo, zt);
+    if (both) k.vec_at(pd, pdu, xo, zd);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      if (TOPK) zt[e] = ft.filter(zt[e]);
+      zd[e] = both ? (TOPK ? fd.filter(zd[e]) : zd[e]) : 0.0f;
+    }
+  };
+  // one pass: the tiles' sums of `weight`, and the totals
+  auto pass = [&](auto weight) {
+    slice_tiles(k, tile_sums, weight);
+    Z = k.total(k.my_total(tile_sums), passes++ & 1, zk, incl);
+  };
+  for (;;) {
+    const bool t_ok = valid(2 * cx);
+    ft.thr = sm.rs.thr[2 * cx];
+    fd.thr = sm.rs.thr[2 * cx + 1];
+    pc.Mt = sm.rs.ms[2 * cx].x; pc.St = sm.rs.ms[2 * cx].y;
+    pc.inv_t = 1.0f / (1.0f + pc.St);
+    int first_child = -1;
+    for (int m = 0; m < N; ++m)
+      if (k.a.parent[m] == cx - 1) { first_child = m; break; }
+    kr = 0;
+    if (first_child < 0 || level >= D) {   // a leaf: bonus token from the target's distribution here
+      pc.mode = 1; pc.Md = 0.0f; pc.Sd = 0.0f; pc.inv_den = pc.inv_t; pc.one_minus_omega = 1.0f;
+      if (!t_ok) status |= 1;
+      drew = t_ok;
+      if (drew) {
+        open(2 * cx, pt, ptu);
+        pass([&](const int xo) {
+          float zt[VEC], zd[VEC], acc = 0.0f;
+          load(xo, false, zt, zd);
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) acc += residual_of(zt[e], 0.0f, pc, omega, 0, tr.inv_z, tr.keep);
+          return acc;
+        });
+      }
+      break;
+    }
+    const bool d_ok = valid(2 * cx + 1);
+    pc.mode = d_ok ? 0 : 1;
+    pc.Md = d_ok ? sm.rs.ms[2 * cx + 1].x : 0.0f; pc.Sd = d_ok ? sm.rs.ms[2 * cx + 1].y : 0.0f;
+    pc.inv_den = pc.inv_t / (1.0f + pc.Sd);
+    omega = tr.omega[level];
+    pc.one_minus_omega = 1.0f - omega;
+    const bool tab = pc.mode == 0;
+    int accepted = -1;
+    for (int m = first_child; m < N; ++m) {
+      if (k.a.parent[m] != cx - 1) continue;
+      // ---- accept test of candidate m against the residual after kr rejections --------------------------------------
+      const int tok = tr.tok[m];
+      float fa = 0.0f;
+      int flag = 0;
+      if (!t_ok || !d_ok) flag = 1;
+      else if (tok < 0 || tok >= f.V) flag = 2;
+      else {
+        const float zt = tr.tokz[0][m], zd = tr.tokz[1][m];
+        const float dt = zt - pc.Mt, dd = zd - pc.Md;
+        if (dd == CSD_NEG_INF) fa = 1.0f;            // q = 0: p/q = +inf, and 0/0 := 1
+        else if (kr == 0) {
+          if (dt == CSD_NEG_INF) fa = 0.0f;          // p = 0 < q
+          else fa = fminf(1.0f, omega * ex2f((dt - dd) * kLog2e) * ((1.0f + pc.Sd) / (1.0f + pc.St)));
+        } else {
+          const float Rm = residual_of(zt, zd, pc, omega, kr, tr.inv_z, tr.keep) * tr.inv_z[kr - 1];
+          const float Q = ex2f(dd * kLog2e) / (1.0f + pc.Sd);
+          fa = Rm > 0.0f ? fminf(1.0f, omega * Rm / Q) : 0.0f;
+        }
+      }
+      status |= flag;
+      if (tr.uni[m] <= fa) { accepted = m; break; }
+      if (!t_ok) continue;   // nothing to update: the emitted token will be -1
+      if (kr >= kMaxSiblings) { status |= 4; continue; }   // (the host refuses such trees)
+      // ---- rejected: one pass over the slices for the normaliser of the next residual -------------------------------
+      if (kr == 0) {
+        open(2 * cx, pt, ptu);
+        if (tab) open(2 * cx + 1, pd, pdu);
+      }
+      __syncthreads();
+      if (tid == 0) tr.keep[kr] = 0;
+      __syncthreads();
+      for (int attempt = 0; attempt < 2; ++attempt) {
+        if (tab && kr >= 1 && attempt == 1) {
+          // the update found an empty positive part and has overwritten the table: bring g_kr back from the logits
+          for (int xo = tid * VEC; xo < n; xo += kSliceThreads * VEC) {
+            float zt[VEC], zd[VEC];
+            load(xo, true, zt, zd);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e)
+              if (xo + e < n) tabG[xo + e] = residual_of(zt[e], zd[e], pc, omega, kr, tr.inv_z, tr.keep);
+          }
+          __syncthreads();
+        }
+        const float iz = kr >= 1 ? tr.inv_z[kr - 1] : 0.0f;
+        const bool kp = tr.keep[kr] != 0;
+        pass([&](const int xo) {
+          float acc = 0.0f;
+          if (tab && kr >= 1) {
+            // g_{kr+1} from the tabulated g_kr and Q: the last step of residual_of's recursion
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+              if (xo + e < n) {
+                const float Rx = tabG[xo + e] * iz;
+                const float gn = kp ? Rx : fmaxf(0.0f, Rx - fminf(tabQ[xo + e], omega * Rx));
+                tabG[xo + e] = gn;
+                acc += gn;
+              }
+            }
+          } else {
+            float zt[VEC], zd[VEC];
+            load(xo, tab, zt, zd);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+              const float gn = residual_of(zt[e], zd[e], pc, omega, kr + 1, tr.inv_z, tr.keep);
+              if (tab && xo + e < n) {   // (kr == 0: the tables are filled here)
+                tabG[xo + e] = gn;
+                tabQ[xo + e] = ex2f((zd[e] - pc.Md) * kLog2e) / (1.0f + pc.Sd);
+              }
+              acc += gn;
+            }
+          }
+          return acc;
+        });
+        const bool good = Z > 0.0 && Z < (double)CSD_POS_INF;
+        if (good || attempt == 1) {
+          if (tid == 0) tr.inv_z[kr] = good ? (float)(1.0 / Z) : 0.0f;
+          break;
+        }
+        status |= 4;   // empty positive part: the residual stays as it is
+        if (tid == 0) tr.keep[kr] = 1;
+        __syncthreads();
+      }
+      __syncthreads();
+      ++kr;
+    }
+    if (accepted >= 0) {
+      if (tid == 0) { tr.path_tok[level] = tr.tok[accepted]; tr.path_node[level] = accepted; }
+      ++level;
+      cx = accepted + 1;
+      continue;
+    }
+    drew = t_ok && kr > 0;
+    break;
+  }
+  // ---- the draw: from the last pass's tile sums -----------------------------------------------------------------
+  const bool usable = drew && Z > 0.0 && Z < (double)CSD_POS_INF;
+  const bool tab = pc.mode == 0 && kr > 0;
+  auto weights_at = [&](const int xo, float (&g)[VEC]) {
+    if (tab) {
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) g[e] = xo + e < n ? tabG[xo + e] : 0.0f;
+    } else {
+      float zt[VEC], zd[VEC];
+      load(xo, false, zt, zd);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) g[e] = xo + e < n ? residual_of(zt[e], 0.0f, pc, omega, kr, tr.inv_z, tr.keep) : 0.0f;
+    }
+  };
+  if (usable) {
+    const double target = (double)u * Z;
+    owner = k.owner_of(target, zk, incl);
+    if (owner == k.me) {
+      if (warp == 0) {
+        const double target_here = target - __shfl_sync(0xffffffffu, incl - zk, k.me);
+        locate_crossing_tile(tile_sums, k.my_tiles, u, lane, sm.fin, &target_here);
+        __syncwarp();
+        const int t = sm.fin.pick_tile;
+        int tok = -1;
+        if (t >= 0) {
+          const int xo = t * Slice<T, CFG>::TILE + lane * VEC;
+          float g[VEC];
+          weights_at(xo, g);
+          tok = pick_in_tile<VEC>(g, k.x_begin + xo, sm.fin.pick_prefix, target_here, lane);
+        }
+        if (lane == 0) sm.fin.token = tok;
+      }
+      __syncthreads();
+      token = sm.fin.token;
+    }
+  }
+  if (f.dbg_G) {   // each block writes its slice
+    float* G_out = f.dbg_G + (int64_t)b * f.V + k.x_begin;
+    const float invZ = usable ? (float)(1.0 / Z) : 0.0f;
+    for (int xo = tid * VEC; xo < n; xo += kSliceThreads * VEC) {
+      float g[VEC];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) g[e] = 0.0f;
+      if (usable) weights_at(xo, g);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e)
+        if (xo + e < n) G_out[xo + e] = g[e] * invZ;
+    }
+  }
+  __syncthreads();
+  if (owner != k.me) return;
+  if (tid <= D) {
+    f.out_tokens[(int64_t)b * (D + 1) + tid] = tid < level ? tr.path_tok[tid] : (tid == level ? token : -1);
+    if (k.a.out_nodes && tid < D) k.a.out_nodes[(int64_t)b * D + tid] = tid < level ? tr.path_node[tid] : -1;
+  }
+  if (tid == 0) {
+    f.out_accept_len[b] = level;
+    if (f.out_status) f.out_status[b] = status | status_any;
+  }
+}
+
+template <typename T, bool CFG, bool TOPK, bool TREE>
 __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const SliceArgs a) {
   extern __shared__ __align__(128) unsigned char fused_smem_raw[];
   SliceSmem& sm = *reinterpret_cast<SliceSmem*>(fused_smem_raw);
@@ -963,9 +1227,9 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   const FinishArgs& f = a.f.fin;
   const int tid = k.tid, lane = k.lane, c = k.c, R = k.R, slots = a.g.slots;
 
-  if (tid < slots) { mbar_init(&sm.full[tid], 1); sm.left[tid] = 1 << a.g.wpr_log2; sm.issued[tid] = 0; sm.cur[tid] = -1; }
+  if (tid < slots) { mbar_init(&sm.full[tid], 1); sm.left[tid] = a.g.parts; sm.issued[tid] = 0; sm.cur[tid] = -1; }
   if (tid == 0) sm.abort = 0;
-  if (TOPK && tid < kSliceRows / 32) reinterpret_cast<SliceTopk*>(fused_smem_raw + a.g.list_off)->need[tid] = 0u;
+  if (TOPK && tid < kSliceRows / 32) reinterpret_cast<SliceTopk*>(fused_smem_raw + a.g.topk_off)->need[tid] = 0u;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
   if (c > 1) cluster_arrive();   // first half; waited for before the first store to a peer
@@ -979,13 +1243,32 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   const int L = f.gamma;
   int tok = -1;
   float uni = 0.0f, omega = 0.0f, ztok = CSD_POS_INF;
-  if (tid <= L) uni = __ldcg(&f.uniforms[(int64_t)k.b * (L + 1) + tid]);
-  if (tid < L) omega = __ldcg(&f.schedule[tid]);
-  if (tid < 2 * L) {
-    tok = __ldcg(&f.tokens[(int64_t)k.b * L + (tid >> 1)]);
-    if (tok >= 0 && tok < f.V) ztok = k.row(tid).load_one(tok);
+  float ztok2 = 0.0f;
+  if (TREE) {   // (thread n takes node n's token, in both rows of its parent's context)
+    if (tid <= a.N) uni = __ldcg(&f.uniforms[(int64_t)k.b * (a.N + 1) + tid]);
+    if (tid < a.D) omega = __ldcg(&f.schedule[tid]);
+    if (tid < a.N) {
+      tok = __ldcg(&f.tokens[(int64_t)k.b * a.N + tid]);
+      const int cx = a.parent[tid] + 1;
+      if (tok >= 0 && tok < f.V) { ztok = k.row(2 * cx).load_one(tok); ztok2 = k.row(2 * cx + 1).load_one(tok); }
+    }
+  } else {
+    if (tid <= L) uni = __ldcg(&f.uniforms[(int64_t)k.b * (L + 1) + tid]);
+    if (tid < L) omega = __ldcg(&f.schedule[tid]);
+    if (tid < 2 * L) {
+      tok = __ldcg(&f.tokens[(int64_t)k.b * L + (tid >> 1)]);
+      if (tok >= 0 && tok < f.V) ztok = k.row(tid).load_one(tok);
+    }
   }
   auto late = [&]() {
+    if (TREE) {
+      SliceTree& tr = *reinterpret_cast<SliceTree*>(fused_smem_raw + a.g.tree_off);
+      if (tid < a.N) { tr.tok[tid] = tok; tr.uni[tid] = uni; tr.tokz[0][tid] = ztok; tr.tokz[1][tid] = ztok2; }
+      if (tid == a.N) tr.u = uni;
+      if (tid < a.D) tr.omega[tid] = omega >= 0.0f ? omega : 0.0f;
+      if (TOPK && tid < R) sm.rs.tokz[tid] = CSD_POS_INF;   // (every row is taken exactly: no rank is asked for)
+      return;
+    }
     if (tid <= L) sm.fst.uni[tid] = uni;
     if (tid < L) sm.fst.omega[tid] = omega >= 0.0f ? omega : 0.0f;
     if (tid < 2 * L && !(tid & 1)) sm.fst.tok[tid >> 1] = tok;
@@ -999,14 +1282,13 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
     late();
   }
   if (!ok) *(volatile int*)&sm.abort = 1;
-  const int wl = a.g.wpr_log2;
   float2* const xs = reinterpret_cast<float2*>(fused_smem_raw + a.g.rec_off);   // [c][parts][R]
   if (!TOPK && !a.g.direct) {   // the warps' parts of a row are merged before they go to the other blocks
     __syncthreads();
     const float2* const stash = reinterpret_cast<const float2*>(fused_smem_raw + a.g.stash_off);
     for (int r0 = 2 * k.warp; r0 < R; r0 += 2 * kSliceWarps) {
       const int r = r0 + (lane >> 4), part = lane & 15;
-      const float2 v = merge_parts((part < (1 << wl) && r < R) ? stash[(r << wl) + part] : make_float2(CSD_NEG_INF, -1.0f), lane, 16);
+      const float2 v = merge_parts((part < a.g.parts && r < R) ? stash[r * a.g.parts + part] : make_float2(CSD_NEG_INF, -1.0f), lane, 16);
       if (part < c && r < R) cluster_store_f2(&xs[k.me * R + r], (uint32_t)part, v);
     }
   }
@@ -1023,7 +1305,7 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   else __syncthreads();
 
   // ---- every row's statistics over the whole vocabulary (top-k: of what the filter keeps) ----------------------------------------------------------
-  const int np = a.g.direct ? c << wl : c;   // parts of a row, at most 32
+  const int np = a.g.direct ? c * a.g.parts : c;   // parts of a row, at most 32
   if (TOPK) {
     slice_settle_rows<T, CFG>(k);
   } else if (np <= 16) {
@@ -1042,7 +1324,8 @@ __global__ void __launch_bounds__(kSliceThreads, 2) verify_slice_kernel(const Sl
   for (int q = 0; q < c; ++q) status_any |= sm.xflag[q] ? 8 : 0;
   if (a.f.error_flag && __ldcg(a.f.error_flag)) status_any |= 8;
   __syncthreads();
-  slice_finish_chain<T, CFG, TOPK>(k, status_any);
+  if (TREE) slice_finish_tree<T, CFG, TOPK>(k, status_any);
+  else slice_finish_chain<T, CFG, TOPK>(k, status_any);
 }
 
 }  // namespace csd
