@@ -313,8 +313,10 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
   const size_t tables = TREE ? 2 * (size_t)(n + 4) * sizeof(float) : 0;
   const size_t scratch = TOPK ? sizeof(SliceSettle) : 0;
   if (TOPK) {
-    const double e = tail * n;   // values a slice's list expects
-    g.list_cap = ((int)(1.25 * e + 6.0 * sqrt(e) + 24.0) + 3) / 4 * 4;
+    // values a slice's list expects, with room for a Student-t row of three degrees of freedom: far out its tail beyond a
+    // level found by moments is several times a Gaussian's (1.9 at 1.5 % of the row, 2.9 at 0.8, 5.3 at 0.3)
+    const double e = tail * n, room_for = tail < 0.035 ? 1.25 * pow(0.035 / tail, 0.6) : 1.25;
+    g.list_cap = ((int)(room_for * e + 6.0 * sqrt(e) + 24.0) + 3) / 4 * 4;
     if (g.list_cap > n) g.list_cap = n;
     g.topk_off = take(sizeof(SliceTopk));
     const size_t lists = owned * c * g.list_cap * sizeof(float);
@@ -343,6 +345,7 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
 // the busiest SM goes through, fitted to (us per call, sliced / position split):
 //   no top-k: 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3, B=16 17.6 / 15.2; 64 K bf16 B=4 18.0 / 23.2, fp32
 //   gamma=16 B=1 31.9 / 41.5, B=8 48 / 42; drafting calls of 64 guided rows of 16 K 8.7 / 11.5, 25 of 23 K 8.3 / 13.3;
+//   (the same 64 rows with eight blocks each, two waves: 18.2; 35 rows of 4.3 K 7.0 - 8.0 by one to four blocks, 14.9 by eight);
 //   top-k: guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; drafting calls of 64
 //   rows of 16 K 15.1 / 13.6, 20 of 30 K 13.9 / 20.5; guided 33 K top-k 1823 gamma=13 B=8 (five turns) 73.7 / 63.6.
 template <typename T, bool CFG, bool TOPK, bool TREE>
@@ -365,7 +368,7 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
     int np, upp;   // the work of a block: its busiest warp's, times its warps
     const double logits = (double)slice_rounds(R, (((ntiles + c - 1) / c) * TILE + kSliceUnit - 1) / kSliceUnit, np, upp) * kSliceUnit * kSliceWarps;
     auto expect = [&](int waves, double per_sm) {
-      return waves * ((TOPK ? 11e3 : 7e3) + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
+      return waves * ((TOPK ? 10e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
     };
     if (expect(1, logits) >= best) continue;
     // a block to an SM where the clusters fit so, with room for more rows at once; else two
@@ -373,8 +376,8 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
     if (cap1 <= 0 || cap2 <= 0) continue;
     const int waves = (f.B + cap2 - 1) / cap2;
     double ns = expect(waves, f.B <= cap1 ? logits : 1.7 * waves * logits);
-    // (more blocks if that is nearly as good: 24 unaligned sequences, bf16: eight blocks each 23.1 us, four 25.9)
-    if (best_c == 0 ? ns >= best : ns * 8 >= best * 7) continue;
+    if (f.B > 0.8 * cap2) ns *= 1.25;   // clusters wait for room in one GPC (trees of 4.8 K fp32, B=30: nine blocks 32.5 us, six 21.6)
+    if (ns >= best) continue;
     SliceGeo g;
     size_t need;
     bool fits = slice_layout<T, CFG, TOPK, TREE>(a, R, c, kSliceSmem[0], tail, g, need);
@@ -426,7 +429,7 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   const double logits = (double)rows * in.fa.V;
   // (a tree: the statistics of all rows, then the walk by one block per sequence)
   const double other_ns = tree ? ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms)
-                          : in.topk ? 5e3 + 0.39 * logits : 9e3 + 0.09 * logits;
+                          : in.topk ? (rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 6e3 + 0.5 * logits) : 9e3 + 0.09 * logits;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;

@@ -27,6 +27,7 @@ constexpr int kSliceRows = 2 * (kMaxTreeNodes + 1);
 constexpr int kSliceUnit = 512;         // logits of a warp's unit of work: 16 per lane
 constexpr int kSliceSample = 4096;      // top-k: logits of a row that the moments are taken from, over all blocks
 constexpr int kSliceBins = 128;         // per row being settled: histogram of the values between the two levels
+constexpr int kSliceTurns = 6;          // ... how often a crowded bin is divided again
 constexpr int kSliceCand = 64;          // per row being settled: values of the bin that holds the threshold
 static_assert(kSliceRows <= kBlockRows, "a block's row results live in RowStats");
 
@@ -653,8 +654,9 @@ struct RowGroup {
 //   below 2^-26 of the normaliser: nothing that fp32 can see.  The row's (m, s) is that of everything gathered and
 //   `lo` serves as its threshold; the drafted token is dropped if k gathered values lie above its logit;
 // - the exact threshold: a histogram of the values between the levels finds the bin of the k-th largest, its rank among
-//   the bin's few values the value.
-// False if neither can be had (the lists do not hold the k largest, a crowded bin): the row is read again.  The group's
+//   the bin's few values the value.  (Heavy tails leave the upper level with more than k values above it; the histogram
+//   then spans everything up to the maximum and its crowded bin is divided again.)
+// False if neither can be had (the lists do not hold the k largest): the row is read again.  The group's
 // results are the same in all its threads.
 // (By one warp a row took 6 us with the short cut and up to 30 without, 16 K and 64 K vocabularies; by the block's warps 1 - 3.)
 template <typename Each>
@@ -713,35 +715,64 @@ __device__ __forceinline__ bool slice_settle(SliceSettle& tk, const RowGroup& g,
     out = make_float4(m, all.x + (all.y - 1.0f), lo, (int)all.w >= k_top ? 1.0f : 0.0f);
     return true;
   }
-  int kk = k_top - n_hi;   // rank of the answer among the values in [lo, hi]
-  const float scale = (float)kSliceBins * rcp_approx(hi - lo);
-  if (!(scale < CSD_POS_INF)) return false;
-  auto bin_of = [&](const float v) { return min(kSliceBins - 1, (int)__fmul_rn(__fsub_rn(v, lo), scale)); };
-  each([&](const float v) { if (!(v > hi)) atomicAdd(&hist[bin_of(v)], 1); });
-  g.sync();
-  int above;
-  const int bin = select_bin_from_top(hist, kSliceBins, kk, lane, &above);
-  kk -= above;
-  each([&](const float v) {
-    if (!(v > hi) && bin_of(v) == bin) {
-      const int at = atomicAdd(&tk.n_cand[g.id], 1);
-      if (at < kSliceCand) cand[at] = v;
+  // the answer has rank kk among the values in [from, to]; a bin that holds too many to be ranked is divided again
+  int kk = k_top - n_hi, nc = 0;
+  float from = lo, to = hi;
+  for (int turn = 0;; ++turn) {
+    if (turn == kSliceTurns) return false;
+    const float scale = (float)kSliceBins * rcp_approx(to - from);
+    if (!(scale < CSD_POS_INF)) return false;
+    // (monotone, so a bin's values are all those between its smallest and its largest)
+    auto bin_of = [&](const float v) { return min(kSliceBins - 1, (int)__fmul_rn(__fsub_rn(v, from), scale)); };
+    each([&](const float v) { if (v >= from && !(v > to)) atomicAdd(&hist[bin_of(v)], 1); });
+    g.sync();
+    int above;
+    const int bin = select_bin_from_top(hist, kSliceBins, kk, lane, &above);
+    kk -= above;
+    nc = hist[bin];
+    float least = CSD_POS_INF, most = CSD_NEG_INF;
+    each([&](const float v) {
+      if (v >= from && !(v > to) && bin_of(v) == bin) {
+        if (nc <= kSliceCand) cand[atomicAdd(&tk.n_cand[g.id], 1)] = v;
+        least = fminf(least, v);
+        most = fmaxf(most, v);
+      }
+    });
+    if (nc <= kSliceCand) break;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      least = fminf(least, __shfl_xor_sync(0xffffffffu, least, off));
+      most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, off));
     }
-  });
-  g.sync();
-  const int nc = tk.n_cand[g.id];
-  if (nc > kSliceCand) return false;
-  const float v0 = lane < nc ? cand[lane] : CSD_NEG_INF, v1 = lane + 32 < nc ? cand[lane + 32] : CSD_NEG_INF;
-  int gt0 = 0, ge0 = 0, gt1 = 0, ge1 = 0;
-  for (int i = 0; i < nc; ++i) {
-    const float w = cand[i];
-    gt0 += (w > v0) ? 1 : 0; ge0 += (w >= v0) ? 1 : 0;
-    gt1 += (w > v1) ? 1 : 0; ge1 += (w >= v1) ? 1 : 0;
+    if (lane == 0) red[g.w] = make_float4(least, most, 0.0f, 0.0f);
+    g.sync();   // (everybody has read the histogram)
+    for (int i = g.w * 32 + lane; i < kSliceBins; i += 32 * g.G) hist[i] = 0;
+    float4 v = red[lane < g.G ? lane : 0];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) {
+      v.x = fminf(v.x, __shfl_xor_sync(0xffffffffu, v.x, off));
+      v.y = fmaxf(v.y, __shfl_xor_sync(0xffffffffu, v.y, off));
+    }
+    from = __shfl_sync(0xffffffffu, v.x, 0);
+    to = __shfl_sync(0xffffffffu, v.y, 0);
+    g.sync();
+    if (from == to) break;   // equal values: they are the answer
   }
-  const unsigned b0 = __ballot_sync(0xffffffffu, lane < nc && gt0 < kk && kk <= ge0);
-  const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < nc && gt1 < kk && kk <= ge1);
-  if ((b0 | b1) == 0u) return false;
-  const float thr = b0 ? __shfl_sync(0xffffffffu, v0, __ffs(b0) - 1) : __shfl_sync(0xffffffffu, v1, __ffs(b1) - 1);
+  float thr = from;
+  if (from < to) {
+    g.sync();
+    const float v0 = lane < nc ? cand[lane] : CSD_NEG_INF, v1 = lane + 32 < nc ? cand[lane + 32] : CSD_NEG_INF;
+    int gt0 = 0, ge0 = 0, gt1 = 0, ge1 = 0;
+    for (int i = 0; i < nc; ++i) {
+      const float w = cand[i];
+      gt0 += (w > v0) ? 1 : 0; ge0 += (w >= v0) ? 1 : 0;
+      gt1 += (w > v1) ? 1 : 0; ge1 += (w >= v1) ? 1 : 0;
+    }
+    const unsigned b0 = __ballot_sync(0xffffffffu, lane < nc && gt0 < kk && kk <= ge0);
+    const unsigned b1 = __ballot_sync(0xffffffffu, lane + 32 < nc && gt1 < kk && kk <= ge1);
+    if ((b0 | b1) == 0u) return false;
+    thr = b0 ? __shfl_sync(0xffffffffu, v0, __ffs(b0) - 1) : __shfl_sync(0xffffffffu, v1, __ffs(b1) - 1);
+  }
   acc = 0.0f;
   cmax = 0;
   each([&](const float v) {

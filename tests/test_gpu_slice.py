@@ -89,6 +89,8 @@ def test_drafting_draws(R, V):
     dict(B=1, gamma=32, V=16384, dtype=W.BF16, top_k=200, bonus_row=True),       # 65 rows: five to a block
     dict(B=2, gamma=8, V=65536, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=2000, bonus_row=True),   # rows in turns
     dict(B=3, gamma=8, V=16384, dtype=W.BF16, law="student3", rho=0.85, top_k=500),
+    dict(B=3, gamma=4, V=48272, dtype=W.BF16, law="student3", rho=0.85, cfg=True, top_k=236),   # far out a heavy tail: bins divided again
+    dict(B=2, gamma=4, V=65536, dtype=W.BF16, scale=0.5, top_k=2000),                          # a hundred equal values at the threshold
     dict(B=3, gamma=8, V=16387, dtype=W.BF16, top_k=500, bonus_row=True), dict(B=3, gamma=8, V=16387, dtype=W.F32, cfg=True, top_k=40),
 ])
 @pytest.mark.parametrize("want_dbg", [False, True])
