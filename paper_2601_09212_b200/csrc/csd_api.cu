@@ -237,6 +237,20 @@ cudaError_t launch_finish(const FinishArgs& a_in, cudaStream_t stream) {
 long long g_wait_limit = kWaitCycles;
 int g_drop_first_copy = 0;
 
+// Into how many blocks the position split cuts a sequence in stream order: powers of two while there are at most two
+// blocks to an SM (with top-k, whose per-row work is longer, four), and without top-k once more if the clusters then fit
+// the three blocks an SM holds with room to spare and the busiest SM has at least a seventh fewer rows.  us per call
+// before and after that doubling: B=100 gamma=12 V=17152 fp32 (400 blocks, 0.81 of the rows) 46.4 and 38.8, B=200 gamma=6
+// V=9000 bf16 (400, 0.81) 24.7 and 21.7; but B=110 gamma=14 (440, 0.90) 30.0 and 39.5, and three to a sequence B=144 gamma=9
+// (432, 0.90) 42.1 and 50.5: clusters do not pack into the last slots.
+int position_split(int B, int gamma, int T, bool topk, int sms) {
+  int c = 1;
+  while (2 * c <= (topk ? 4 : 2) * sms / B && 2 * c <= gamma && 2 * c <= kMaxCluster) c *= 2;
+  if (topk || 2 * c > gamma || 2 * c > kMaxCluster || 2LL * c * B * 4 > 11LL * sms) return c;
+  auto load = [&](int n) { return ((B * n + sms - 1) / sms) * (2 * ((gamma + n - 1) / n) + (T > gamma ? 1 : 0)); };
+  return load(2 * c) * 7 <= load(c) * 6 ? 2 * c : c;
+}
+
 // ---- the vocabulary-sliced kernel (csd_slice.cuh) ------------------------------------------------------------
 constexpr size_t kSliceSmem[2] = {113 * 1024, 226 * 1024};   // two blocks per SM, one block per SM
 
@@ -303,10 +317,13 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
   g.slot_bytes = (n * ES + (g.vec_ok ? 0 : 16)) * ARR;
   slice_rounds(R, upr, g.parts, g.upp);
   g.direct = c * g.parts <= 32 ? 1 : 0;
+  g.su = kSliceSample / kSliceUnit / c;
+  if (g.su < 1) g.su = 1;
+  if (g.su > upr) g.su = upr;
   size_t off = kSliceHeader;
   auto take = [&](size_t want) { const size_t o = off; off += (want + 127) / 128 * 128; return (int)o; };
   const size_t owned = (size_t)(R + c - 1) / c;   // top-k: rows whose lists a block receives
-  g.rec_off = take((size_t)R * (TOPK ? (size_t)c * sizeof(float4) : (size_t)(g.direct ? c * g.parts : c) * sizeof(float2)));
+  g.rec_off = take((size_t)R * (TOPK ? (size_t)c * g.su * sizeof(float4) : (size_t)(g.direct ? c * g.parts : c) * sizeof(float2)));
   g.tile_off = take((size_t)tiles * sizeof(double));
   g.stash_off = take(TOPK ? owned * c * sizeof(int) : (g.direct ? 0 : (size_t)R * g.parts * sizeof(float2)));
   g.tree_off = take(TREE ? sizeof(SliceTree) : 0);
@@ -368,7 +385,7 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
     int np, upp;   // the work of a block: its busiest warp's, times its warps
     const double logits = (double)slice_rounds(R, (((ntiles + c - 1) / c) * TILE + kSliceUnit - 1) / kSliceUnit, np, upp) * kSliceUnit * kSliceWarps;
     auto expect = [&](int waves, double per_sm) {
-      return waves * ((TOPK ? 10e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
+      return waves * ((TOPK ? 11e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
     };
     if (expect(1, logits) >= best) continue;
     // a block to an SM where the clusters fit so, with room for more rows at once; else two
@@ -421,15 +438,13 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   // streams better than slices do (fp32 B=32: 16.9 us, sliced 21.1).
   const int B = in.fa.B, gamma = in.fa.gamma;
   const bool tree = in.N > 0;
-  int pos = 1;
-  const int split_below = (in.topk ? 4 : 2) * in.sms;
-  while (2 * pos <= split_below / B && 2 * pos <= gamma && 2 * pos <= kMaxCluster) pos *= 2;
+  const int pos = position_split(B, gamma, in.fa.T, in.topk, in.sms);
   if (in.fa.vec_ok && !tree && (long long)B * pos > in.sms) return cudaSuccess;
   const int rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
   const double logits = (double)rows * in.fa.V;
   // (a tree: the statistics of all rows, then the walk by one block per sequence)
   const double other_ns = tree ? ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms)
-                          : in.topk ? (rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 6e3 + 0.5 * logits) : 9e3 + 0.09 * logits;
+                          : in.topk ? (rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 5e3 + 0.5 * logits) : 9e3 + 0.09 * logits;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;
@@ -503,16 +518,17 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     // ctas_per_seq blocks of one cluster (each with both rows of its positions; 2, 4 or 8 blocks)
     // until the GPU is full.
     const long long merge_above = 8LL * sms;   // beyond this many sequences a block takes several
-    // (measured: the top-k kernel, with its longer per-row work, gains from the finer split)
     TopkGuess guess;
     const bool guessed = topk && topk_guess(in.top_k, in.V, guess);
     const double tk_v = in.V, tk_tail = topk ? guess.tail : 0.0;
     const bool tk_large = topk && tk_tail * tk_v >= 0.8 * (kTopkWarps * kWarpList);
-    const long long split_below = in.back_to_back ? 16 : (topk ? 4LL : 2LL) * sms;
     long long c = 1, spc = 1;
-    if (in.B > merge_above) spc = (in.B + merge_above - 1) / merge_above;
-    else if (in.B < split_below) {
-      const long long want = split_below / in.B;
+    if (in.B > merge_above) {
+      spc = (in.B + merge_above - 1) / merge_above;
+    } else if (!in.back_to_back) {
+      c = position_split(in.B, in.gamma, in.fa.T, topk, sms);
+    } else if (in.B < 16) {
+      const long long want = 16 / in.B;
       while (2 * c <= want && 2 * c <= in.gamma && 2 * c <= kMaxCluster) c *= 2;
     }
     while (spc > 1 && spc * rows_per_seq > kBlockRows) --spc;   // rows_per_seq <= 65 < kBlockRows

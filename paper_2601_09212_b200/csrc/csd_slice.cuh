@@ -37,6 +37,7 @@ struct SliceGeo {
   int vec_ok;              // rows are whole 16-byte vectors at 16-byte aligned addresses
   int parts, upp;          // a row's slice is dealt out to the warps in this many parts, of this many units each
   int direct;              // the warps' parts of a row go to the other blocks as they are (else merged first)
+  int su;                  // top-k: units of a slice in the sample that the moments are taken from
   int list_cap;            // top-k: values a row's list holds
   int exact;               // top-k: every row's exact threshold is wanted
   // dynamic shared memory after SliceSmem: offsets in bytes
@@ -447,29 +448,29 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
   const FusedArgs& a = k.a.f;
   const int slots = k.a.g.slots, R = k.R, cap = k.a.g.list_cap, lane = k.lane, c = k.c;
   const int np = k.a.g.parts, upp = k.a.g.upp;
-  float4* const mom = reinterpret_cast<float4*>(k.base + k.a.g.rec_off);   // [c][R]: sum, sum of |deviations|, values
+  float4* const mom = reinterpret_cast<float4*>(k.base + k.a.g.rec_off);   // [c][su][R]: sum, sum of |deviations|, values
   float* const lists = reinterpret_cast<float*>(k.base + k.a.g.list_off);   // of the group's rows
   float* const own = reinterpret_cast<float*>(k.base + k.a.g.own_off);     // [rows owned][c][cap]
   int* const own_cnt = reinterpret_cast<int*>(k.base + k.a.g.stash_off);   // [rows owned][c]
   const int groups = (R + slots - 1) / slots, G = (R + groups - 1) / groups;
   const uint32_t lanemask_lt = (1u << lane) - 1u;
-  // units of a row's slice in the sample: one warp takes them one after the other
-  const int su = min(k.upr, (kSliceSample / kSliceUnit + c - 1) / c);
+  const int su = k.a.g.su;
   bool ok = true, peers = c == 1;
   for (int g0 = 0; g0 < R; g0 += G) {
     const int g1 = min(R, g0 + G);
     // ---- moments of the sample: its sum, and the sum of absolute deviations from each unit's mean --------------------
-    for (int r = g0 + k.warp; r < g1; r += kSliceWarps) {
+    for (int i = k.warp; i < (g1 - g0) * su; i += kSliceWarps) {
+      const int r = g0 + i / su, u = i % su;
       if (ok && !k.wait_row(r)) ok = false;
       const unsigned char *p, *pu;
       k.slice_at(r, p, pu);
-      float s1 = 0.0f, s2 = 0.0f, cnt = 0.0f;
-      for (int u = 0; u < su; ++u) {
-        const int valid = min(kSliceUnit, k.n - u * kSliceUnit);
-        if (valid < kSliceUnit && u > 0) break;
+      // (a unit cut short counts only if it is all there is of the slice)
+      const int left = k.n - u * kSliceUnit, valid = left >= kSliceUnit ? kSliceUnit : (u == 0 ? left : 0);
+      float s1 = 0.0f, s2 = 0.0f;
+      if (valid > 0) {
         float z[16];
         k.unit(p, pu, u, z);
-        if (valid < kSliceUnit) {   // a slice of less than a unit: what lies beyond it does not count
+        if (valid < kSliceUnit) {
 #pragma unroll
           for (int e = 0; e < 16; ++e)
             if (k.unit_index(e) >= valid) z[e] = 0.0f;
@@ -479,10 +480,10 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
         for (int e = 0; e < 16; e += 2) s1p = add2(s1p, pack2(z[e], z[e + 1]));
         float x0, x1;
         unpack2(s1p, x0, x1);
-        float us = x0 + x1;
+        s1 = x0 + x1;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) us += __shfl_xor_sync(0xffffffffu, us, off);
-        const float wm = us * rcp_approx((float)valid);
+        for (int off = 16; off > 0; off >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        const float wm = s1 * rcp_approx((float)valid);
         const uint64_t nwm = pack2(-wm, -wm);
         float d0 = 0.0f, d1 = 0.0f;
 #pragma unroll
@@ -495,14 +496,12 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
           d0 += fabsf(x0);
           d1 += fabsf(x1);
         }
-        s1 += us;
-        s2 += d0 + d1;
-        cnt += (float)valid;
-      }
+        s2 = d0 + d1;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+        for (int off = 16; off > 0; off >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+      }
       if (!peers) { cluster_wait(); peers = true; }   // every peer is running
-      if (lane < c) cluster_store_f4(&mom[k.me * R + r], (uint32_t)lane, make_float4(s1, s2, cnt, 0.0f));
+      if (lane < c) cluster_store_f4(&mom[(k.me * su + u) * R + r], (uint32_t)lane, make_float4(s1, s2, (float)max(valid, 0), 0.0f));
     }
     if (!peers) { cluster_wait(); peers = true; }
     if (c > 1) { cluster_arrive(); cluster_wait(); }
@@ -510,7 +509,7 @@ __device__ __forceinline__ bool slice_rows_topk(const Slice<T, CFG>& k, Late lat
     if (k.tid < g1 - g0) {
       const int r = g0 + k.tid;
       float s1 = 0.0f, s2 = 0.0f, cnt = 0.0f;
-      for (int q = 0; q < c; ++q) {
+      for (int q = 0; q < c * su; ++q) {
         const float4 v = mom[q * R + r];
         s1 += v.x; s2 += v.y; cnt += v.z;
       }
