@@ -492,6 +492,8 @@ struct FusedPlan {
   float2* stats_out;
   float* thr_out;
   cudaStream_t stream;
+  float4* records = nullptr;   // with stats_out (see FusedArgs)
+  int v_offset = 0;
 };
 cudaError_t plan_and_launch_fused(const FusedPlan& in) {
   const int sms = in.sms, es = in.es, rows_per_seq = in.rows_per_seq;
@@ -508,6 +510,8 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     ua.error_flag = in.error_flag;
     ua.stats_out = in.stats_out;
     ua.thr_out = in.thr_out;
+    ua.records = in.records;
+    ua.v_offset = in.v_offset;
     ua.wait_limit = g_wait_limit;
     ua.drop_first_copy = g_drop_first_copy;
     // Blocks are aligned with sequences and positions.  For calls enqueued back to back a block owns a
@@ -1151,6 +1155,23 @@ int csd_shard_stats(const csd_shard_params* pp, void* out_records) {
   shard_args(p, sms, sa, st);
   sa.local = reinterpret_cast<float4*>(out_records);
   const bool cfg = p.target_uncond != nullptr;
+  if (sa.fin.vec_ok && (size_t)p.Vs * elem_size(p.dtype) >= 512) {
+    // one launch: the streaming kernel writes the records itself (it was two, 64 sequences of a quarter of 16 K: see the
+    // statistics and merge kernels below, which serve what it cannot take)
+    FusedPlan fp;
+    fp.fa = sa.fin;
+    fp.fa.parts = 1;
+    fp.B = p.B; fp.gamma = p.gamma; fp.V = p.Vs; fp.top_k = 0; fp.dtype = p.dtype;
+    fp.rows_per_seq = p.target_rows + p.gamma; fp.rows = (long long)p.B * fp.rows_per_seq; fp.sms = sms; fp.es = elem_size(p.dtype);
+    fp.cfg = cfg; fp.topk = false; fp.back_to_back = false; fp.allow_short_cut = false;
+    fp.error_flag = nullptr;
+    fp.stats_out = reinterpret_cast<float2*>((char*)p.workspace);   // (marks the call; the records carry the results)
+    fp.thr_out = nullptr;
+    fp.stream = (cudaStream_t)p.stream;
+    fp.records = reinterpret_cast<float4*>(out_records);
+    fp.v_offset = p.v_offset;
+    return plan_and_launch_fused(fp) == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+  }
   const int U = st.part_elems / (kStatsThreads * vec_width(p.dtype));
   cudaStream_t stream = (cudaStream_t)p.stream;
   const unsigned grid = (unsigned)((p.B * (p.target_rows + p.gamma) + 7) / 8);
@@ -1331,27 +1352,6 @@ size_t csd_host_staging_size(const csd_params* host) {
   return pl.total;
 }
 
-int csd_verify_host(const csd_params* host, void* staging, size_t staging_bytes) {
-  if (!host) return CSD_ERR_NULL;
-  const csd_params& h = *host;
-  if (!h.target_logits || !h.draft_logits || !h.draft_tokens || !h.uniforms || !h.relax_schedule ||
-      !h.out_tokens || !h.out_accept_len)
-    return CSD_ERR_NULL;
-  if (h.dtype != CSD_F32 && h.dtype != CSD_BF16) return CSD_ERR_DTYPE;
-  if ((h.target_uncond == nullptr) != (h.draft_uncond == nullptr)) return CSD_ERR_ARG;
-  HostPlan pl;
-  if (!host_plan(h, pl)) return CSD_ERR_SHAPE;
-  if (!staging || ((uintptr_t)staging % kAlign) != 0 || staging_bytes < pl.total) return CSD_ERR_WORKSPACE;
-  char* base = (char*)staging;
-  cudaStream_t stream = (cudaStream_t)h.stream;
-  auto h2d = [&](size_t off, const void* src, size_t bytes) {
-    return cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, stream);
-  };
-  auto d2h = [&](void* dst, size_t off, size_t bytes) {
-    return cudaMemcpyAsync(dst, base + off, bytes, cudaMemcpyDeviceToHost, stream);
-  };
-  cudaError_t e = h2d(pl.off_t, h.target_logits, pl.logits_t);
-  if (e == cudaSuccess) e = h2d(pl.off_d, h.draft_logits, pl.logits_d);
 }  // extern "C"
 namespace {
 // The host form's small inputs, read from mapped host memory, and the workspace header: one launch instead of three
@@ -1379,6 +1379,27 @@ void* mapped(const void* p) {
 }  // namespace
 extern "C" {
 
+int csd_verify_host(const csd_params* host, void* staging, size_t staging_bytes) {
+  if (!host) return CSD_ERR_NULL;
+  const csd_params& h = *host;
+  if (!h.target_logits || !h.draft_logits || !h.draft_tokens || !h.uniforms || !h.relax_schedule ||
+      !h.out_tokens || !h.out_accept_len)
+    return CSD_ERR_NULL;
+  if (h.dtype != CSD_F32 && h.dtype != CSD_BF16) return CSD_ERR_DTYPE;
+  if ((h.target_uncond == nullptr) != (h.draft_uncond == nullptr)) return CSD_ERR_ARG;
+  HostPlan pl;
+  if (!host_plan(h, pl)) return CSD_ERR_SHAPE;
+  if (!staging || ((uintptr_t)staging % kAlign) != 0 || staging_bytes < pl.total) return CSD_ERR_WORKSPACE;
+  char* base = (char*)staging;
+  cudaStream_t stream = (cudaStream_t)h.stream;
+  auto h2d = [&](size_t off, const void* src, size_t bytes) {
+    return cudaMemcpyAsync(base + off, src, bytes, cudaMemcpyHostToDevice, stream);
+  };
+  auto d2h = [&](void* dst, size_t off, size_t bytes) {
+    return cudaMemcpyAsync(dst, base + off, bytes, cudaMemcpyDeviceToHost, stream);
+  };
+  cudaError_t e = h2d(pl.off_t, h.target_logits, pl.logits_t);
+  if (e == cudaSuccess) e = h2d(pl.off_d, h.draft_logits, pl.logits_d);
   if (e == cudaSuccess && h.target_uncond) e = h2d(pl.off_tu, h.target_uncond, pl.logits_t);
   if (e == cudaSuccess && h.draft_uncond) e = h2d(pl.off_du, h.draft_uncond, pl.logits_d);
   // Pinned memory is reached from the device: the small inputs come by one kernel, and the small outputs are written where

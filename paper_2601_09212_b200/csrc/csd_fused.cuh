@@ -124,8 +124,12 @@ constexpr int kMaxCluster = 8;   // portable cluster size
 // of fp32 rows: 16.4 -> 15.1 us a call, one draft position of 64 rows: 16.4 -> 13.6).  The signal follows the
 // wait, so that a call that may overlap this one still starts after everything ahead of this one has completed.
 __device__ __forceinline__ void call_begin(const int ordered, const bool signal) {
-  if (ordered) pdl_wait();
+  if (!ordered) return;   // (such a call signals as its blocks start: call_enter)
+  pdl_wait();
   if (signal) pdl_launch_dependents();
+}
+__device__ __forceinline__ void call_enter(const int ordered, const bool signal) {
+  if (!ordered && signal) pdl_launch_dependents();
 }
 
 template <typename T>
@@ -185,6 +189,8 @@ struct FusedArgs {
   long long wait_limit; // cycles a wait on a copy may take (kWaitCycles unless a test shortens it)
   int large_lists;      // top-k: the instance with the large candidate lists (set by the host from k and V)
   float2* stats_out;    // not null: stop after the streaming phase and write every local row's (m, s) here,
+  float4* records;      // with stats_out, not null: (m, s, logit of the drafted token if this slice holds it) instead,
+  int v_offset;         //   for a slice of the vocabulary that begins at this token
   float* thr_out;       //   and its top-k threshold there (may be null), at row b * (T + gamma) + (target ? i : T + i)
   int ordered;          // ordinary stream order: nothing of the call's inputs is read before everything ahead of it
                         // on the stream has completed
@@ -952,6 +958,7 @@ __device__ void finish_block(const FusedArgs& ua, const BlockShare& sh, const Ro
 // Stats-only calls (FusedArgs::stats_out): the block's rows go to global memory in the row order of the
 // multi-launch kernels, after the previous operation on the stream has completed (its finishing kernel
 // may still be reading the same arrays).
+template <typename T, bool CFG>
 __device__ __forceinline__ void write_row_stats(const FusedArgs& a, const BlockShare& sh, const RowStats& rs, const int tid,
                                                 const int nthreads, const bool aborted) {
   pdl_wait();
@@ -960,6 +967,16 @@ __device__ __forceinline__ void write_row_stats(const FusedArgs& a, const BlockS
     int b, which, i;
     local_row(sh, r, f.gamma, b, which, i);
     const int64_t row_id = (int64_t)b * (f.T + f.gamma) + (which == 0 ? i : f.T + i);
+    if (a.records) {
+      float z = CSD_NEG_INF;
+      if (i < f.gamma) {
+        const int loc = __ldcg(&f.tokens[(int64_t)b * f.gamma + i]) - a.v_offset;
+        if (loc >= 0 && loc < f.V) z = row_at<T, CFG>(f, b, which, i).load_one(loc);
+      }
+      const float2 ms = aborted ? make_float2(__int_as_float(0x7fc00000), 0.0f) : rs.ms[r];
+      a.records[row_id] = make_float4(ms.x, ms.y, z, 0.0f);
+      continue;
+    }
     a.stats_out[row_id] = aborted ? make_float2(__int_as_float(0x7fc00000), 0.0f) : rs.ms[r];   // (a row of a call that
     if (a.thr_out) a.thr_out[row_id] = rs.thr[r];                                              //  gave up reads as unusable)
   }
@@ -1000,6 +1017,7 @@ __global__ void __launch_bounds__(kPlainThreads, 3) verify_plain_kernel(const Fu
   extern __shared__ __align__(128) unsigned char fused_smem_raw[];
   PlainSmem& sm = *reinterpret_cast<PlainSmem*>(fused_smem_raw);
 
+  call_enter(a.ordered, a.signal != 0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const FinishArgs& f = a.fin;
   const int V = f.V;
@@ -1264,7 +1282,7 @@ __global__ void __launch_bounds__(kPlainThreads, 3) verify_plain_kernel(const Fu
   }
   __syncthreads();
   if (stats_only) {
-    write_row_stats(a, sh, sm.rs, tid, kPlainThreads, sm.abort != 0);
+    write_row_stats<T, CFG>(a, sh, sm.rs, tid, kPlainThreads, sm.abort != 0);
     return;
   }
   finish_block<T, CFG, kPlainThreads, false>(a, sh, sm.rs, tid, sm.abort != 0, &sm.ring[0][0][0], kPlainRingBytes,
@@ -1487,6 +1505,7 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   constexpr int kListCap = kTopkWarps * WL;
   Smem& sm = *reinterpret_cast<Smem*>(fused_smem_raw);
 
+  call_enter(a.ordered, a.signal != 0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const FinishArgs& f = a.fin;
   const int V = f.V;
@@ -1962,7 +1981,7 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   // ================================= phase 2 ===========================================
   __syncthreads();
   if (stats_only) {
-    write_row_stats(a, sh, sm.rs, tid, kTopkThreads, sm.abort != 0);
+    write_row_stats<T, CFG>(a, sh, sm.rs, tid, kTopkThreads, sm.abort != 0);
     return;
   }
   static_assert(sizeof(sm.list) >= kFinTiles * sizeof(double), "tile sums live in the list area");
