@@ -231,8 +231,8 @@ int csd_verify_ex(const csd_params* p);
  * (any target_rows, guidance and top-k setting).  0 if the sizes are invalid. */
 size_t csd_workspace_size(int B, int gamma, int V, int dtype);
 
-/* Number of kernels csd_verify_ex(p) would enqueue (1 on the fused path; 2, or 3 with
- * top-k, on the path for unaligned or very small rows), or a negative csd_error.
+/* Number of kernels csd_verify_ex(p) would enqueue (1 on the single-launch paths; 2, or 3 with
+ * top-k, for rows of fewer than 512 tokens or bytes that those do not take), or a negative csd_error.
  * Validates like csd_verify_ex and enqueues nothing. */
 int csd_launch_count(const csd_params* p);
 
@@ -252,7 +252,9 @@ int csd_workspace_init(void* workspace, size_t workspace_bytes, void* stream);
  * and for its workspace.  The call enqueues host->device copies, the kernels and
  * device->host copies of out_tokens / out_accept_len / out_status (and any
  * diagnostics requested) on host->stream and returns; results are in the host
- * arrays once the stream has been synchronised.
+ * arrays once the stream has been synchronised.  Where the small arrays are pinned
+ * (mapped) memory the kernels read and write them there instead of through copies:
+ * as with any asynchronous copy they stay the call's until then.
  */
 int csd_verify_host(const csd_params* host, void* staging, size_t staging_bytes);
 size_t csd_host_staging_size(const csd_params* host);

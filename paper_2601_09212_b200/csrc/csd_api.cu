@@ -237,6 +237,13 @@ cudaError_t launch_finish(const FinishArgs& a_in, cudaStream_t stream) {
 long long g_wait_limit = kWaitCycles;
 int g_drop_first_copy = 0;
 
+// Rows of the busiest of c blocks that share a sequence's positions (see block_share).
+int busiest_rows(int gamma, int T, int c) {
+  if (c <= 1) return T + gamma;
+  const int most = 2 * ((gamma + c - 1) / c), last = 2 * (gamma / c) + (T > gamma ? 1 : 0);
+  return most > last ? most : last;
+}
+
 // Into how many blocks the position split cuts a sequence in stream order: powers of two while there are at most two
 // blocks to an SM (with top-k, whose per-row work is longer, four), and without top-k once more if the clusters then fit
 // the three blocks an SM holds with room to spare and the busiest SM has at least a seventh fewer rows.  us per call
@@ -247,7 +254,7 @@ int position_split(int B, int gamma, int T, bool topk, int sms) {
   int c = 1;
   while (2 * c <= (topk ? 4 : 2) * sms / B && 2 * c <= gamma && 2 * c <= kMaxCluster) c *= 2;
   if (topk || 2 * c > gamma || 2 * c > kMaxCluster || 2LL * c * B * 4 > 11LL * sms) return c;
-  auto load = [&](int n) { return ((B * n + sms - 1) / sms) * (2 * ((gamma + n - 1) / n) + (T > gamma ? 1 : 0)); };
+  auto load = [&](int n) { return ((B * n + sms - 1) / sms) * busiest_rows(gamma, T, n); };
   return load(2 * c) * 7 <= load(c) * 6 ? 2 * c : c;
 }
 
@@ -440,7 +447,7 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   const bool tree = in.N > 0;
   const int pos = position_split(B, gamma, in.fa.T, in.topk, in.sms);
   if (in.fa.vec_ok && !tree && (long long)B * pos > in.sms) return cudaSuccess;
-  const int rows = pos > 1 ? 2 * ((gamma + pos - 1) / pos) + (in.fa.T > gamma ? 1 : 0) : in.fa.T + gamma;
+  const int rows = busiest_rows(gamma, in.fa.T, pos);
   const double logits = (double)rows * in.fa.V;
   // (a tree: the statistics of all rows, then the walk by one block per sequence)
   const double other_ns = tree ? ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms)
@@ -558,7 +565,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
       // (its items are a contiguous eighth of the block's items; an item costs its stages plus about
       // half a stage of fixed work).  Long items are better for their own sake -- fewer changes of
       // the running maximum, fewer reductions -- so ties go to the fewer parts.
-      const long long rows_b = (c > 1) ? (2LL * ((in.gamma + c - 1) / c) + 1) : spc * rows_per_seq;
+      const long long rows_b = (c > 1) ? busiest_rows(in.gamma, in.fa.T, (int)c) : spc * rows_per_seq;
       long long cpp = cpr;
       double best = -1.0;
       for (long long np = 1; np <= 16 && np <= cpr; ++np) {
@@ -582,7 +589,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
       // a block keeps one stash entry per item
       for (;;) {
         const long long parts = (cpr + cpp - 1) / cpp;
-        const long long rows_block = (c > 1) ? (2LL * ((in.gamma + c - 1) / c) + 1) : spc * rows_per_seq;
+        const long long rows_block = (c > 1) ? busiest_rows(in.gamma, in.fa.T, (int)c) : spc * rows_per_seq;
         if (rows_block * parts <= kBlockStash) break;
         if (cpp < cpr) cpp = (cpp * 2 < cpr) ? cpp * 2 : cpr;
         else if (spc > 1) --spc;

@@ -222,8 +222,10 @@ __device__ __forceinline__ BlockShare block_share(const FusedArgs& a) {
     const int j = blockIdx.x - b * a.ctas_per_seq;
     sh.seq_begin = b;
     sh.seq_end = b + 1;
-    sh.pos_begin = L * j / a.ctas_per_seq;
-    sh.pos_end = L * (j + 1) / a.ctas_per_seq;
+    // (rounded up, so that the last block, which has the bonus row too, is never among those with one position more: ten
+    // positions over four blocks are 6, 4, 6 and 5 rows, and not 4, 6, 4 and 7)
+    sh.pos_begin = (L * j + a.ctas_per_seq - 1) / a.ctas_per_seq;
+    sh.pos_end = (L * (j + 1) + a.ctas_per_seq - 1) / a.ctas_per_seq;
     sh.bonus = (has_bonus_row && j == a.ctas_per_seq - 1) ? 1 : 0;
     sh.slot = j;
   } else {
