@@ -364,12 +364,12 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
 }
 
 // Launches the sliced kernel if it suits the call; *launched says whether it did (with `dry`, whether it would).
-// The split is the one with the least expected time, which where rows are aligned has to be below `other_ns`, what the
-// position split should take.  Expected times are a fixed part for each wave of clusters and a rate over the logits that
-// the busiest SM goes through, fitted to (us per call, sliced / position split):
+// The split is the one with the least expected time, which has to be below `other_ns`, what the path that the call would
+// otherwise take should need.  Expected times are a fixed part for each wave of clusters and a rate over the logits that the
+// busiest SM goes through, fitted to (us per call, sliced / position split):
 //   no top-k: 16 K vocabulary fp32 B=1 gamma=4 8.0 / 12.5, B=14 12.4 / 14.3, B=16 17.6 / 15.2; 64 K bf16 B=4 18.0 / 23.2, fp32
 //   gamma=16 B=1 31.9 / 41.5, B=8 48 / 42; drafting calls of 64 guided rows of 16 K 8.7 / 11.5, 25 of 23 K 8.3 / 13.3;
-//   (the same 64 rows with eight blocks each, two waves: 18.2; 35 rows of 4.3 K 7.0 - 8.0 by one to four blocks, 14.9 by eight);
+//   (the same 64 rows with eight blocks each, two waves: 18.2; 35 rows of 4.3 K 7.0 - 8.0 by one to four, 14.9 by eight);
 //   top-k: guided bf16 top-k 1000 B=4 18.0 / 23.6, B=14 21.8 / 24.8, 64 K top-k 2000 B=4 37.2 / 85.5; drafting calls of 64
 //   rows of 16 K 15.1 / 13.6, 20 of 30 K 13.9 / 20.5; guided 33 K top-k 1823 gamma=13 B=8 (five turns) 73.7 / 63.6.
 template <typename T, bool CFG, bool TOPK, bool TREE>
@@ -383,7 +383,7 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (R > kSliceRows) return cudaSuccess;
-  double best = a.g.vec_ok ? other_ns : 1e30;
+  double best = other_ns;
   SliceGeo geo;
   size_t bytes = 0;
   int best_c = 0;
@@ -391,8 +391,11 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
     if (c > ntiles || (c > 1 && f.V / c < kSliceUnit)) continue;
     int np, upp;   // the work of a block: its busiest warp's, times its warps
     const double logits = (double)slice_rounds(R, (((ntiles + c - 1) / c) * TILE + kSliceUnit - 1) / kSliceUnit, np, upp) * kSliceUnit * kSliceWarps;
+    // (unaligned rows are read from shared memory value by value, and mixed so: 169 guided fp32 sequences of three
+    // positions took 64.9 us sliced and take 50.7 by the scalar kernels)
+    const double rate = (TOPK ? 0.30 : 0.15) * (a.g.vec_ok ? 1.0 : (CFG ? 2.1 : 1.4));
     auto expect = [&](int waves, double per_sm) {
-      return waves * ((TOPK ? 11e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + (TOPK ? 0.30 : 0.15) * per_sm;
+      return waves * ((TOPK ? 11e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + rate * per_sm;
     };
     if (expect(1, logits) >= best) continue;
     // a block to an SM where the clusters fit so, with room for more rows at once; else two
@@ -450,8 +453,18 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   const int rows = busiest_rows(gamma, in.fa.T, pos);
   const double logits = (double)rows * in.fa.V;
   // (a tree: the statistics of all rows, then the walk by one block per sequence)
-  const double other_ns = tree ? ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms)
-                          : in.topk ? (rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 5e3 + 0.5 * logits) : 9e3 + 0.09 * logits;
+  // Unaligned rows otherwise take the scalar kernels of the multi-launch path: three launches' latencies, of which some grow
+  // with the row, and a rate over all logits (us: bf16 of 16 K 5.9 M logits 34.6, 31.5 M 118, two sequences of 61 K 34.9; fp32
+  // of 16 K 24 M 65.5; top-k, bf16: two sequences of 18 K 50.0, 5.9 M of 16 K 80.5).
+  double other_ns;
+  if (tree) other_ns = ((in.topk ? 4.0 : 2.6) * in.fa.V + 300.0 * B) * ((B + in.sms - 1) / in.sms) * (in.fa.vec_ok ? 1.0 : 2.0);
+  else if (!in.fa.vec_ok) {
+    const double all = (double)B * (in.fa.T + gamma) * in.fa.V;
+    other_ns = in.topk ? 25e3 + 1.1 * in.fa.V + 6e-3 * all
+                       : 12e3 + 0.3 * in.fa.V + (in.dtype == CSD_F32 ? 2.0e-3 : 3.0e-3) * (in.cfg ? 1.4 : 1.0) * all;
+  }
+  else if (!in.topk) other_ns = 9e3 + 0.09 * logits;
+  else other_ns = rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 5e3 + 0.5 * logits;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;

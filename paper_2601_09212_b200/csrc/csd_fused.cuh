@@ -696,16 +696,17 @@ __device__ void draw_position(const FusedArgs& ua, const BlockShare& sh, const i
 }
 
 // Emits sequence b from the record of the block that decides it (winner): the accepted prefix, the
-// drawn token, padding; accepted length; status; optionally the distribution drawn from.
+// drawn token, padding; accepted length; status; optionally the distribution drawn from.  `tokens`: the sequence's
+// drafted tokens where this block has staged them all, or null.
 template <typename T, bool CFG, int NT>
 __device__ void emit_sequence(const FusedArgs& ua, const int b, const SeqRecord& win, const int status_any,
-                              const int tid) {
+                              const int tid, const int* tokens) {
   const FinishArgs& a = ua.fin;
   const int L = a.gamma;
   const int tau = win.first_rej >= 0 ? win.first_rej : L;
   if (tid <= L) {
     int v = -1;
-    if (tid < tau) v = __ldcg(&a.tokens[(int64_t)b * L + tid]);
+    if (tid < tau) v = tokens ? tokens[tid] : __ldcg(&a.tokens[(int64_t)b * L + tid]);
     else if (tid == tau) v = win.token;
     a.out_tokens[(int64_t)b * (L + 1) + tid] = v;
   }
@@ -894,7 +895,7 @@ __device__ void finish_block(const FusedArgs& ua, const BlockShare& sh, const Ro
         sticky = (ua.error_flag && __ldcg(ua.error_flag)) ? 8 : 0;
       }
       write_pqf(b);
-      emit_sequence<T, CFG, NT>(ua, b, st.rec, st.rec.status_any | sticky, tid);
+      emit_sequence<T, CFG, NT>(ua, b, st.rec, st.rec.status_any | sticky, tid, st.tok);
       __syncthreads();
     }
     return;
@@ -954,7 +955,7 @@ __device__ void finish_block(const FusedArgs& ua, const BlockShare& sh, const Ro
   pdl_wait();   // the previous call has completed: outputs of consecutive calls stay in order
   if (ua.error_flag && __ldcg(ua.error_flag)) any = 8;
   write_pqf(b);
-  emit_sequence<T, CFG, NT>(ua, b, st.rec, any, tid);
+  emit_sequence<T, CFG, NT>(ua, b, st.rec, any, tid, nullptr);   // (other blocks staged the other positions' tokens)
 }
 
 // Stats-only calls (FusedArgs::stats_out): the block's rows go to global memory in the row order of the
