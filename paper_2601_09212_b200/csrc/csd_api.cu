@@ -338,7 +338,7 @@ bool slice_layout(const SliceArgs& a, int R, int c, size_t room, double tail, Sl
   const size_t scratch = TOPK ? sizeof(SliceSettle) : 0;
   if (TOPK) {
     // values a slice's list expects, with room for a Student-t row of three degrees of freedom: far out its tail beyond a
-    // level found by moments is several times a Gaussian's (1.9 at 1.5 % of the row, 2.9 at 0.8, 5.3 at 0.3)
+    // level found by moments is several times a Gaussian's (1.9 at 1.5 % of the row, 2.8 at 0.8, 5.3 at 0.3)
     const double e = tail * n, room_for = tail < 0.035 ? 1.25 * pow(0.035 / tail, 0.6) : 1.25;
     g.list_cap = ((int)(room_for * e + 6.0 * sqrt(e) + 24.0) + 3) / 4 * 4;
     if (g.list_cap > n) g.list_cap = n;

@@ -117,3 +117,40 @@ def test_topk_slices_on_rows_the_guess_misses(kind):
             t[1, 2, 777] = float("nan")
     rep, _, _ = check(w)
     assert rep.ok, rep.summary()
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=24, gamma=10, V=8192, bonus_row=True),    # ten positions over four blocks: three, two, three, two and the bonus row
+    dict(B=40, gamma=7, V=4096, bonus_row=True), dict(B=40, gamma=7, V=4096),
+    dict(B=100, gamma=12, V=4096), dict(B=100, gamma=12, V=4096, dtype=W.BF16, bonus_row=True),   # doubled to three blocks an SM
+    dict(B=200, gamma=6, V=4104, dtype=W.BF16, bonus_row=True),
+    dict(B=24, gamma=10, V=8192, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=400, bonus_row=True),
+])
+def test_position_split_edges(kw):
+    """Positions that the blocks of a cluster cannot share evenly, and the split's last doubling."""
+    rep, _, _ = check(_make(kw), want_dbg=False)
+    assert rep.ok and rep.tau_mismatch_near + rep.token_mismatch_near <= 1, rep.summary()
+
+
+@pytest.mark.parametrize("B,gamma,V", [(1, 1, 520), (9, 4, 4096), (300, 3, 1024)])
+@pytest.mark.parametrize("pinned", ["inputs", "outputs", "neither", "all"])
+def test_host_form_with_pinned_and_pageable_arrays(pinned, B, gamma, V):
+    """Small inputs are pulled and small outputs written in place where they are pinned, copied where they are not: the
+    same integers.  Outputs begin off a 16-byte boundary, their neighbours stay as they were."""
+    w = _make(dict(B=B, gamma=gamma, V=V, dtype=W.BF16, bonus_row=True), seed=11)
+    got = run_gpu(w, want_dbg=False)
+    pin = lambda t, yes: t.cpu().pin_memory() if yes else t.cpu()
+    ins, outs = pinned in ("inputs", "all"), pinned in ("outputs", "all")
+    sizes = (B * (gamma + 1), B, B)
+    bufs = [pin(torch.full((n + 2,), -7, dtype=torch.int32), outs) for n in sizes]
+    tok, tau, status = (b[1:-1] for b in bufs)
+    args = [pin(w.target_logits, True), pin(w.draft_logits, True), pin(w.draft_tokens, ins), pin(w.uniforms, ins),
+            pin(w.relax_schedule, ins), tok.view(B, gamma + 1), tau]   # (kept: the parameter block holds raw pointers)
+    prm = csd.make_params(*args, out_status=status, host=True)
+    staging = torch.full((csd.csd_host_staging_size(prm),), 255, dtype=torch.uint8, device=DEV)
+    for _ in range(2):
+        csd.csd_verify_host(prm, staging)
+        torch.cuda.synchronize()
+        assert np.array_equal(tok.view(B, gamma + 1).numpy(), got["tokens"])
+        assert np.array_equal(tau.numpy(), got["accept_len"]) and np.array_equal(status.numpy(), got["status"])
+    assert all(b[0] == -7 and b[-1] == -7 for b in bufs)
