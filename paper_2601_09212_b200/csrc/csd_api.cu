@@ -392,7 +392,7 @@ cudaError_t try_slice(SliceArgs& a, double other_ns, double tail, bool dry, cuda
     int np, upp;   // the work of a block: its busiest warp's, times its warps
     const double logits = (double)slice_rounds(R, (((ntiles + c - 1) / c) * TILE + kSliceUnit - 1) / kSliceUnit, np, upp) * kSliceUnit * kSliceWarps;
     // (unaligned rows are read from shared memory value by value, and mixed so: 169 guided fp32 sequences of three
-    // positions took 64.9 us sliced and take 50.7 by the scalar kernels)
+    // positions took 64.9 us sliced and take 51 - 55 by the scalar kernels)
     const double rate = (TOPK ? 0.30 : 0.15) * (a.g.vec_ok ? 1.0 : (CFG ? 2.1 : 1.4));
     auto expect = [&](int waves, double per_sm) {
       return waves * ((TOPK ? 11e3 : 6.4e3) + 80.0 * c + (TREE ? (TOPK ? 17e3 : 8e3) : 0.0)) + rate * per_sm;
