@@ -238,8 +238,8 @@ int csd_verify_ex(const csd_params* p);
  * (any target_rows, guidance and top-k setting).  0 if the sizes are invalid. */
 size_t csd_workspace_size(int B, int gamma, int V, int dtype);
 
-/* Number of kernels csd_verify_ex(p) would enqueue, or a negative csd_error: 1 on the single-launch paths;
- * 2, or 3 with top-k, for rows that those do not take -- fewer than 512 bytes, more than 131072 tokens
+/* Number of kernels csd_verify_ex(p) would enqueue, or a negative csd_error: 1 on the single-launch paths; 2 for large
+ * calls in stream order whose statistics are dealt out evenly over the GPU; 2, or 3 with top-k, for rows that those do not take -- fewer than 512 bytes, more than 131072 tokens
  * (fp32; 262144 bf16) or not aligned, where a split over the vocabulary is not possible or not faster.
  * Validates like csd_verify_ex and enqueues nothing. */
 int csd_launch_count(const csd_params* p);
@@ -466,11 +466,11 @@ int csd_checked_report(int32_t* out_host);
 
 /*
  * Testing aid: which way the calling thread's most recent call took, written to HOST out_host[6]:
- *   [0] 1: its sequences were split over the vocabulary; 2: by positions, or not at all, in one launch;
- *       3: several launches; 0: no call yet, or the latest was refused
- *   [1] thread blocks per sequence (0 with several launches)
+ *   [0] 1: its sequences were split over the vocabulary; 2: by positions, by rows, or not at all; 3: several launches of the
+ *       kernels that take any rows; 0: no call yet, or the latest was refused
+ *   [1] thread blocks per sequence (by rows: those of the second launch, which finishes the sequences; 0 on path 3)
  *   [2] split over the vocabulary: rows of a sequence that a block holds at once; 0 otherwise
- *   [3] ... warps that a row's slice is dealt out to
+ *   [3] ... warps that a row's slice is dealt out to; by rows: pieces that a row may be cut into; 0 otherwise
  *   [4] ... 1 if their results are exchanged as they are, 0 if merged first
  *   [5] rows of a sequence
  * For csd_shard_* it tells of csd_shard_stats.  Returns CSD_OK or CSD_ERR_NULL.

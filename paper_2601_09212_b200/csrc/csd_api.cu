@@ -12,6 +12,7 @@
 #include "../../include/csd.h"
 #include "csd_kernels.cuh"
 #include "csd_fused.cuh"
+#include "csd_flat.cuh"
 #include "csd_slice.cuh"
 #include "csd_tree.cuh"
 #include "csd_shard.cuh"
@@ -27,6 +28,7 @@ static_assert(sizeof(PlainSmem) <= 75 * 1024, "three blocks of the plain kernel 
 constexpr int kMaxV = 1 << 20;
 constexpr int kMaxDevices = 64;
 constexpr size_t kAlign = 256;
+constexpr int kFlatTopkBlocks = 4;   // blocks of the top-k kernel per SM when all rows are dealt out
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 inline int elem_size(int dtype) { return dtype == CSD_F32 ? 4 : 2; }
@@ -107,13 +109,13 @@ bool topk_guess(double k, double v, TopkGuess& g) {
 // Launches one of the single-launch kernels (KERNEL: 0 plain, 1 top-k on rows that are a whole
 // number of stages, 2 top-k on any row length, 3 and 4 the same two with the large candidate lists) with its shared-memory size, as a programmatic
 // dependent launch and, for ctas_per_seq > 1, as clusters of that many blocks.
-template <typename T, bool CFG, int KERNEL>
+template <typename T, bool CFG, int KERNEL, bool DEALT = false>
 cudaError_t launch_fused(const FusedArgs& a, int grid, cudaStream_t stream) {
   auto kern = KERNEL == 0 ? verify_plain_kernel<T, CFG>
-              : KERNEL == 1 ? verify_topk_kernel<T, CFG, false, kWarpList>
-              : KERNEL == 2 ? verify_topk_kernel<T, CFG, true, kWarpList>
-              : KERNEL == 3 ? verify_topk_kernel<T, CFG, false, kWarpListLarge>
-                            : verify_topk_kernel<T, CFG, true, kWarpListLarge>;
+              : KERNEL == 1 ? verify_topk_kernel<T, CFG, false, kWarpList, DEALT>
+              : KERNEL == 2 ? verify_topk_kernel<T, CFG, true, kWarpList, DEALT>
+              : KERNEL == 3 ? verify_topk_kernel<T, CFG, false, kWarpListLarge, DEALT>
+                            : verify_topk_kernel<T, CFG, true, kWarpListLarge, DEALT>;
   constexpr size_t kSmem = KERNEL == 0 ? sizeof(PlainSmem) : (KERNEL <= 2 ? sizeof(TopkSmem) : sizeof(TopkSmemT<kWarpListLarge>));
   constexpr int kThreads = KERNEL ? kTopkThreads : kPlainThreads;
   // the attribute belongs to (function, device): set it once per device (setting it twice is harmless)
@@ -154,6 +156,10 @@ cudaError_t launch_fused_t(const FusedArgs& a, bool topk, int grid, cudaStream_t
   if (!topk) return launch_fused<T, CFG, 0>(a, grid, stream);
   constexpr int kStageElems = kTkStageBytes / ((int)sizeof(T) * (CFG ? 2 : 1));
   const bool whole = a.fin.V % kStageElems == 0;
+  if (a.rows_out) {
+    if (a.large_lists) return whole ? launch_fused<T, CFG, 3, true>(a, grid, stream) : launch_fused<T, CFG, 4, true>(a, grid, stream);
+    return whole ? launch_fused<T, CFG, 1, true>(a, grid, stream) : launch_fused<T, CFG, 2, true>(a, grid, stream);
+  }
   if (a.large_lists) return whole ? launch_fused<T, CFG, 3>(a, grid, stream) : launch_fused<T, CFG, 4>(a, grid, stream);
   return whole ? launch_fused<T, CFG, 1>(a, grid, stream) : launch_fused<T, CFG, 2>(a, grid, stream);
 }
@@ -161,18 +167,25 @@ cudaError_t launch_fused_t(const FusedArgs& a, bool topk, int grid, cudaStream_t
 // A kernel that begins with griddepcontrol.wait, as a programmatic dependent launch: its blocks are resident
 // and set up when the operation before it completes.
 template <typename K, typename A>
-cudaError_t launch_after(K kern, const A& a, unsigned grid, unsigned block, size_t smem, cudaStream_t stream) {
+cudaError_t launch_after(K kern, const A& a, unsigned grid, unsigned block, size_t smem, cudaStream_t stream, int cluster = 1) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (cluster > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
@@ -462,6 +475,7 @@ struct SliceCall {
   bool cfg, topk, exact;   // exact: every row's exact threshold is wanted
   int* error_flag;
   int sms;
+  double dealt_ns = 0.0;   // what the call should take with its rows dealt out; 0: it cannot go that way, or would not
   int N = 0, D = 0;        // N > 0: a tree (fa: gamma = T = N + 1 contexts)
   int32_t* out_nodes = nullptr;
   const int32_t* parent = nullptr;
@@ -489,6 +503,9 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   }
   else if (!in.topk) other_ns = 9e3 + 0.09 * logits;
   else other_ns = rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 5e3 + 0.5 * logits;
+  // (both expectations are off by a sixth, so rows are dealt out instead where that promises a fifth less: of 37 random calls
+  // that would be sliced and have a row for every SM, 27 go so, in 0.52 - 0.98 of the time, all 37 in 0.76 in the mean)
+  if (in.dealt_ns > 0.0 && 1.25 * in.dealt_ns < other_ns) other_ns = 1.25 * in.dealt_ns;
   SliceArgs a;
   memset(&a, 0, sizeof a);
   a.f.fin = in.fa;
@@ -538,6 +555,7 @@ struct FusedPlan {
   cudaStream_t stream;
   float4* records = nullptr;   // with stats_out (see FusedArgs)
   int v_offset = 0;
+  float4* rows_out = nullptr;  // top-k: all rows dealt out (see FusedArgs)
 };
 cudaError_t plan_and_launch_fused(const FusedPlan& in) {
   const int sms = in.sms, es = in.es, rows_per_seq = in.rows_per_seq;
@@ -556,6 +574,8 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     ua.thr_out = in.thr_out;
     ua.records = in.records;
     ua.v_offset = in.v_offset;
+    ua.rows_out = in.rows_out;
+    ua.rows_per_block = 0;
     ua.wait_limit = g_wait_limit;
     ua.drop_first_copy = g_drop_first_copy == 1;
     // Blocks are aligned with sequences and positions.  For calls enqueued back to back a block owns a
@@ -635,7 +655,12 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
       ua.chunks_per_part = (int)cpp;
       ua.parts_per_row = (int)((cpr + cpp - 1) / cpp);
     }
-    const long long grid = c > 1 ? (long long)in.B * c : (in.B + spc - 1) / spc;
+    long long grid = c > 1 ? (long long)in.B * c : (in.B + spc - 1) / spc;
+    if (in.rows_out) {   // one wave of four blocks per SM
+      c = spc = 1;
+      ua.rows_per_block = (int)((in.rows + kFlatTopkBlocks * sms - 1) / (kFlatTopkBlocks * sms));
+      grid = (in.rows + ua.rows_per_block - 1) / ua.rows_per_block;
+    }
     g_plan = Plan{2, (int)c, 0, 0, 0, rows_per_seq};
     ua.ctas_per_seq = (int)c;
     ua.seqs_per_cta = (int)spc;
@@ -645,7 +670,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     // with more, they would fill the SMs that happen to have room and end up unevenly spread (256 sequences of 16
     // positions, 256 blocks: 67.6 us a call without the early signal, 85.8 with it).  A stats-only call is
     // followed by its finishing kernel, whose large blocks would only sit on SMs this kernel needs.
-    ua.signal = (in.stats_out == nullptr && (in.back_to_back || grid <= sms)) ? 1 : 0;
+    ua.signal = (in.rows_out != nullptr || (in.stats_out == nullptr && (in.back_to_back || grid <= sms))) ? 1 : 0;
     if (in.dtype == CSD_F32)
       fe = cfg ? launch_fused_t<float, true>(ua, topk, (int)grid, stream)
                : launch_fused_t<float, false>(ua, topk, (int)grid, stream);
@@ -654,6 +679,105 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
                : launch_fused_t<__nv_bfloat16, false>(ua, topk, (int)grid, stream);
     return fe;
   }
+}
+
+// ---- statistics dealt out evenly, then one cluster per sequence (csd_flat.cuh) ------------------------------------
+template <typename T, bool CFG, bool FILT>
+cudaError_t launch_flat_finish(FlatArgs& a, int sms, cudaStream_t stream) {
+  // two finishing blocks per SM, each warp with a tile at least
+  constexpr int TILE = 32 * Elem<T>::kVec;
+  const FinishArgs& f = a.fin;
+  const int tiles = (f.V + TILE - 1) / TILE;
+  int c = 1;
+  while (2 * c <= kMaxCluster && 2LL * c * f.B <= 2 * sms && tiles >= 2 * c * (kFlatThreads / 32)) c *= 2;
+  a.finish_blocks = c;
+  g_plan = Plan{2, c, 0, f.parts, 0, f.T + f.gamma};
+  return launch_after(flat_finish_kernel<T, CFG, FILT>, a, (unsigned)(f.B * c), kFlatThreads, (size_t)tiles * sizeof(double), stream, c);
+}
+// Whether a call should go that way rather than by the position split (plan_and_launch_fused, c blocks to a sequence).  Expected
+// times in ns: of the split a rate over the logits of the busiest SM and one over those of a block, of this form a rate over
+// the GPU's average and the draw's, and the launch more in its fixed part.  Fitted to 300 random calls on inputs that
+// change from call to call (6 - 256 sequences, 4096 - 65536 tokens; both forms within 4 - 10 %): those that go this way take 0.83
+// of the split's time in the mean; of all calls the rule picks the slower form, by 3 - 5 %, for five of 178.  us, split /
+// dealt out: B=256 gamma=16 heavy-tailed bf16 64.8 / 57.5, B=64 gamma=8 V=16384 fp32 21.6 / 18.4, B=94 gamma=9 V=6832 fp32 20.5 /
+// 15.2, B=173 guided bf16 of 7840 26.0 / 21.5; but B=74 gamma=15 V=9144 fp32, which the split spreads evenly, 24.2 / 31.6.
+struct FlatRate {
+  double split, split_sm, split_block, flat, flat_sm, flat_v;
+};
+constexpr FlatRate kFlatRate[2][2] = {   // [bf16][guidance]
+    {{9.16e3, 0.0647, 0.0467, 10.65e3, 0.1061, 0.0447}, {7.53e3, 0.1140, 0.0984, 10.51e3, 0.1934, 0.0627}},
+    {{10.69e3, 0.0440, 0.0239, 11.70e3, 0.0566, 0.0435}, {11.64e3, 0.0739, 0.0636, 9.88e3, 0.1066, 0.1094}}};
+bool flat_suits(const FusedPlan& in) {
+  const FlatRate& r = kFlatRate[in.dtype == CSD_BF16][in.cfg];
+  const int c = position_split(in.B, in.gamma, in.fa.T, false, in.sms);
+  const double block = (double)busiest_rows(in.gamma, in.fa.T, c) * in.V;
+  const double per_sm = (double)(((long long)in.B * c + in.sms - 1) / in.sms);
+  const double mean = (double)in.rows * in.V / in.sms;
+  return r.flat + r.flat_sm * mean + r.flat_v * in.V < 0.98 * (r.split + r.split_sm * per_sm * block + r.split_block * block);
+}
+// The same with top-k, whose rows are dealt out whole: the rows of the busiest SM and those that one of its blocks takes one after
+// another.  Over 77 random calls (6 - 256 sequences) the calls that go this way took 0.75 of the split's time in the mean, one of
+// them 1.05; those with equal sums 1.02 - 1.18.
+bool flat_suits_topk(const FusedPlan& in) {
+  const int c = position_split(in.B, in.gamma, in.fa.T, true, in.sms);
+  const long long split_each = busiest_rows(in.gamma, in.fa.T, c), split = ((long long)in.B * c + in.sms - 1) / in.sms * split_each;
+  const long long slots = (long long)kFlatTopkBlocks * in.sms, each = (in.rows + slots - 1) / slots, blocks = (in.rows + each - 1) / each;
+  return (blocks + in.sms - 1) / in.sms * each + each < split + split_each;
+}
+
+// What such a call should take, in ns: a fixed part, a rate over the logits that a block takes one after another, one over those of
+// the busiest SM, and a part per row of a block (fitted to 194 random calls, within 11 - 14 %); 0 where that is not known: guided fp32
+// rows, whose sample is half as large, miss their guess too often.
+double flat_topk_ns(const FusedPlan& in) {
+  if (in.dtype == CSD_F32 && in.cfg) return 0.0;
+  const long long slots = (long long)kFlatTopkBlocks * in.sms, each = (in.rows + slots - 1) / slots, blocks = (in.rows + each - 1) / each;
+  const double block = (double)each * in.V, sm = (double)((blocks + in.sms - 1) / in.sms) * block;
+  if (in.dtype == CSD_F32) return 4.8e3 + 0.284 * block + 0.069 * sm + 6.3e3 * each;
+  return in.cfg ? 8.8e3 + 0.167 * block + 0.117 * sm + 3.1e3 * each : 8.4e3 + 0.104 * block + 0.097 * sm + 3.6e3 * each;
+}
+
+// The slots that a row's pieces need in the workspace (top-k: whose rows are not cut, 1); 0 if the call cannot go that way.
+int flat_parts(const FusedPlan& in, size_t max_parts) {
+  if (in.topk) return max_parts >= 2 && in.rows <= (long long)kBlockRows * kFlatTopkBlocks * in.sms ? 1 : 0;   // (16 bytes a row; rows of a block)
+  const int eps = (in.dtype == CSD_F32 ? kFlatStageBytes<float> : kFlatStageBytes<__nv_bfloat16>) / (in.es * (in.cfg ? 2 : 1));
+  const long long spr = (in.V + eps - 1) / eps, least = in.rows * spr / ((long long)kFlatBlocks * in.sms * kPlainWarps);   // stages of a piece
+  if (least < 2) return 0;   // (a copy under the arithmetic of the stage before it; shorter pieces gained nothing)
+  const long long parts = spr < 2 ? 1 : (spr - 2) / least + 2;   // as many as a row can be cut into
+  return parts <= (long long)max_parts ? (int)parts : 0;
+}
+template <typename T, bool CFG>
+cudaError_t launch_flat(const FusedPlan& in, const int parts) {
+  FlatArgs a;
+  memset(&a, 0, sizeof a);
+  a.fin = in.fa;
+  a.error_flag = in.error_flag;
+  a.wait_limit = g_wait_limit;
+  a.drop_first_copy = g_drop_first_copy == 1;
+  if (in.topk) {
+    FusedPlan fp = in;
+    a.fin.parts = 1;
+    fp.rows_out = reinterpret_cast<float4*>(const_cast<float2*>(in.fa.partials));
+    a.rows = fp.rows_out;
+    const cudaError_t e = plan_and_launch_fused(fp);
+    return e == cudaSuccess ? launch_flat_finish<T, CFG, true>(a, in.sms, in.stream) : e;
+  }
+  constexpr int EPS = StageStats<T, CFG, kFlatStageBytes<T>>::EPS;
+  a.stages_per_row = (in.V + EPS - 1) / EPS;
+  a.stages = in.rows * a.stages_per_row;
+  const int grid = kFlatBlocks * in.sms;
+  a.warps = grid * kPlainWarps;
+  a.fin.parts = parts;
+  a.partials = const_cast<float2*>(in.fa.partials);
+  static bool configured[kMaxDevices] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!configured[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(flat_stats_kernel<T, CFG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FlatSmem<T>));
+    if (e != cudaSuccess) return e;
+    configured[dev] = true;
+  }
+  const cudaError_t e = launch_after(flat_stats_kernel<T, CFG>, a, (unsigned)grid, kPlainThreads, sizeof(FlatSmem<T>), in.stream);
+  return e == cudaSuccess ? launch_flat_finish<T, CFG, false>(a, in.sms, in.stream) : e;
 }
 
 // sampling: the degenerate round used by csd_sample_rows -- no draft positions (gamma = 0), one
@@ -762,6 +886,19 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
   // statistics still come from the streaming kernels (one launch, every logit read once)
   const bool stream_stats = !fused && similar.nbr != nullptr && !no_workspace && vec_ok && (size_t)p.V * es >= 512 &&
                             (p.V + 32 * vw - 1) / (32 * vw) <= kFinTiles;
+  FusedPlan fp;
+  fp.fa = fa;
+  fp.B = p.B; fp.gamma = p.gamma; fp.V = p.V; fp.top_k = p.top_k; fp.dtype = p.dtype;
+  fp.rows_per_seq = rows_per_seq; fp.rows = rows; fp.sms = sms; fp.es = es;
+  fp.cfg = cfg; fp.topk = topk; fp.back_to_back = p.back_to_back != 0;
+  fp.allow_short_cut = !p.dbg_G && !p.diag_accept_mass && !p.diag_bound_term;
+  fp.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
+  fp.stats_out = nullptr; fp.thr_out = nullptr;
+  fp.stream = stream;
+  // ---- stream order, many rows: statistics dealt out evenly, where that is expected to be faster
+  int parts = 0;
+  if (fused && !no_workspace && !p.back_to_back && p.gamma > 0 && !p.diag_accept_mass && !p.diag_bound_term && (topk ? flat_suits_topk(fp) : flat_suits(fp)))
+    parts = flat_parts(fp, lay.max_parts);
   // ---- stream order, few sequences or unaligned rows: the vocabulary-sliced kernel -----------------------------
   bool sliced = false;
   if (similar.nbr == nullptr && !p.diag_accept_mass && !p.diag_bound_term && (!fused || !p.back_to_back) && p.V >= 512) {
@@ -770,42 +907,33 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
     sc.dtype = p.dtype; sc.top_k = p.top_k; sc.cfg = cfg; sc.topk = topk; sc.exact = p.dbg_G != nullptr;
     sc.sms = sms;
     sc.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
+    if (topk && parts && rows >= sms) sc.dealt_ns = flat_topk_ns(fp);
     const cudaError_t e = slice_call(sc, plan_only != nullptr, stream, &sliced);
     if (e != cudaSuccess) return CSD_ERR_LAUNCH;
     if (sliced && !plan_only) return CSD_OK;
   }
   if (plan_only) {  // number of kernels this call would enqueue
-    *plan_only = (fused || sliced) ? 1 : (stream_stats ? 2 : (topk ? 3 : 2));
+    *plan_only = sliced ? 1 : fused ? (parts ? 2 : 1) : (stream_stats ? 2 : (topk ? 3 : 2));
     return CSD_OK;
   }
   if (fused) {
-    FusedPlan fp;
-    fp.fa = fa;
-    fp.B = p.B; fp.gamma = p.gamma; fp.V = p.V; fp.top_k = p.top_k; fp.dtype = p.dtype;
-    fp.rows_per_seq = rows_per_seq; fp.rows = rows; fp.sms = sms; fp.es = es;
-    fp.cfg = cfg; fp.topk = topk; fp.back_to_back = p.back_to_back != 0;
-    fp.allow_short_cut = !p.dbg_G && !p.diag_accept_mass && !p.diag_bound_term;
-    fp.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
-    fp.stats_out = nullptr; fp.thr_out = nullptr;
-    fp.stream = stream;
-    return plan_and_launch_fused(fp) == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
+    cudaError_t e;
+    if (!parts) e = plan_and_launch_fused(fp);
+    else if (p.dtype == CSD_F32) e = cfg ? launch_flat<float, true>(fp, parts) : launch_flat<float, false>(fp, parts);
+    else e = cfg ? launch_flat<__nv_bfloat16, true>(fp, parts) : launch_flat<__nv_bfloat16, false>(fp, parts);
+    return e == cudaSuccess ? CSD_OK : CSD_ERR_LAUNCH;
   }
 
   cudaError_t e = cudaSuccess;
   const Plan several{3, 0, 0, 0, 0, rows_per_seq};
   g_plan = several;
   if (stream_stats) {
-    FusedPlan fp;
     fa.parts = 1;
     fp.fa = fa;
-    fp.B = p.B; fp.gamma = p.gamma; fp.V = p.V; fp.top_k = p.top_k; fp.dtype = p.dtype;
-    fp.rows_per_seq = rows_per_seq; fp.rows = rows; fp.sms = sms; fp.es = es;
-    fp.cfg = cfg; fp.topk = topk; fp.back_to_back = false;
+    fp.back_to_back = false;
     fp.allow_short_cut = false;   // the finishing kernel filters by the exact threshold
-    fp.error_flag = reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
     fp.stats_out = sa.partials;
     fp.thr_out = topk ? se.thresholds : nullptr;
-    fp.stream = stream;
     e = plan_and_launch_fused(fp);
     g_plan = several;
     if (e == cudaSuccess) {

@@ -1,0 +1,371 @@
+// Large calls in stream order (sm_100a): row statistics dealt out evenly over the GPU, then one cluster per sequence.
+//
+// The single launch of csd_fused.cuh aligns its blocks with sequences, so a call that runs alone ends with its busiest
+// SM: 256 sequences on 148 SMs leave two blocks on 108 of them and one on 40.  Here the stages of all rows form one list
+// that is cut into as many equal pieces as warps are resident (flat_stats_kernel, one wave of three blocks per SM); with top-k
+// whole rows are dealt out to one wave of verify_topk_kernel's blocks.  A row's pieces are merged by the kernel that finishes its
+// sequence (flat_finish_kernel), which is resident and has fetched its small inputs when the last statistics arrive.
+// us a call before and after, on inputs that change from call to call: 256 sequences of 16 positions, 16 K heavy-tailed bf16 65.0
+// and 58.3 (of which the statistics 51, instruction issue at 5.3 TB/s, the finish 7); 64 of 8, 16 K guided bf16 with top-k 1000 36.3 and
+// 31.2; 173 guided bf16 of 7.8 K 26.0 and 21.5.
+#pragma once
+#include "csd_fused.cuh"
+
+namespace csd {
+
+constexpr int kFlatStages = 2;
+// bytes of a warp's stage: fp32 rows 4 KB (B=64 gamma=8 V=16384 18.3 us a call, 18.8 with 3 KB), bf16 rows, whose values wait
+// packed in registers, 3 KB (B=256 gamma=16 57.5 us, 60.0 with 4 KB)
+template <typename T> constexpr int kFlatStageBytes = sizeof(T) == 4 ? 4096 : 3072;
+// blocks per SM: three (with four, of 64 registers a thread, B=256 64 K fp32 211 -> 243 us, guided 22 K 96 -> 133; two: heavy-tailed bf16 58 -> 74)
+constexpr int kFlatBlocks = 3;
+
+struct FlatArgs {
+  FinishArgs fin;        // (partials: of one row `fin.parts` slots, rows in the order of finish_kernel)
+  const float4* rows;    // top-k: rows' results (see FusedArgs::rows_out), in the same order
+  int stages_per_row;
+  int warps;             // of the whole grid
+  long long stages;      // of all rows
+  float2* partials;
+  int* error_flag;       // set when a bounded wait gave up
+  long long wait_limit;
+  int drop_first_copy;   // (test aid, see FusedArgs)
+  int finish_blocks;     // blocks that share a sequence's draw: one cluster
+};
+
+// first stage of warp w's piece, and the warp whose piece holds stage g
+__host__ __device__ inline long long flat_begin(const long long stages, const int warps, const int w) { return stages * w / warps; }
+__host__ __device__ inline int flat_owner(const long long stages, const int warps, const long long g) {
+  return (int)(((g + 1) * warps - 1) / stages);
+}
+
+template <typename T>
+struct FlatSmem {
+  alignas(128) unsigned char ring[kPlainWarps][kFlatStages][kFlatStageBytes<T>];
+  alignas(8) uint64_t full[kPlainWarps][kFlatStages];
+};
+
+template <typename T, bool CFG>
+__global__ void __launch_bounds__(kPlainThreads, kFlatBlocks) flat_stats_kernel(const FlatArgs a) {
+  constexpr int ARR = CFG ? 2 : 1;
+  constexpr int EPS = StageStats<T, CFG, kFlatStageBytes<T>>::EPS;
+  extern __shared__ __align__(128) unsigned char fused_smem_raw[];
+  FlatSmem<T>& sm = *reinterpret_cast<FlatSmem<T>*>(fused_smem_raw);
+  const FinishArgs& f = a.fin;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int V = f.V, spr = a.stages_per_row, rows_per_seq = f.T + f.gamma;
+  if (lane == 0) {
+    for (int s = 0; s < kFlatStages; ++s) mbar_init(&sm.full[warp][s], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  pdl_wait();
+  // the finishing kernel's blocks take the places that this kernel's leave (the grid is one wave), and the operation ahead
+  // of this call has completed: they may read its results
+  pdl_launch_dependents();
+
+  const int w = blockIdx.x * kPlainWarps + warp;
+  const long long g0 = flat_begin(a.stages, a.warps, w), g1 = flat_begin(a.stages, a.warps, w + 1);
+  const int row0 = (int)(g0 / spr), first = (int)(g0 - (long long)row0 * spr);
+  const int count = (int)(g1 - g0);   // stages of this warp
+  auto row_at_id = [&](const int row_id) {
+    const int b = row_id / rows_per_seq, r = row_id - b * rows_per_seq;
+    return row_at<T, CFG>(f, b, r < f.T ? 0 : 1, r < f.T ? r : r - f.T);
+  };
+
+  // producer cursor (meaningful in lane 0): the next stage to copy
+  int p_row = row0, p_st = first, p_s = 0, p_count = 0;
+  const T *p_cond = nullptr, *p_uncond = nullptr;
+  bool drop_next = a.drop_first_copy != 0 && w == 0;
+  auto open_row = [&]() {
+    const Row<T, CFG> row = row_at_id(p_row);
+    p_cond = row.cond;
+    p_uncond = row.uncond;
+  };
+  auto issue = [&]() {
+    if (p_count == count) return;
+    const int x = p_st * EPS;
+    const uint32_t bytes = (uint32_t)(min(EPS, V - x) * (int)sizeof(T));
+    mbar_expect_tx(&sm.full[warp][p_s], bytes * ARR);
+    if (!drop_next) {
+      bulk_load_row(&sm.ring[warp][p_s][0], p_cond, x, bytes, V, &sm.full[warp][p_s]);
+      if (CFG) bulk_load_row(&sm.ring[warp][p_s][kFlatStageBytes<T> / 2], p_uncond, x, bytes, V, &sm.full[warp][p_s]);
+    }
+    drop_next = false;
+    p_s = p_s + 1 == kFlatStages ? 0 : p_s + 1;
+    if (++p_st == spr) {
+      p_st = 0;
+      ++p_row;
+      if (p_count + 1 < count) open_row();
+    }
+    ++p_count;
+  };
+  if (lane == 0 && count > 0) {
+    open_row();
+    for (int s = 0; s < kFlatStages; ++s) issue();
+  }
+
+  int c_s = 0, waited = 0, done = 0, st = first, row = row0;
+  uint32_t c_par = 0;
+  bool ok = true;   // false once a wait has run out: from then on nothing is waited for or issued
+  while (done < count) {
+    StageStats<T, CFG, kFlatStageBytes<T>> run;
+    run.begin();
+    const int st0 = st, st1 = min(spr, st + count - done);
+    for (; st < st1; ++st) {
+      if (ok) {
+        if (mbar_wait(&sm.full[warp][c_s], c_par, a.wait_limit)) ++waited; else ok = false;
+      }
+      typename StageStats<T, CFG, kFlatStageBytes<T>>::Values values;
+      run.load(values, &sm.ring[warp][c_s][0], min(EPS, V - st * EPS), f.cfg_scale, lane);
+      if (lane == 0 && ok) {   // every lane has read the stage: refill it with the one kFlatStages ahead
+        fence_before_bulk();
+        issue();
+      }
+      run.add(values);
+      if (++c_s == kFlatStages) { c_s = 0; c_par ^= 1u; }
+    }
+    done += st1 - st0;
+    const float2 v = run.end();
+    // the row's slots are numbered by the warps that share it; whoever has its first stage fills those that nobody has
+    const long long start = (long long)row * spr;
+    const int w0 = flat_owner(a.stages, a.warps, start);
+    float2* const slots = a.partials + (long long)row * f.parts;
+    if (lane == 0) slots[w - w0] = ok ? v : make_float2(__int_as_float(0x7fc00000), 0.0f);   // (reads as unusable)
+    if (st0 == 0) {
+      const int used = flat_owner(a.stages, a.warps, start + spr - 1) - w0 + 1;
+      for (int q = used + lane; q < f.parts; q += 32) slots[q] = make_float2(CSD_NEG_INF, -1.0f);
+    }
+    st = 0;
+    ++row;
+  }
+  if (!ok && lane == 0) {
+    if (a.error_flag) atomicExch(a.error_flag, 1);
+    // copies that may still be in flight: those of stages [waited, p_count), at most one per slot of the ring
+    for (int c = waited; c < p_count; ++c)
+      (void)mbar_wait(&sm.full[warp][c % kFlatStages], (uint32_t)(c / kFlatStages) & 1u, a.wait_limit);
+  }
+}
+
+constexpr int kFlatThreads = 512;   // two blocks per SM
+constexpr int kFlatRows = 2 * kMaxGamma + 1;
+
+struct FlatFinishSmem {
+  float2 ms[kFlatRows];      // rows in the order of the partials
+  float tokz[kFlatRows], thr[kFlatRows];
+  int tok[kMaxGamma];
+  float uni[kMaxGamma + 1], omega[kMaxGamma];
+  double zs[2][kMaxCluster];   // by attempt: its total over each block's tiles
+  FinishSmem fin;
+};
+
+// Bound by the latency of a chain: the statistics' end, a trip to L2 for the rows' results, one for the draw's rows, the cluster's
+// exchange, the pick.  Where the sequences leave the GPU idle, 2, 4 or 8 blocks share one: each knows all its rows' statistics, takes all accept tests
+// and sums its range of the draw's tiles; the totals go round, and the block whose range holds the crossing picks the
+// token and emits.
+
+template <typename T, bool CFG, bool FILT>
+__global__ void __launch_bounds__(kFlatThreads, 2) flat_finish_kernel(const FlatArgs a) {
+  constexpr int VEC = Elem<T>::kVec;
+  constexpr int TILE = 32 * VEC;
+  extern __shared__ double tile_sums[];   // one fp64 sum per tile
+  __shared__ FlatFinishSmem sm;
+  const FinishArgs& f = a.fin;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c = a.finish_blocks, b = blockIdx.x / c, me = blockIdx.x - b * c;
+  const int L = f.gamma, T_ = f.T, R = T_ + L, V = f.V;
+  const int ntiles = (V + TILE - 1) / TILE;
+  const int tile_begin = (int)((long long)ntiles * me / c), tiles = (int)((long long)ntiles * (me + 1) / c) - tile_begin;
+  if (c > 1) cluster_arrive();   // first half; waited for before the first store to a peer
+  // ---- the small inputs and the drafted tokens' logits, while the statistics are still coming in (through L2: L1 may hold
+  // what an earlier kernel read there)
+  if (tid <= L) sm.uni[tid] = __ldcg(&f.uniforms[(int64_t)b * (L + 1) + tid]);
+  if (tid < L) {
+    const float om = __ldcg(&f.schedule[tid]);
+    sm.omega[tid] = om >= 0.0f ? om : 0.0f;
+  }
+  if (FILT) {
+    if (tid < L) sm.tok[tid] = __ldcg(&f.tokens[(int64_t)b * L + tid]);
+  } else if (tid < 2 * L) {
+    const int i = tid >> 1, which = tid & 1;
+    const int tok = __ldcg(&f.tokens[(int64_t)b * L + i]);
+    if (which == 0) sm.tok[i] = tok;
+    sm.tokz[which == 0 ? i : T_ + i] = tok >= 0 && tok < V ? row_at<T, CFG>(f, b, which, i).load_one_l2(tok) : 0.0f;
+  }
+  if (c > 1) cluster_wait();
+  pdl_wait();
+  pdl_launch_dependents();
+  if (FILT && tid < R) {
+    const float4 v = __ldcg(a.rows + (int64_t)b * R + tid);
+    sm.ms[tid] = make_float2(v.x, v.y);
+    sm.thr[tid] = v.z;
+    sm.tokz[tid] = v.w < v.z ? CSD_NEG_INF : v.w;
+  } else if (!FILT && tid < R) {
+    const float2* const slots = f.partials + ((int64_t)b * R + tid) * f.parts;
+    float m = CSD_NEG_INF, s = -1.0f;
+    for (int p = 0; p < f.parts; ++p) {
+      const float2 v = __ldcg(slots + p);
+      stat_merge(m, s, v.x, v.y);
+    }
+    sm.ms[tid] = make_float2(m, s);
+  }
+  const int lost = a.error_flag ? __ldcg(a.error_flag) : 0;
+  __syncthreads();
+  // ---- Eq. relax and the accept tests: every warp takes them all, one position per lane
+  auto usable = [](const float2 v) { return v.x > CSD_NEG_INF && v.x < CSD_POS_INF && v.y >= 0.0f && v.y < CSD_POS_INF; };
+  bool acc = true;
+  int flag = 0;
+  if (lane < L) {
+    const float2 t = sm.ms[lane], d = sm.ms[T_ + lane];
+    const int tok = sm.tok[lane];
+    float fa = 0.0f, p = __int_as_float(0x7fc00000), q = p;
+    if (!usable(t) || !usable(d)) flag = 1;
+    else if (tok < 0 || tok >= V) flag = 2;
+    else {
+      const float dt = sm.tokz[lane] - t.x, dd = sm.tokz[T_ + lane] - d.x;
+      p = ex2f(dt * kLog2e) / (1.0f + t.y);
+      q = ex2f(dd * kLog2e) / (1.0f + d.y);
+      if (dd == CSD_NEG_INF) fa = 1.0f;         // q = 0: p/q = +inf, and 0/0 := 1
+      else if (dt == CSD_NEG_INF) fa = 0.0f;    // p = 0 < q
+      else fa = fminf(1.0f, sm.omega[lane] * ex2f((dt - dd) * kLog2e) * ((1.0f + d.y) / (1.0f + t.y)));
+    }
+    acc = sm.uni[lane] <= fa;
+    if (warp == 0 && me == 0) {
+      if (f.dbg_p) f.dbg_p[(int64_t)b * L + lane] = p;
+      if (f.dbg_q) f.dbg_q[(int64_t)b * L + lane] = q;
+      if (f.dbg_f) f.dbg_f[(int64_t)b * L + lane] = fa;
+    }
+  }
+  const unsigned rej = __ballot_sync(0xffffffffu, !acc);
+  const int j = rej ? __ffs(rej) - 1 : L, tau = j;   // the for/break of Algorithm 1
+  int status = lost ? 8 : 0, token = -1;
+  bool draw = false;
+  PairCtx ctx;
+  ctx.mode = 1;
+  if (j < L) {
+    status |= __shfl_sync(0xffffffffu, flag, j);
+    draw = usable(sm.ms[j]);
+    ctx.mode = usable(sm.ms[T_ + j]) ? 0 : 1;
+  } else if (T_ == L + 1) {
+    draw = usable(sm.ms[L]);
+    if (!draw) status |= 1;
+  }
+  // ---- Eq. opt_G (or P), one sum per tile of this block; the crossing's tile; the token in it
+  double Z = 0.0;
+  int owner = 0;   // the block that emits
+  if (draw) {
+    ctx.Mt = sm.ms[j].x; ctx.St = sm.ms[j].y;
+    ctx.Md = j < L ? sm.ms[T_ + j].x : 0.0f; ctx.Sd = j < L ? sm.ms[T_ + j].y : 0.0f;
+    ctx.inv_t = 1.0f / (1.0f + ctx.St);
+    ctx.inv_den = ctx.inv_t / (1.0f + ctx.Sd);
+    ctx.one_minus_omega = 1.0f - (j < L ? sm.omega[j] : 0.0f);
+    Row<T, CFG> rt = row_at<T, CFG>(f, b, 0, j), rd = j < L ? row_at<T, CFG>(f, b, 1, j) : rt;
+    if (FILT) { rt.thr = sm.thr[j]; rd.thr = sm.thr[j < L ? T_ + j : j]; }
+    auto load = [&](const int x0, float (&zt)[VEC], float (&zd)[VEC]) {   // filtered; a drafter's row that is not used reads 0
+      rt.load_tile(x0, V, 1, zt);
+      if (ctx.mode == 0) rd.load_tile(x0, V, 1, zd);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        if (FILT) zt[e] = rt.filter(zt[e]);
+        zd[e] = ctx.mode == 0 ? (FILT ? rd.filter(zd[e]) : zd[e]) : 0.0f;
+      }
+    };
+    const float u = sm.uni[L];
+    for (int attempt = 0; attempt < 2; ++attempt) {
+      constexpr int UNR = (sizeof(T) == 4 ? 4 : 2) / (CFG ? 2 : 1);   // all loads of a trip ahead of its arithmetic
+      for (int t0 = warp; t0 < tiles; t0 += UNR * (kFlatThreads / 32)) {
+        float zt[UNR][VEC], zd[UNR][VEC];
+#pragma unroll
+        for (int r = 0; r < UNR; ++r) {
+          const int t = t0 + r * (kFlatThreads / 32), x0 = t < tiles ? (tile_begin + t) * TILE + lane * VEC : V;
+          load(x0, zt[r], zd[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < UNR; ++r) {
+          const int t = t0 + r * (kFlatThreads / 32);
+          float sum = 0.0f;
+#pragma unroll
+          for (int e = 0; e < VEC; e += 2) {
+            float w0, w1;
+            weight_of_pair(zt[r][e], zt[r][e + 1], zd[r][e], zd[r][e + 1], ctx, w0, w1);
+            sum += w0;
+            sum += w1;
+          }
+#pragma unroll
+          for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+          if (lane == 0 && t < tiles) tile_sums[t] = (double)sum;
+        }
+      }
+      __syncthreads();
+      if (warp == 0) {
+        double mine = 0.0;
+        for (int t = lane; t < tiles; t += 32) mine += tile_sums[t];
+        mine = warp_sum_double(mine);
+        if (lane < c) cluster_store_f64(&sm.zs[attempt][me], (uint32_t)lane, mine);
+      }
+      if (c > 1) { cluster_arrive(); cluster_wait(); }
+      else __syncthreads();
+      double before = 0.0, first = 0.0, last = 0.0;   // running totals ahead of the owner / of the last block with mass
+      int has = -1, cross = -1;
+      Z = 0.0;
+      for (int q = 0; q < c; ++q) Z += sm.zs[attempt][q];
+      const double target = (double)u * Z;
+      for (int q = 0; q < c; ++q) {   // the first block whose running total passes the target; if rounding leaves none, the last with mass
+        const double zq = sm.zs[attempt][q];
+        if (zq > 0.0) { has = q; last = before; }
+        if (cross < 0 && zq > 0.0 && before + zq > target) { cross = q; first = before; }
+        before += zq;
+      }
+      if (Z > 0.0 && Z < (double)CSD_POS_INF) {
+        owner = cross >= 0 ? cross : has;
+        if (owner == me) {
+          if (warp == 0) {
+            const double target_here = target - (cross >= 0 ? first : last);
+            locate_crossing_tile(tile_sums, tiles, u, lane, sm.fin, &target_here);
+            __syncwarp();
+            int tok = -1;
+            if (sm.fin.pick_tile >= 0) {
+              const int x0 = (tile_begin + sm.fin.pick_tile) * TILE + lane * VEC;
+              float zt[VEC], zd[VEC], g[VEC];
+              load(x0, zt, zd);
+#pragma unroll
+              for (int e = 0; e < VEC; ++e) g[e] = weight_of(zt[e], zd[e], ctx);
+              tok = pick_in_tile<VEC>(g, x0, sm.fin.pick_prefix, target_here, lane);
+            }
+            if (lane == 0) sm.fin.token = tok;
+          }
+          __syncthreads();
+          token = sm.fin.token;
+        }
+        break;
+      }
+      Z = 0.0;
+      if (attempt == 1 || ctx.mode == 1) break;   // nothing to draw from
+      ctx.mode = 1;   // empty positive part: fall back to G := P_j
+      status |= 4;
+      __syncthreads();
+    }
+    if (f.dbg_G && Z > 0.0) {   // each block writes its range
+      const float invZ = (float)(1.0 / Z);
+      for (int t = warp; t < tiles; t += kFlatThreads / 32) {
+        const int x0 = (tile_begin + t) * TILE + lane * VEC;
+        float zt[VEC], zd[VEC];
+        load(x0, zt, zd);
+#pragma unroll
+        for (int e = 0; e < VEC; ++e)
+          if (x0 + e < V) f.dbg_G[(int64_t)b * V + x0 + e] = weight_of(zt[e], zd[e], ctx) * invZ;
+      }
+    }
+  }
+  if (f.dbg_G && !(Z > 0.0))
+    for (int x = tile_begin * TILE + tid; x < min(V, (tile_begin + tiles) * TILE); x += kFlatThreads) f.dbg_G[(int64_t)b * V + x] = 0.0f;
+  if (owner != me) return;
+  // ---- emit x_{1:tau+1}
+  if (tid <= L) f.out_tokens[(int64_t)b * (L + 1) + tid] = tid < tau ? sm.tok[tid] : (tid == tau ? token : -1);
+  if (tid == 0) {
+    if (f.out_accept_len) f.out_accept_len[b] = tau;
+    if (f.out_status) f.out_status[b] = status;
+  }
+}
+
+}  // namespace csd

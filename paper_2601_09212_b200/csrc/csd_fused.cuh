@@ -192,6 +192,8 @@ struct FusedArgs {
   float4* records;      // with stats_out, not null: (m, s, logit of the drafted token if this slice holds it) instead,
   int v_offset;         //   for a slice of the vocabulary that begins at this token
   float* thr_out;       //   and its top-k threshold there (may be null), at row b * (T + gamma) + (target ? i : T + i)
+  float4* rows_out;     // top-k, not null: the rows of all sequences are dealt out to the blocks, rows_per_block each; stop after the
+  int rows_per_block;   //   streaming phase and write (m, s, threshold, logit of the drafted token or -inf if it is dropped) here
   int ordered;          // ordinary stream order: nothing of the call's inputs is read before everything ahead of it
                         // on the stream has completed
   int signal;           // let the next call's blocks in as soon as this call's have started (set by the host)
@@ -282,10 +284,10 @@ struct RowStats {
 // The logit of every local row's drafted token, by scalar loads straight from global memory (mixed like
 // the rows), when the kernel starts: the loads are long complete when the row's statistics are.
 template <typename T, bool CFG, int NT>
-__device__ __forceinline__ void load_token_logits(const FinishArgs& f, const BlockShare& sh, const int tid, RowStats& rs) {
+__device__ __forceinline__ void load_token_logits(const FinishArgs& f, const BlockShare& sh, const int tid, RowStats& rs, const int row0 = 0) {
   for (int r = tid; r < sh.n_rows && r < kBlockRows; r += NT) {
     int b, which, i;
-    local_row(sh, r, f.gamma, b, which, i);
+    local_row(sh, row0 + r, f.gamma, b, which, i);
     if (i >= f.gamma) continue;   // the bonus row has no drafted token
     const int tok = __ldcg(&f.tokens[(int64_t)b * f.gamma + i]);
     if (tok >= 0 && tok < f.V) rs.tokz[r] = row_at<T, CFG>(f, b, which, i).load_one(tok);
@@ -998,6 +1000,177 @@ constexpr int kWStageBytes = 3072;
 constexpr int kBlockStash = 1536;   // items (row parts) a block may own
 constexpr int kPlainRingBytes = kPlainWarps * kWStages * kWStageBytes;
 
+// Running statistics of a warp over stages of one row, relative to a maximum that is the same in every lane of
+// the warp: Mw = largest value met so far by any lane, s = this lane's sum of
+// exp(z - Mw) over its values below Mw, cnt = this lane's number of values equal to Mw.
+// Because the reference is warp-uniform, a group of values below it is summed with no
+// test per value, and the exact treatment of values equal to it is a uniform branch
+// taken only where the maximum sits.
+// The exponent (z - Mw) log2(e) is formed by one fused multiply-add, z * log2(e) - MwL with MwL
+// the ROUNDED product Mw * log2(e); its rounding error dlt = Mw * log2(e) - MwL (exact, again by
+// a fused multiply-add) is a common factor 2^dlt of the sum and is divided out once per item.
+// -inf or NaN, and with 0 here its exponential is 0 or NaN as it should be)
+template <typename T, bool CFG, int BYTES>
+struct StageStats {
+  static constexpr int VEC = Elem<T>::kVec;
+  static constexpr int ARR = CFG ? 2 : 1;
+  static constexpr int EPS = BYTES / ((int)sizeof(T) * ARR);   // elements of a row per warp stage
+  static constexpr int VPL = EPS / 32;                                // values per lane per stage
+  static constexpr int NVS = VPL / VEC;                               // 16-byte vectors per lane per stage
+  static_assert(NVS >= 1, "a stage holds at least one vector per lane");
+  float Mw, s_run;
+  float nMwL, dlt;   // -MwL and dlt of the current reference (while Mw is -inf every value is -inf or NaN, and with 0 here
+                     // its exponential is 0 or NaN as it should be)
+  int cnt_run;
+  __device__ __forceinline__ void begin() { Mw = CSD_NEG_INF; s_run = 0.0f; nMwL = 0.0f; dlt = 0.0f; cnt_run = 0; }
+  // The values of one stage in registers (packed bf16 pairs where nothing has to be mixed).
+  static constexpr bool PACKED = !CFG && sizeof(T) == 2;
+  static constexpr int NW = PACKED ? NVS * 4 : 1;
+  static constexpr int NF = PACKED ? 1 : NVS * VEC;
+  struct Values {
+    uint32_t w[NW];
+    float f[NF];
+    float largest;   // over the warp
+  };
+  // The n values of one stage: once this is back every lane has read them, and the stage can be filled again.
+  __device__ __forceinline__ void load(Values& val, const unsigned char* stage, const int n, const float scale, const int lane) const {
+    uint32_t (&w)[NW] = val.w;
+    float (&vals)[NF] = val.f;
+    const bool full = n == EPS;   // (after a timeout the data is garbage anyway: the call is flagged)
+    // The whole stage is one group: its values (packed bf16 pairs where nothing has to be mixed) sit
+    // in registers, one reduction gives the warp's largest, and since that result depends on every
+    // lane's loads the stage can be handed back for its refill before the exponentials are taken.
+    float gm;   // this lane's largest value of the stage
+    if (PACKED && full) {
+#pragma unroll
+      for (int v = 0; v < NVS; ++v) {
+        const uint4 q4 = *reinterpret_cast<const uint4*>(stage + (v * 32 + lane) * VEC * (int)sizeof(T));
+        w[(v * 4 + 0) % NW] = q4.x; w[(v * 4 + 1) % NW] = q4.y; w[(v * 4 + 2) % NW] = q4.z; w[(v * 4 + 3) % NW] = q4.w;
+      }
+      uint32_t m2[4] = {w[0], w[1 % NW], w[2 % NW], w[3 % NW]};
+#pragma unroll
+      for (int k = 4; k < NW; ++k) asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[k & 3]) : "r"(w[k]));
+      asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[0]) : "r"(m2[1]));
+      asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[2]) : "r"(m2[3]));
+      asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[0]) : "r"(m2[2]));
+      gm = fmaxf(__uint_as_float(m2[0] << 16), __uint_as_float(m2[0] & 0xffff0000u));
+    } else if (PACKED) {
+      // ragged last stage of a packed row: out-of-range pairs read as -inf (0xff80 twice)
+#pragma unroll
+      for (int v = 0; v < NVS; ++v) {
+        const int xo = (v * 32 + lane) * VEC;
+        uint4 q4 = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+        if (xo < n) q4 = *reinterpret_cast<const uint4*>(stage + xo * (int)sizeof(T));
+        w[(v * 4 + 0) % NW] = q4.x; w[(v * 4 + 1) % NW] = q4.y; w[(v * 4 + 2) % NW] = q4.z; w[(v * 4 + 3) % NW] = q4.w;
+      }
+      uint32_t m2 = w[0];
+#pragma unroll
+      for (int k = 1; k < NW; ++k) asm("max.bf16x2 %0, %0, %1;" : "+r"(m2) : "r"(w[k]));
+      gm = fmaxf(__uint_as_float(m2 << 16), __uint_as_float(m2 & 0xffff0000u));
+    } else {
+#pragma unroll
+      for (int v = 0; v < NVS; ++v) {
+        const int xo = (v * 32 + lane) * VEC;
+        float zc[VEC];
+        if (full || xo < n) {
+          unpack_vec<T>(stage + xo * (int)sizeof(T), zc);
+          if (CFG) {
+            float zu[VEC];
+            unpack_vec<T>(stage + BYTES / 2 + xo * (int)sizeof(T), zu);
+            cfg_mix_vec<VEC>(zc, zu, scale);
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) zc[e] = CSD_NEG_INF;
+        }
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) vals[(v * VEC + e) % NF] = zc[e];
+      }
+      float m4[4] = {CSD_NEG_INF, CSD_NEG_INF, CSD_NEG_INF, CSD_NEG_INF};
+#pragma unroll
+      for (int e = 0; e < NF; ++e) m4[e & 3] = fmaxf(m4[e & 3], vals[e]);
+      gm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+    }
+    // the stage's largest value over the warp (one integer reduction on order-preserving keys)
+    int key = __float_as_int(gm);
+    key ^= (key >> 31) & 0x7fffffff;
+    key = __reduce_max_sync(0xffffffffu, key);
+    key ^= (key >> 31) & 0x7fffffff;
+    val.largest = __int_as_float(key);
+  }
+  __device__ __forceinline__ void add(Values& val) {
+    uint32_t (&w)[NW] = val.w;
+    float (&vals)[NF] = val.f;
+    const float wm = val.largest;
+    if (wm > Mw) {   // a new maximum: what was counted as "equal to the maximum" becomes ordinary mass
+      const float MwL = wm * kLog2e;
+      const float dlt_new = fmaf(wm, kLog2e, -MwL);
+      s_run = (s_run * ex2f(-dlt) + (float)cnt_run) * ex2f((Mw - wm) * kLog2e) * ex2f(dlt_new);
+      cnt_run = 0;
+      Mw = wm;
+      nMwL = -MwL;
+      dlt = dlt_new;
+    }
+    float acc4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (PACKED) {
+      if (wm == Mw) {
+        // values equal to the reference may be present: they are counted, not summed.  On the packed
+        // pairs: one compare per pair marks them, the marked halves become -inf (their exponential is
+        // then exactly 0) and are counted, 16 bits of the counter per half.
+        const uint32_t m16 = __float_as_uint(Mw) >> 16;
+        const uint32_t Mw2 = m16 | (m16 << 16);
+        uint32_t c2 = 0;
+#pragma unroll
+        for (int k = 0; k < NW; k += 2) {
+          uint32_t e0, e1;
+          asm("set.eq.u32.bf16x2 %0, %1, %2;" : "=r"(e0) : "r"(w[k]), "r"(Mw2));
+          asm("set.eq.u32.bf16x2 %0, %1, %2;" : "=r"(e1) : "r"(w[(k + 1) % NW]), "r"(Mw2));
+          w[k] = (w[k] & ~e0) | (0xff80ff80u & e0);
+          w[(k + 1) % NW] = (w[(k + 1) % NW] & ~e1) | (0xff80ff80u & e1);
+          c2 += (e0 & 0x00010001u) + (e1 & 0x00010001u);
+        }
+        static_assert(NW % 2 == 0 || NW == 1, "pairs of words");
+        cnt_run += (int)((c2 & 0xffffu) + (c2 >> 16));
+      }
+      // exponents and sums two values per instruction (each half the IEEE operation: the same bits as
+      // the scalar form); NaN values poison the sum, which marks the row
+      const uint64_t l2e2 = pack2(kLog2e, kLog2e), nm2 = pack2(nMwL, nMwL);
+      uint64_t accp[2] = {pack2(0.0f, 0.0f), pack2(0.0f, 0.0f)};
+#pragma unroll
+      for (int k = 0; k < NW; ++k) {
+        float x0, x1;
+        unpack2(fma2(pack2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xffff0000u)), l2e2, nm2), x0, x1);
+        accp[k & 1] = add2(accp[k & 1], pack2(ex2f(x0), ex2f(x1)));
+      }
+      unpack2(accp[0], acc4[0], acc4[1]);
+      unpack2(accp[1], acc4[2], acc4[3]);
+    } else if (wm == Mw) {
+      // (branch-free: the exponential of a value equal to the reference is replaced by 0)
+      int c4[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int e = 0; e < NF; ++e) {
+        const float ex = ex2f(fmaf(vals[e], kLog2e, nMwL));
+        acc4[e & 3] += vals[e] == Mw ? 0.0f : ex;
+        c4[e & 3] += vals[e] == Mw ? 1 : 0;
+      }
+      cnt_run += (c4[0] + c4[1]) + (c4[2] + c4[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < NF; ++e) acc4[e & 3] += ex2f(fmaf(vals[e], kLog2e, nMwL));
+    }
+    s_run += (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
+  }
+  // The pair of everything added: m = Mw, s = sum over everything except one entry at the maximum; valid in every lane.
+  __device__ __forceinline__ float2 end() {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s_run += __shfl_xor_sync(0xffffffffu, s_run, off);
+      cnt_run += __shfl_xor_sync(0xffffffffu, cnt_run, off);
+    }
+    return make_float2(Mw, s_run * ex2f(-dlt) + (float)(cnt_run - 1));
+  }
+};
+
 struct PlainSmem {
   alignas(128) unsigned char ring[kPlainWarps][kWStages][kWStageBytes];
   alignas(8) uint64_t full[kPlainWarps][kWStages];
@@ -1012,12 +1185,8 @@ static_assert(sizeof(float2) * kBlockStash >= sizeof(double) * kFinTiles, "tile 
 
 template <typename T, bool CFG>
 __global__ void __launch_bounds__(kPlainThreads, 3) verify_plain_kernel(const FusedArgs a) {
-  constexpr int VEC = Elem<T>::kVec;
   constexpr int ARR = CFG ? 2 : 1;
-  constexpr int EPS = kWStageBytes / ((int)sizeof(T) * ARR);   // elements of a row per warp stage
-  constexpr int VPL = EPS / 32;                                // values per lane per stage
-  constexpr int NVS = VPL / VEC;                               // 16-byte vectors per lane per stage
-  static_assert(NVS >= 1, "a stage holds at least one vector per lane");
+  constexpr int EPS = StageStats<T, CFG, kWStageBytes>::EPS;   // elements of a row per warp stage
   extern __shared__ __align__(128) unsigned char fused_smem_raw[];
   PlainSmem& sm = *reinterpret_cast<PlainSmem*>(fused_smem_raw);
 
@@ -1104,161 +1273,25 @@ __global__ void __launch_bounds__(kPlainThreads, 3) verify_plain_kernel(const Fu
       if (part == parts) part = 0;
       const int x_begin = part * part_elems;
       const int x_end = min(V, x_begin + part_elems);
-      // Running statistics of the item, relative to a maximum that is the same in every lane of
-      // the warp: Mw = largest value met so far by any lane, s = this lane's sum of
-      // exp(z - Mw) over its values below Mw, cnt = this lane's number of values equal to Mw.
-      // Because the reference is warp-uniform, a group of values below it is summed with no
-      // test per value, and the exact treatment of values equal to it is a uniform branch
-      // taken only where the maximum sits.
-      // The exponent (z - Mw) log2(e) is formed by one fused multiply-add, z * log2(e) - MwL with MwL
-      // the ROUNDED product Mw * log2(e); its rounding error dlt = Mw * log2(e) - MwL (exact, again by
-      // a fused multiply-add) is a common factor 2^dlt of the sum and is divided out once per item.
-      float Mw = CSD_NEG_INF, s_run = 0.0f;
-      float nMwL = 0.0f, dlt = 0.0f;   // -MwL and dlt of the current reference (while Mw is -inf every value is
-                                       // -inf or NaN, and with 0 here its exponential is 0 or NaN as it should be)
-      int cnt_run = 0;
+      StageStats<T, CFG, kWStageBytes> run;
+      run.begin();
       for (int x0 = x_begin; x0 < x_end; x0 += EPS) {
         if (ok) {
           if (mbar_wait(&sm.full[warp][c_s], c_par, a.wait_limit)) ++waited; else ok = false;
         }
         const int n = min(EPS, x_end - x0);
         const unsigned char* stage = &sm.ring[warp][c_s][0];
-        const bool full = n == EPS;   // (after a timeout the data is garbage anyway: the call is flagged)
-        // The whole stage is one group: its values (packed bf16 pairs where nothing has to be mixed) sit
-        // in registers, one reduction gives the warp's largest, and since that result depends on every
-        // lane's loads the stage can be handed back for its refill before the exponentials are taken.
-        constexpr bool PACKED = !CFG && sizeof(T) == 2;
-        constexpr int NW = PACKED ? NVS * 4 : 1;
-        constexpr int NF = PACKED ? 1 : NVS * VEC;
-        uint32_t w[NW];
-        float vals[NF];
-        float gm;   // this lane's largest value of the stage
-        if (PACKED && full) {
-#pragma unroll
-          for (int v = 0; v < NVS; ++v) {
-            const uint4 q4 = *reinterpret_cast<const uint4*>(stage + (v * 32 + lane) * VEC * (int)sizeof(T));
-            w[(v * 4 + 0) % NW] = q4.x; w[(v * 4 + 1) % NW] = q4.y; w[(v * 4 + 2) % NW] = q4.z; w[(v * 4 + 3) % NW] = q4.w;
-          }
-          uint32_t m2[4] = {w[0], w[1 % NW], w[2 % NW], w[3 % NW]};
-#pragma unroll
-          for (int k = 4; k < NW; ++k) asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[k & 3]) : "r"(w[k]));
-          asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[0]) : "r"(m2[1]));
-          asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[2]) : "r"(m2[3]));
-          asm("max.bf16x2 %0, %0, %1;" : "+r"(m2[0]) : "r"(m2[2]));
-          gm = fmaxf(__uint_as_float(m2[0] << 16), __uint_as_float(m2[0] & 0xffff0000u));
-        } else if (PACKED) {
-          // ragged last stage of a packed row: out-of-range pairs read as -inf (0xff80 twice)
-#pragma unroll
-          for (int v = 0; v < NVS; ++v) {
-            const int xo = (v * 32 + lane) * VEC;
-            uint4 q4 = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-            if (xo < n) q4 = *reinterpret_cast<const uint4*>(stage + xo * (int)sizeof(T));
-            w[(v * 4 + 0) % NW] = q4.x; w[(v * 4 + 1) % NW] = q4.y; w[(v * 4 + 2) % NW] = q4.z; w[(v * 4 + 3) % NW] = q4.w;
-          }
-          uint32_t m2 = w[0];
-#pragma unroll
-          for (int k = 1; k < NW; ++k) asm("max.bf16x2 %0, %0, %1;" : "+r"(m2) : "r"(w[k]));
-          gm = fmaxf(__uint_as_float(m2 << 16), __uint_as_float(m2 & 0xffff0000u));
-        } else {
-#pragma unroll
-          for (int v = 0; v < NVS; ++v) {
-            const int xo = (v * 32 + lane) * VEC;
-            float zc[VEC];
-            if (full || xo < n) {
-              unpack_vec<T>(stage + xo * (int)sizeof(T), zc);
-              if (CFG) {
-                float zu[VEC];
-                unpack_vec<T>(stage + kWStageBytes / 2 + xo * (int)sizeof(T), zu);
-                cfg_mix_vec<VEC>(zc, zu, f.cfg_scale);
-              }
-            } else {
-#pragma unroll
-              for (int e = 0; e < VEC; ++e) zc[e] = CSD_NEG_INF;
-            }
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) vals[(v * VEC + e) % NF] = zc[e];
-          }
-          float m4[4] = {CSD_NEG_INF, CSD_NEG_INF, CSD_NEG_INF, CSD_NEG_INF};
-#pragma unroll
-          for (int e = 0; e < NF; ++e) m4[e & 3] = fmaxf(m4[e & 3], vals[e]);
-          gm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-        }
-        // the stage's largest value over the warp (one integer reduction on order-preserving keys)
-        int key = __float_as_int(gm);
-        key ^= (key >> 31) & 0x7fffffff;
-        key = __reduce_max_sync(0xffffffffu, key);
-        key ^= (key >> 31) & 0x7fffffff;
-        const float wm = __int_as_float(key);
+        typename StageStats<T, CFG, kWStageBytes>::Values values;
+        run.load(values, stage, n, f.cfg_scale, lane);
         if (lane == 0 && ok) {   // every lane has read the stage: refill it with the chunk kWStages ahead
           fence_before_bulk();
           producer_issue();
         }
-        if (wm > Mw) {   // a new maximum: what was counted as "equal to the maximum" becomes ordinary mass
-          const float MwL = wm * kLog2e;
-          const float dlt_new = fmaf(wm, kLog2e, -MwL);
-          s_run = (s_run * ex2f(-dlt) + (float)cnt_run) * ex2f((Mw - wm) * kLog2e) * ex2f(dlt_new);
-          cnt_run = 0;
-          Mw = wm;
-          nMwL = -MwL;
-          dlt = dlt_new;
-        }
-        float acc4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (PACKED) {
-          if (wm == Mw) {
-            // values equal to the reference may be present: they are counted, not summed.  On the packed
-            // pairs: one compare per pair marks them, the marked halves become -inf (their exponential is
-            // then exactly 0) and are counted, 16 bits of the counter per half.
-            const uint32_t m16 = __float_as_uint(Mw) >> 16;
-            const uint32_t Mw2 = m16 | (m16 << 16);
-            uint32_t c2 = 0;
-#pragma unroll
-            for (int k = 0; k < NW; k += 2) {
-              uint32_t e0, e1;
-              asm("set.eq.u32.bf16x2 %0, %1, %2;" : "=r"(e0) : "r"(w[k]), "r"(Mw2));
-              asm("set.eq.u32.bf16x2 %0, %1, %2;" : "=r"(e1) : "r"(w[(k + 1) % NW]), "r"(Mw2));
-              w[k] = (w[k] & ~e0) | (0xff80ff80u & e0);
-              w[(k + 1) % NW] = (w[(k + 1) % NW] & ~e1) | (0xff80ff80u & e1);
-              c2 += (e0 & 0x00010001u) + (e1 & 0x00010001u);
-            }
-            static_assert(NW % 2 == 0 || NW == 1, "pairs of words");
-            cnt_run += (int)((c2 & 0xffffu) + (c2 >> 16));
-          }
-          // exponents and sums two values per instruction (each half the IEEE operation: the same bits as
-          // the scalar form); NaN values poison the sum, which marks the row
-          const uint64_t l2e2 = pack2(kLog2e, kLog2e), nm2 = pack2(nMwL, nMwL);
-          uint64_t accp[2] = {pack2(0.0f, 0.0f), pack2(0.0f, 0.0f)};
-#pragma unroll
-          for (int k = 0; k < NW; ++k) {
-            float x0, x1;
-            unpack2(fma2(pack2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xffff0000u)), l2e2, nm2), x0, x1);
-            accp[k & 1] = add2(accp[k & 1], pack2(ex2f(x0), ex2f(x1)));
-          }
-          unpack2(accp[0], acc4[0], acc4[1]);
-          unpack2(accp[1], acc4[2], acc4[3]);
-        } else if (wm == Mw) {
-          // (branch-free: the exponential of a value equal to the reference is replaced by 0)
-          int c4[4] = {0, 0, 0, 0};
-#pragma unroll
-          for (int e = 0; e < NF; ++e) {
-            const float ex = ex2f(fmaf(vals[e], kLog2e, nMwL));
-            acc4[e & 3] += vals[e] == Mw ? 0.0f : ex;
-            c4[e & 3] += vals[e] == Mw ? 1 : 0;
-          }
-          cnt_run += (c4[0] + c4[1]) + (c4[2] + c4[3]);
-        } else {
-#pragma unroll
-          for (int e = 0; e < NF; ++e) acc4[e & 3] += ex2f(fmaf(vals[e], kLog2e, nMwL));
-        }
-        s_run += (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
+        run.add(values);
         if (++c_s == kWStages) { c_s = 0; c_par ^= 1u; }
       }
-      // the item's pair: m = Mw, s = sum over everything except one entry at the maximum
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        s_run += __shfl_xor_sync(0xffffffffu, s_run, off);
-        cnt_run += __shfl_xor_sync(0xffffffffu, cnt_run, off);
-      }
-      if (lane == 0 && item < kBlockStash) sm.stash[item] = make_float2(Mw, s_run * ex2f(-dlt) + (float)(cnt_run - 1));
+      const float2 v = run.end();
+      if (lane == 0 && item < kBlockStash) sm.stash[item] = v;
     }
     if (!ok) {
       sm.abort = 1;
@@ -1494,8 +1527,10 @@ __device__ __forceinline__ void load_stage(const uint32_t base, const int n, con
 }
 
 // RAGGED: V is not a whole number of stages, so the last stage of a row is partly filled (the host
-// picks the instance; without it the streaming loop has no bounds tests at all).
-template <typename T, bool CFG, bool RAGGED, int WL>
+// picks the instance; without it the streaming loop has no bounds tests at all).  DEALT: all sequences' rows are dealt out to the
+// blocks, and the kernel stops with their results (FusedArgs::rows_out; an instance of its own, since its few instructions cost the
+// overlapping calls 0.5 %).
+template <typename T, bool CFG, bool RAGGED, int WL, bool DEALT>
 __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const FusedArgs a) {
   constexpr int VEC = Elem<T>::kVec;
   constexpr int ARR = CFG ? 2 : 1;
@@ -1538,15 +1573,17 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   if (a.ctas_per_seq > 1) cluster_arrive();   // first half; finish_block waits before it writes to a peer
   call_begin(a.ordered, a.signal != 0);
 
-  // this block's local rows (see block_share)
-  const BlockShare sh = block_share(a);
+  // this block's local rows (see block_share), or a run of all sequences' rows
+  BlockShare sh = block_share(a);
   const bool stats_only = a.stats_out != nullptr;
+  const int row0 = DEALT ? a.rows_per_block * (int)blockIdx.x : 0;
+  if (DEALT) { sh.seq_begin = 0; sh.n_rows = max(0, min(a.rows_per_block, f.B * sh.rows_per_seq - row0)); }
   const int n_rows = sh.n_rows;
   const int n_chunks = n_rows * cpr;
 
   auto row_of = [&](int row_id) -> Row<T, CFG> {
     int b, which, i;
-    local_row(sh, row_id, f.gamma, b, which, i);
+    local_row(sh, row0 + row_id, f.gamma, b, which, i);
     return row_at<T, CFG>(f, b, which, i);
   };
   // Issues the copies of chunk q of this block (chunk q % cpr of its local row q / cpr), if there is
@@ -1571,8 +1608,8 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   // (the first copies are under way: the block's small inputs and the drafted tokens' logits -- two dependent
   // trips to memory -- are fetched in their shadow)
   if (!stats_only) {
-    stage_inputs(a, sh, 0, tid, sm.fst);
-    load_token_logits<T, CFG, kTopkThreads>(f, sh, tid, sm.rs);
+    if (!DEALT) stage_inputs(a, sh, 0, tid, sm.fst);
+    load_token_logits<T, CFG, kTopkThreads>(f, sh, tid, sm.rs, row0);
   } else {
     for (int r = tid; r < kBlockRows; r += kTopkThreads) sm.rs.tokz[r] = 0.0f;   // (read by the short cut's rank, unused here)
   }
@@ -1986,6 +2023,15 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   __syncthreads();
   if (stats_only) {
     write_row_stats<T, CFG>(a, sh, sm.rs, tid, kTopkThreads, sm.abort != 0);
+    return;
+  }
+  if (DEALT) {
+    for (int r = tid; r < n_rows && r < kBlockRows; r += kTopkThreads) {
+      int b, which, i;
+      local_row(sh, row0 + r, f.gamma, b, which, i);
+      const float2 ms = sm.abort ? make_float2(__int_as_float(0x7fc00000), 0.0f) : sm.rs.ms[r];   // (reads as unusable)
+      a.rows_out[(int64_t)b * sh.rows_per_seq + (which == 0 ? i : f.T + i)] = make_float4(ms.x, ms.y, sm.rs.thr[r], sm.rs.tokz[r]);
+    }
     return;
   }
   static_assert(sizeof(sm.list) >= kFinTiles * sizeof(double), "tile sums live in the list area");

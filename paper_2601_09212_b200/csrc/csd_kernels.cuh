@@ -134,6 +134,7 @@ template <> struct Elem<float> {
   }
   template <bool FROZEN = false>
   __device__ static __forceinline__ float load_one(const float* p) { return FROZEN ? __ldg(p) : __ldca(p); }
+  __device__ static __forceinline__ float load_one_l2(const float* p) { return __ldcg(p); }
 };
 template <> struct Elem<__nv_bfloat16> {
   static constexpr int kVec = 8;
@@ -152,6 +153,9 @@ template <> struct Elem<__nv_bfloat16> {
   __device__ static __forceinline__ float load_one(const __nv_bfloat16* p) {
     const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
     return __uint_as_float(((uint32_t)(FROZEN ? __ldg(q) : __ldca(q))) << 16);
+  }
+  __device__ static __forceinline__ float load_one_l2(const __nv_bfloat16* p) {
+    return __uint_as_float(((uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(p))) << 16);
   }
 };
 
@@ -231,6 +235,15 @@ struct Row {
 #endif
     float z = Elem<T>::template load_one<FROZEN>(cond + x);
     if (CFG) z = cfg_mix(z, Elem<T>::template load_one<FROZEN>(uncond + x), scale);
+    return z;
+  }
+  // the same past L1
+  __device__ __forceinline__ float load_one_l2(int x) const {
+#ifdef CSD_CHECKED
+    if (!checked_ok(x, 1, n, 2)) return CSD_NEG_INF;
+#endif
+    float z = Elem<T>::load_one_l2(cond + x);
+    if (CFG) z = cfg_mix(z, Elem<T>::load_one_l2(uncond + x), scale);
     return z;
   }
   // vector when allowed, otherwise bounds-checked scalars; out-of-range -> -inf

@@ -1,0 +1,133 @@
+"""Row statistics dealt out evenly over the GPU, then one cluster per sequence (csd_flat.cuh), at the edges of its pieces: rows of one
+stage and just beside it, pieces that cut rows everywhere, ragged last stages, draws shared by 1 to 8 blocks, more sequences
+than finishing blocks fit at once.  Tolerances are those of the other parity tests (tests/gpu_util.py)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2601_09212_b200 as csd
+from paper_2601_09212_b200 import workloads as W
+from gpu_util import check, run_gpu
+from oracle.compare import compare
+
+DEV = "cuda"
+
+
+def _make(kw, seed=5):
+    L = kw["gamma"]
+    return W.make("t", schedule=csd.csd_make_schedule(1, 1.2, 0.6, L), seed=seed, device=DEV, **kw)
+
+
+def _dealt():
+    plan = csd.csd_last_plan()
+    return plan.path == 2 and plan.parts > 0
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=300, gamma=16, V=1536, dtype=W.BF16, bonus_row=True),          # rows of one stage; more sequences than blocks at once
+    dict(B=300, gamma=31, V=2048, dtype=W.F32),                           # ... of two
+    dict(B=300, gamma=31, V=2052, dtype=W.F32, bonus_row=True),           # ... and four values more
+    dict(B=150, gamma=32, V=2056, dtype=W.BF16, bonus_row=True),          # 65 rows, the draw by one block
+    dict(B=330, gamma=20, V=3080, dtype=W.BF16, rho=0.7),
+    dict(B=76, gamma=6, V=16388, dtype=W.F32, rho=0.7),                   # ... by two
+    dict(B=74, gamma=4, V=65536, dtype=W.BF16, rho=0.97, bonus_row=True), # ... by four, rows of 43 stages
+    dict(B=36, gamma=8, V=32776, dtype=W.BF16, bonus_row=True),           # ... by eight
+    dict(B=20, gamma=16, V=32768, dtype=W.BF16, cfg=True, cfg_scale=3.0, bonus_row=True),
+    dict(B=80, gamma=5, V=6148, dtype=W.F32, cfg=True, cfg_scale=2.0),
+    # top-k: rows dealt out whole, one to a block or several, lists of both sizes, rows selected exactly, heavy tails
+    dict(B=24, gamma=10, V=8192, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=400, bonus_row=True),
+    dict(B=64, gamma=8, V=4104, dtype=W.BF16, cfg=True, cfg_scale=5.0, top_k=250, bonus_row=True),
+    dict(B=150, gamma=9, V=4100, dtype=W.F32, top_k=300, bonus_row=True),
+    dict(B=40, gamma=7, V=16384, dtype=W.BF16, top_k=1900, law="student3"),
+    dict(B=40, gamma=9, V=4096, dtype=W.F32, top_k=2500, bonus_row=True),
+])
+def test_pieces(kw):
+    w = _make(kw)
+    some = slice(0, None, max(1, kw["B"] * kw["V"] // 600000))
+    rep, _, ref = check(w, rows=some, want_dbg=kw["B"] * kw["V"] <= 1 << 21)
+    h = {k: v if v is None or k == "relax_schedule" else v[some] for k, v in w.host_arrays().items()}
+    assert _dealt()
+    assert rep.ok and rep.tau_mismatch_near + rep.token_mismatch_near <= 2, rep.summary()
+    got = run_gpu(w, want_dbg=False)   # (with top-k: without the exact thresholds that the distribution asks for)
+    rep = compare(ref, got["tokens"][some], got["accept_len"][some], h["draft_tokens"], h["uniforms"], status=got["status"][some])
+    assert rep.ok, rep.summary()
+    other = run_gpu(w, want_dbg=False, back_to_back=True)   # the same round, a block to a sequence
+    assert not _dealt()
+    same = (got["tokens"] == other["tokens"]).all(axis=1) & (got["accept_len"] == other["accept_len"])
+    assert (~same).sum() <= 2, kw   # (two summation orders: a sequence may sit on a boundary)
+    again = run_gpu(w, want_dbg=False)
+    for key in ("tokens", "accept_len", "status"):
+        assert np.array_equal(got[key], again[key]), key
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=76, gamma=6, V=16388, dtype=W.F32, bonus_row=True),
+    dict(B=80, gamma=8, V=12296, dtype=W.BF16, cfg=True, cfg_scale=2.5),
+    dict(B=64, gamma=8, V=4104, dtype=W.BF16, cfg=True, cfg_scale=5.0, top_k=250, bonus_row=True),
+])
+def test_padded_batches(kw):
+    """Sequences that lie further apart than their rows need: the same results as from contiguous ones, bit for bit."""
+    w = _make(kw)
+    B, L, T, V = w.B, w.gamma, w.target_logits.shape[1], w.V
+    want = run_gpu(w, want_dbg=False)
+    assert _dealt()
+
+    def embed(t, gap):
+        if t is None:
+            return None
+        big = torch.full((B, t[0].numel() + gap), float("nan"), dtype=t.dtype, device=DEV)
+        big[:, :t[0].numel()] = t.reshape(B, -1)
+        return big
+
+    big = [embed(w.target_logits, 8), embed(w.draft_logits, 24), embed(w.target_uncond, 8), embed(w.draft_uncond, 24)]
+    out = [torch.full((B, n), -7, dtype=torch.int32, device=DEV) for n in (L + 1, 1, 1)]
+    ws = csd.new_workspace(B, L, V, w.dtype)
+    prm = csd.make_params(w.target_logits, w.draft_logits, w.draft_tokens, w.uniforms, w.relax_schedule, out[0], out[1][:, 0],
+                          target_uncond=w.target_uncond, draft_uncond=w.draft_uncond, cfg_scale=w.cfg_scale, top_k=w.top_k,
+                          out_status=out[2][:, 0], workspace=ws)
+    prm.target_logits, prm.draft_logits = big[0].data_ptr(), big[1].data_ptr()
+    if big[2] is not None:
+        prm.target_uncond, prm.draft_uncond = big[2].data_ptr(), big[3].data_ptr()
+    prm.target_batch_stride, prm.draft_batch_stride = big[0].shape[1], big[1].shape[1]
+    csd.csd_verify_ex(prm)
+    torch.cuda.synchronize()
+    assert _dealt()
+    for got, key in zip(out, ("tokens", "accept_len", "status")):
+        assert np.array_equal(got.cpu().numpy().reshape(want[key].shape), want[key]), key
+
+
+def test_unusable_rows_and_tokens():
+    """NaN, +inf and fully masked rows and tokens out of range in some sequences; their neighbours are not touched."""
+    w = _make(dict(B=76, gamma=6, V=16384, dtype=W.F32, bonus_row=True))
+    w.target_logits[3, 1, 77] = float("nan")
+    w.draft_logits[7, 0, 8000] = float("inf")
+    w.target_logits[11, :, :] = float("-inf")
+    w.draft_logits[15, 2, :] = float("-inf")
+    w.draft_tokens[19, 0] = 16384
+    w.draft_tokens[23, 1] = -5
+    rep, got, _ = check(w, rows=slice(0, 26))
+    assert _dealt()
+    assert rep.ok, rep.summary()
+
+
+def test_wait_that_runs_out_is_reported():
+    """A stage that is announced and never copied: the call returns and says so until the workspace is cleared."""
+    w = _make(dict(B=76, gamma=6, V=16384, dtype=W.F32))
+    ws = csd.new_workspace(w.B, w.gamma, w.V, w.dtype)
+    good = run_gpu(w, want_dbg=False, workspace=ws)
+    assert _dealt() and np.all(good["status"] == 0)
+    csd.csd_test_hooks(21, True)
+    try:
+        bad = run_gpu(w, want_dbg=False, workspace=ws)
+    finally:
+        csd.csd_test_hooks()
+    assert np.all(bad["status"] & csd.CSD_STATUS_TIMEOUT)
+    csd.csd_workspace_init(ws)
+    clean = run_gpu(w, want_dbg=False, workspace=ws)
+    for key in ("tokens", "accept_len", "status"):
+        assert np.array_equal(clean[key], good[key]), key
