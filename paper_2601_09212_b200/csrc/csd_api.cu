@@ -156,7 +156,7 @@ cudaError_t launch_fused_t(const FusedArgs& a, bool topk, int grid, cudaStream_t
   if (!topk) return launch_fused<T, CFG, 0>(a, grid, stream);
   constexpr int kStageElems = kTkStageBytes / ((int)sizeof(T) * (CFG ? 2 : 1));
   const bool whole = a.fin.V % kStageElems == 0;
-  if (a.rows_out) {
+  if (a.rows_per_block > 0) {
     if (a.large_lists) return whole ? launch_fused<T, CFG, 3, true>(a, grid, stream) : launch_fused<T, CFG, 4, true>(a, grid, stream);
     return whole ? launch_fused<T, CFG, 1, true>(a, grid, stream) : launch_fused<T, CFG, 2, true>(a, grid, stream);
   }
@@ -503,8 +503,8 @@ cudaError_t slice_call(const SliceCall& in, bool dry, cudaStream_t stream, bool*
   }
   else if (!in.topk) other_ns = 9e3 + 0.09 * logits;
   else other_ns = rows > 1 ? 7e3 + 2.5e3 * rows + 0.33 * logits : 5e3 + 0.5 * logits;
-  // (both expectations are off by a sixth, so rows are dealt out instead where that promises a fifth less: of 37 random calls
-  // that would be sliced and have a row for every SM, 27 go so, in 0.52 - 0.98 of the time, all 37 in 0.76 in the mean)
+  // (both expectations are off by a sixth, so rows are dealt out instead where that promises a fifth less: of 40 random calls
+  // that would be sliced and have a row for every second SM, 31 go so, in 0.52 - 0.98 of the time, all 40 in 0.75 in the mean)
   if (in.dealt_ns > 0.0 && 1.25 * in.dealt_ns < other_ns) other_ns = 1.25 * in.dealt_ns;
   SliceArgs a;
   memset(&a, 0, sizeof a);
@@ -555,7 +555,8 @@ struct FusedPlan {
   cudaStream_t stream;
   float4* records = nullptr;   // with stats_out (see FusedArgs)
   int v_offset = 0;
-  float4* rows_out = nullptr;  // top-k: all rows dealt out (see FusedArgs)
+  bool dealt = false;          // top-k: all rows dealt out (see FusedArgs), into rows_out or stats_out
+  float4* rows_out = nullptr;
 };
 cudaError_t plan_and_launch_fused(const FusedPlan& in) {
   const int sms = in.sms, es = in.es, rows_per_seq = in.rows_per_seq;
@@ -656,7 +657,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
       ua.parts_per_row = (int)((cpr + cpp - 1) / cpp);
     }
     long long grid = c > 1 ? (long long)in.B * c : (in.B + spc - 1) / spc;
-    if (in.rows_out) {   // one wave of four blocks per SM
+    if (in.dealt) {   // one wave of four blocks per SM
       c = spc = 1;
       ua.rows_per_block = (int)((in.rows + kFlatTopkBlocks * sms - 1) / (kFlatTopkBlocks * sms));
       grid = (in.rows + ua.rows_per_block - 1) / ua.rows_per_block;
@@ -670,7 +671,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     // with more, they would fill the SMs that happen to have room and end up unevenly spread (256 sequences of 16
     // positions, 256 blocks: 67.6 us a call without the early signal, 85.8 with it).  A stats-only call is
     // followed by its finishing kernel, whose large blocks would only sit on SMs this kernel needs.
-    ua.signal = (in.rows_out != nullptr || (in.stats_out == nullptr && (in.back_to_back || grid <= sms))) ? 1 : 0;
+    ua.signal = (in.dealt || (in.stats_out == nullptr && (in.back_to_back || grid <= sms))) ? 1 : 0;
     if (in.dtype == CSD_F32)
       fe = cfg ? launch_fused_t<float, true>(ua, topk, (int)grid, stream)
                : launch_fused_t<float, false>(ua, topk, (int)grid, stream);
@@ -745,28 +746,27 @@ int flat_parts(const FusedPlan& in, size_t max_parts) {
   const long long parts = spr < 2 ? 1 : (spr - 2) / least + 2;   // as many as a row can be cut into
   return parts <= (long long)max_parts ? (int)parts : 0;
 }
+// Their statistics: without top-k `parts` slots of fa.partials per row, with it one record per row in in.rows_out, or in.stats_out
+// and in.thr_out.
 template <typename T, bool CFG>
-cudaError_t launch_flat(const FusedPlan& in, const int parts) {
-  FlatArgs a;
+cudaError_t launch_flat_stats(const FusedPlan& in, const int parts, FlatArgs& a) {
   memset(&a, 0, sizeof a);
   a.fin = in.fa;
+  a.fin.parts = parts;
   a.error_flag = in.error_flag;
-  a.wait_limit = g_wait_limit;
-  a.drop_first_copy = g_drop_first_copy == 1;
+  a.rows = in.rows_out;
   if (in.topk) {
     FusedPlan fp = in;
-    a.fin.parts = 1;
-    fp.rows_out = reinterpret_cast<float4*>(const_cast<float2*>(in.fa.partials));
-    a.rows = fp.rows_out;
-    const cudaError_t e = plan_and_launch_fused(fp);
-    return e == cudaSuccess ? launch_flat_finish<T, CFG, true>(a, in.sms, in.stream) : e;
+    fp.dealt = true;
+    return plan_and_launch_fused(fp);
   }
+  a.wait_limit = g_wait_limit;
+  a.drop_first_copy = g_drop_first_copy == 1;
   constexpr int EPS = StageStats<T, CFG, kFlatStageBytes<T>>::EPS;
   a.stages_per_row = (in.V + EPS - 1) / EPS;
   a.stages = in.rows * a.stages_per_row;
   const int grid = kFlatBlocks * in.sms;
   a.warps = grid * kPlainWarps;
-  a.fin.parts = parts;
   a.partials = const_cast<float2*>(in.fa.partials);
   static bool configured[kMaxDevices] = {};
   int dev = 0;
@@ -776,8 +776,24 @@ cudaError_t launch_flat(const FusedPlan& in, const int parts) {
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  const cudaError_t e = launch_after(flat_stats_kernel<T, CFG>, a, (unsigned)grid, kPlainThreads, sizeof(FlatSmem<T>), in.stream);
-  return e == cudaSuccess ? launch_flat_finish<T, CFG, false>(a, in.sms, in.stream) : e;
+  return launch_after(flat_stats_kernel<T, CFG>, a, (unsigned)grid, kPlainThreads, sizeof(FlatSmem<T>), in.stream);
+}
+template <typename T, bool CFG>
+cudaError_t launch_flat(FusedPlan in, const int parts) {
+  FlatArgs a;
+  if (in.topk) in.rows_out = reinterpret_cast<float4*>(const_cast<float2*>(in.fa.partials));
+  const cudaError_t e = launch_flat_stats<T, CFG>(in, parts, a);
+  if (e != cudaSuccess) return e;
+  return in.topk ? launch_flat_finish<T, CFG, true>(a, in.sms, in.stream) : launch_flat_finish<T, CFG, false>(a, in.sms, in.stream);
+}
+// Statistics for a finishing kernel of the multi-launch path (in.stats_out: one part per row, or as many as `parts` says): dealt
+// out where the rows are many enough, else by the position split.
+cudaError_t launch_stats_only(const FusedPlan& in, size_t max_parts, int& parts) {
+  FlatArgs a;
+  parts = (!in.topk || flat_suits_topk(in)) ? flat_parts(in, in.topk ? 2 : max_parts) : 0;
+  if (parts == 0) { parts = 1; return plan_and_launch_fused(in); }
+  if (in.dtype == CSD_F32) return in.cfg ? launch_flat_stats<float, true>(in, parts, a) : launch_flat_stats<float, false>(in, parts, a);
+  return in.cfg ? launch_flat_stats<__nv_bfloat16, true>(in, parts, a) : launch_flat_stats<__nv_bfloat16, false>(in, parts, a);
 }
 
 // sampling: the degenerate round used by csd_sample_rows -- no draft positions (gamma = 0), one
@@ -907,7 +923,7 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
     sc.dtype = p.dtype; sc.top_k = p.top_k; sc.cfg = cfg; sc.topk = topk; sc.exact = p.dbg_G != nullptr;
     sc.sms = sms;
     sc.error_flag = no_workspace ? nullptr : reinterpret_cast<int*>((char*)p.workspace + lay.header_off);
-    if (topk && parts && rows >= sms) sc.dealt_ns = flat_topk_ns(fp);
+    if (topk && parts && 2 * rows >= sms) sc.dealt_ns = flat_topk_ns(fp);
     const cudaError_t e = slice_call(sc, plan_only != nullptr, stream, &sliced);
     if (e != cudaSuccess) return CSD_ERR_LAUNCH;
     if (sliced && !plan_only) return CSD_OK;
@@ -934,7 +950,7 @@ int verify_impl(const csd_params& p, int* plan_only = nullptr, bool sampling = f
     fp.allow_short_cut = false;   // the finishing kernel filters by the exact threshold
     fp.stats_out = sa.partials;
     fp.thr_out = topk ? se.thresholds : nullptr;
-    e = plan_and_launch_fused(fp);
+    e = launch_stats_only(fp, lay.max_parts, fa.parts);
     g_plan = several;
     if (e == cudaSuccess) {
       if (p.dtype == CSD_F32) e = cfg ? launch_finish<float, true>(fa, stream) : launch_finish<float, false>(fa, stream);
@@ -1224,9 +1240,8 @@ int csd_verify_tree(const csd_tree_params* pp) {
     fp.stats_out = sa.partials;
     fp.thr_out = topk ? se.thresholds : nullptr;
     fp.stream = stream;
-    e = plan_and_launch_fused(fp);
+    e = launch_stats_only(fp, lay.max_parts, fa.parts);
     g_plan = several;
-    fa.parts = 1;
     if (e == cudaSuccess) {
       if (p.dtype == CSD_F32) e = cfg ? launch_tree_finish<float, true>(ta, stream) : launch_tree_finish<float, false>(ta, stream);
       else e = cfg ? launch_tree_finish<__nv_bfloat16, true>(ta, stream) : launch_tree_finish<__nv_bfloat16, false>(ta, stream);

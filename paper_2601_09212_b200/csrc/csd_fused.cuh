@@ -192,8 +192,9 @@ struct FusedArgs {
   float4* records;      // with stats_out, not null: (m, s, logit of the drafted token if this slice holds it) instead,
   int v_offset;         //   for a slice of the vocabulary that begins at this token
   float* thr_out;       //   and its top-k threshold there (may be null), at row b * (T + gamma) + (target ? i : T + i)
-  float4* rows_out;     // top-k, not null: the rows of all sequences are dealt out to the blocks, rows_per_block each; stop after the
-  int rows_per_block;   //   streaming phase and write (m, s, threshold, logit of the drafted token or -inf if it is dropped) here
+  int rows_per_block;   // top-k, > 0: the rows of all sequences are dealt out to the blocks, this many each (csd_flat.cuh)
+  float4* rows_out;     // ... not null: stop after the streaming phase and write (m, s, threshold, logit of the drafted token
+                        //   or -inf if it is dropped) here, in the order of stats_out
   int ordered;          // ordinary stream order: nothing of the call's inputs is read before everything ahead of it
                         // on the stream has completed
   int signal;           // let the next call's blocks in as soon as this call's have started (set by the host)
@@ -1528,7 +1529,7 @@ __device__ __forceinline__ void load_stage(const uint32_t base, const int n, con
 
 // RAGGED: V is not a whole number of stages, so the last stage of a row is partly filled (the host
 // picks the instance; without it the streaming loop has no bounds tests at all).  DEALT: all sequences' rows are dealt out to the
-// blocks, and the kernel stops with their results (FusedArgs::rows_out; an instance of its own, since its few instructions cost the
+// blocks, and the kernel stops with their results (FusedArgs::rows_per_block; an instance of its own, since its few instructions cost the
 // overlapping calls 0.5 %).
 template <typename T, bool CFG, bool RAGGED, int WL, bool DEALT>
 __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const FusedArgs a) {
@@ -2021,17 +2022,23 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
 
   // ================================= phase 2 ===========================================
   __syncthreads();
-  if (stats_only) {
-    write_row_stats<T, CFG>(a, sh, sm.rs, tid, kTopkThreads, sm.abort != 0);
-    return;
-  }
-  if (DEALT) {
+  if (DEALT) {   // (the call is in stream order: it has waited for the operation ahead of it)
     for (int r = tid; r < n_rows && r < kBlockRows; r += kTopkThreads) {
       int b, which, i;
       local_row(sh, row0 + r, f.gamma, b, which, i);
+      const int64_t row_id = (int64_t)b * sh.rows_per_seq + (which == 0 ? i : f.T + i);
       const float2 ms = sm.abort ? make_float2(__int_as_float(0x7fc00000), 0.0f) : sm.rs.ms[r];   // (reads as unusable)
-      a.rows_out[(int64_t)b * sh.rows_per_seq + (which == 0 ? i : f.T + i)] = make_float4(ms.x, ms.y, sm.rs.thr[r], sm.rs.tokz[r]);
+      if (a.rows_out) {
+        a.rows_out[row_id] = make_float4(ms.x, ms.y, sm.rs.thr[r], sm.rs.tokz[r]);
+      } else {
+        a.stats_out[row_id] = ms;
+        if (a.thr_out) a.thr_out[row_id] = sm.rs.thr[r];
+      }
     }
+    return;
+  }
+  if (stats_only) {
+    write_row_stats<T, CFG>(a, sh, sm.rs, tid, kTopkThreads, sm.abort != 0);
     return;
   }
   static_assert(sizeof(sm.list) >= kFinTiles * sizeof(double), "tile sums live in the list area");
