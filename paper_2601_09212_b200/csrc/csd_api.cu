@@ -558,6 +558,30 @@ struct FusedPlan {
   bool dealt = false;          // top-k: all rows dealt out (see FusedArgs), into rows_out or stats_out
   float4* rows_out = nullptr;
 };
+// Rows with top-k dealt out to one wave of blocks: `each` to all and one more to the first of them, which go to different SMs; or
+// the same number to as few blocks as that takes, where these are more than three to an SM already and the busiest SM would not
+// have an eighth fewer.  us a call, the same number / one more: 612 rows of 13.4 K bf16 27.9 / 23.4, 1921 guided of 48.5 K 144.7 / 127.9,
+// 1320 guided fp32 of 19.6 K (the same rows on the busiest SM, four blocks instead of three) 89.9 / 77.3; but 930 guided fp32 of 26.9 K
+// 56.6 / 58.2, 972 guided bf16 of 4.8 K 23.3 / 24.0.
+struct Deal {
+  long long blocks, each, more;
+  Deal(long long rows, int sms) {
+    const long long slots = (long long)kFlatTopkBlocks * sms;
+    lay(rows, rows < slots ? rows : slots);
+    if (more > 0) {
+      Deal even = *this;
+      even.lay(rows, (rows + each) / (each + 1));
+      if (even.blocks > 3LL * sms && 8 * of_sm(sms) >= 7 * even.of_sm(sms)) *this = even;
+    }
+  }
+  void lay(long long rows, long long n) { blocks = n; each = rows / n; more = rows - each * n; }
+  long long of_block() const { return each + (more > 0); }
+  long long of_sm(int sms) const {   // of the busiest
+    const long long k = (blocks + sms - 1) / sms, first = (more + sms - 1) / sms;
+    return k * each + (first < k ? first : k);
+  }
+};
+
 cudaError_t plan_and_launch_fused(const FusedPlan& in) {
   const int sms = in.sms, es = in.es, rows_per_seq = in.rows_per_seq;
   const bool cfg = in.cfg, topk = in.topk;
@@ -576,7 +600,7 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
     ua.records = in.records;
     ua.v_offset = in.v_offset;
     ua.rows_out = in.rows_out;
-    ua.rows_per_block = 0;
+    ua.rows_per_block = ua.blocks_with_more = 0;
     ua.wait_limit = g_wait_limit;
     ua.drop_first_copy = g_drop_first_copy == 1;
     // Blocks are aligned with sequences and positions.  For calls enqueued back to back a block owns a
@@ -657,10 +681,12 @@ cudaError_t plan_and_launch_fused(const FusedPlan& in) {
       ua.parts_per_row = (int)((cpr + cpp - 1) / cpp);
     }
     long long grid = c > 1 ? (long long)in.B * c : (in.B + spc - 1) / spc;
-    if (in.dealt) {   // one wave of four blocks per SM
+    if (in.dealt) {
       c = spc = 1;
-      ua.rows_per_block = (int)((in.rows + kFlatTopkBlocks * sms - 1) / (kFlatTopkBlocks * sms));
-      grid = (in.rows + ua.rows_per_block - 1) / ua.rows_per_block;
+      const Deal d(in.rows, sms);
+      ua.rows_per_block = (int)d.each;
+      ua.blocks_with_more = (int)d.more;
+      grid = d.blocks;
     }
     g_plan = Plan{2, (int)c, 0, 0, 0, rows_per_seq};
     ua.ctas_per_seq = (int)c;
@@ -717,13 +743,13 @@ bool flat_suits(const FusedPlan& in) {
   return r.flat + r.flat_sm * mean + r.flat_v * in.V < 0.98 * (r.split + r.split_sm * per_sm * block + r.split_block * block);
 }
 // The same with top-k, whose rows are dealt out whole: the rows of the busiest SM and those that one of its blocks takes one after
-// another.  Over 77 random calls (6 - 256 sequences) the calls that go this way took 0.75 of the split's time in the mean, one of
-// them 1.05; those with equal sums 1.02 - 1.18.
+// another, against the split's.  Of 77 random calls (6 - 256 sequences) those with a ratio of at most 0.83 took 0.54 - 0.96 of the split's
+// time, the others 0.96 - 1.18.
 bool flat_suits_topk(const FusedPlan& in) {
   const int c = position_split(in.B, in.gamma, in.fa.T, true, in.sms);
   const long long split_each = busiest_rows(in.gamma, in.fa.T, c), split = ((long long)in.B * c + in.sms - 1) / in.sms * split_each;
-  const long long slots = (long long)kFlatTopkBlocks * in.sms, each = (in.rows + slots - 1) / slots, blocks = (in.rows + each - 1) / each;
-  return (blocks + in.sms - 1) / in.sms * each + each < split + split_each;
+  const Deal d(in.rows, in.sms);
+  return 6 * (d.of_sm(in.sms) + d.of_block()) <= 5 * (split + split_each);
 }
 
 // What such a call should take, in ns: a fixed part, a rate over the logits that a block takes one after another, one over those of
@@ -731,8 +757,8 @@ bool flat_suits_topk(const FusedPlan& in) {
 // rows, whose sample is half as large, miss their guess too often.
 double flat_topk_ns(const FusedPlan& in) {
   if (in.dtype == CSD_F32 && in.cfg) return 0.0;
-  const long long slots = (long long)kFlatTopkBlocks * in.sms, each = (in.rows + slots - 1) / slots, blocks = (in.rows + each - 1) / each;
-  const double block = (double)each * in.V, sm = (double)((blocks + in.sms - 1) / in.sms) * block;
+  const Deal d(in.rows, in.sms);
+  const double each = (double)d.of_block(), block = each * in.V, sm = (double)d.of_sm(in.sms) * in.V;
   if (in.dtype == CSD_F32) return 4.8e3 + 0.284 * block + 0.069 * sm + 6.3e3 * each;
   return in.cfg ? 8.8e3 + 0.167 * block + 0.117 * sm + 3.1e3 * each : 8.4e3 + 0.104 * block + 0.097 * sm + 3.6e3 * each;
 }

@@ -192,7 +192,8 @@ struct FusedArgs {
   float4* records;      // with stats_out, not null: (m, s, logit of the drafted token if this slice holds it) instead,
   int v_offset;         //   for a slice of the vocabulary that begins at this token
   float* thr_out;       //   and its top-k threshold there (may be null), at row b * (T + gamma) + (target ? i : T + i)
-  int rows_per_block;   // top-k, > 0: the rows of all sequences are dealt out to the blocks, this many each (csd_flat.cuh)
+  int rows_per_block;   // top-k, > 0: the rows of all sequences are dealt out to the blocks, this many each (csd_flat.cuh) ...
+  int blocks_with_more; // ... and to this many, the first, one more
   float4* rows_out;     // ... not null: stop after the streaming phase and write (m, s, threshold, logit of the drafted token
                         //   or -inf if it is dropped) here, in the order of stats_out
   int ordered;          // ordinary stream order: nothing of the call's inputs is read before everything ahead of it
@@ -1577,8 +1578,8 @@ __global__ void __launch_bounds__(kTopkThreads, 4) verify_topk_kernel(const Fuse
   // this block's local rows (see block_share), or a run of all sequences' rows
   BlockShare sh = block_share(a);
   const bool stats_only = a.stats_out != nullptr;
-  const int row0 = DEALT ? a.rows_per_block * (int)blockIdx.x : 0;
-  if (DEALT) { sh.seq_begin = 0; sh.n_rows = max(0, min(a.rows_per_block, f.B * sh.rows_per_seq - row0)); }
+  const int row0 = DEALT ? a.rows_per_block * (int)blockIdx.x + min((int)blockIdx.x, a.blocks_with_more) : 0;
+  if (DEALT) { sh.seq_begin = 0; sh.n_rows = a.rows_per_block + ((int)blockIdx.x < a.blocks_with_more ? 1 : 0); }
   const int n_rows = sh.n_rows;
   const int n_chunks = n_rows * cpr;
 

@@ -131,3 +131,23 @@ def test_wait_that_runs_out_is_reported():
     clean = run_gpu(w, want_dbg=False, workspace=ws)
     for key in ("tokens", "accept_len", "status"):
         assert np.array_equal(clean[key], good[key]), key
+
+
+@pytest.mark.parametrize("kw", [
+    dict(B=76, gamma=6, V=16388, dtype=W.F32, bonus_row=True),
+    dict(B=90, gamma=8, V=12296, dtype=W.BF16, cfg=True, cfg_scale=2.5, bonus_row=True),
+    dict(B=64, gamma=8, V=4104, dtype=W.BF16, cfg=True, cfg_scale=5.0, top_k=250, bonus_row=True),
+])
+def test_nothing_is_read_beside_a_row(kw):
+    """The bounds-checked build, with tokens out of range among the drafted ones."""
+    w = _make(kw)
+    w.draft_tokens[::3, 1] = kw["V"]
+    w.draft_tokens[1::3, 0] = -1
+    want = run_gpu(w, want_dbg=False)
+    with csd.checked_library() as report:
+        before = report()[0]
+        got = run_gpu(w, want_dbg=False)
+        assert _dealt()
+        assert report()[0] == before, report()
+    for key in ("tokens", "accept_len", "status"):
+        assert np.array_equal(got[key], want[key]), key
