@@ -721,6 +721,17 @@ cudaError_t launch_flat_finish(FlatArgs& a, int sms, cudaStream_t stream) {
   g_plan = Plan{2, c, 0, f.parts, 0, f.T + f.gamma};
   return launch_after(flat_finish_kernel<T, CFG, FILT>, a, (unsigned)(f.B * c), kFlatThreads, (size_t)tiles * sizeof(double), stream, c);
 }
+// Pieces of a single stage gain less, and the fit is off for them: of 25 such calls fp32 rows of 10 K and more took 0.84 - 1.02 of the
+// split's time, shorter ones and bf16 0.94 - 1.09.  With this rule 14 of 36 random calls of 13 - 32 MB go this way, in 0.78 - 1.03 of it
+// (16 sequences of 8 positions, 16 K: 15.0 and 14.6).
+long long flat_stages_per_row(const FusedPlan& in) {
+  const int eps = (in.dtype == CSD_F32 ? kFlatStageBytes<float> : kFlatStageBytes<__nv_bfloat16>) / (in.es * (in.cfg ? 2 : 1));
+  return (in.V + eps - 1) / eps;
+}
+long long flat_least(const FusedPlan& in) {   // stages of the smallest piece
+  return in.rows * flat_stages_per_row(in) / ((long long)kFlatBlocks * in.sms * kPlainWarps);
+}
+bool flat_short(const FusedPlan& in) { return in.dtype == CSD_F32 && !in.cfg && in.V >= 10240 && flat_least(in) == 1; }
 // Whether a call should go that way rather than by the position split (plan_and_launch_fused, c blocks to a sequence).  Expected
 // times in ns: of the split a rate over the logits of the busiest SM and one over those of a block, of this form a rate over
 // the GPU's average and the draw's, and the launch more in its fixed part.  Fitted to 300 random calls on inputs that
@@ -740,7 +751,7 @@ bool flat_suits(const FusedPlan& in) {
   const double block = (double)busiest_rows(in.gamma, in.fa.T, c) * in.V;
   const double per_sm = (double)(((long long)in.B * c + in.sms - 1) / in.sms);
   const double mean = (double)in.rows * in.V / in.sms;
-  return r.flat + r.flat_sm * mean + r.flat_v * in.V < 0.98 * (r.split + r.split_sm * per_sm * block + r.split_block * block);
+  return r.flat + r.flat_sm * mean + r.flat_v * in.V < (flat_short(in) ? 1.03 : 0.98) * (r.split + r.split_sm * per_sm * block + r.split_block * block);
 }
 // The same with top-k, whose rows are dealt out whole: the rows of the busiest SM and those that one of its blocks takes one after
 // another, against the split's.  Of 77 random calls (6 - 256 sequences) those with a ratio of at most 0.83 took 0.54 - 0.96 of the split's
@@ -766,9 +777,8 @@ double flat_topk_ns(const FusedPlan& in) {
 // The slots that a row's pieces need in the workspace (top-k: whose rows are not cut, 1); 0 if the call cannot go that way.
 int flat_parts(const FusedPlan& in, size_t max_parts) {
   if (in.topk) return max_parts >= 2 && in.rows <= (long long)kBlockRows * kFlatTopkBlocks * in.sms ? 1 : 0;   // (16 bytes a row; rows of a block)
-  const int eps = (in.dtype == CSD_F32 ? kFlatStageBytes<float> : kFlatStageBytes<__nv_bfloat16>) / (in.es * (in.cfg ? 2 : 1));
-  const long long spr = (in.V + eps - 1) / eps, least = in.rows * spr / ((long long)kFlatBlocks * in.sms * kPlainWarps);   // stages of a piece
-  if (least < 2) return 0;   // (a copy under the arithmetic of the stage before it; shorter pieces gained nothing)
+  const long long spr = flat_stages_per_row(in), least = flat_least(in);
+  if (least < 1 || (least == 1 && !flat_short(in))) return 0;
   const long long parts = spr < 2 ? 1 : (spr - 2) / least + 2;   // as many as a row can be cut into
   return parts <= (long long)max_parts ? (int)parts : 0;
 }
