@@ -48,7 +48,7 @@ FALLBACK_HBM_GBS = 6650.0
 # DRAM traffic of one launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum,
 # one ncu capture of this workload).  Reported only while the kernel sources still have the digest
 # the capture was taken with; null otherwise.
-NCU_TRAFFIC = {"sources_sha256": "e00f6d673ea05db9", "workload": "C3", "bytes_per_launch": 67206400}
+NCU_TRAFFIC = {"sources_sha256": "63b3f5ba3e960181", "workload": "C3", "bytes_per_launch": 67874560}
 
 
 def sources_digest() -> str:
