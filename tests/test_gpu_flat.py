@@ -12,8 +12,10 @@ if not torch.cuda.is_available():
 
 import paper_2601_09212_b200 as csd
 from paper_2601_09212_b200 import workloads as W
-from gpu_util import check, run_gpu
+from gpu_util import TOL, check, run_gpu, run_oracle
 from oracle.compare import compare
+from test_gpu_similar import neighbour_table, run_similar
+from test_gpu_tree import compare_tree, run_tree_gpu, run_tree_oracle
 
 DEV = "cuda"
 
@@ -151,3 +153,29 @@ def test_nothing_is_read_beside_a_row(kw):
         assert report()[0] == before, report()
     for key in ("tokens", "accept_len", "status"):
         assert np.array_equal(got[key], want[key]), key
+
+
+@pytest.mark.parametrize("B,kw", [
+    (300, dict(V=2052, dtype=W.F32)),                                          # more trees than the GPU has SMs: rows in two pieces
+    (170, dict(V=4104, dtype=W.BF16, cfg=True, cfg_scale=2.0)),                # ... in three
+    (200, dict(V=2056, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=150)),     # whole rows, several to a block
+    (200, dict(V=2048, dtype=W.F32, top_k=200)),
+])
+def test_statistics_of_trees(B, kw):
+    parent = W.static_tree([4, 3, 2, 2])
+    w = W.make_tree(parent, B=B, rho=0.9, schedule=csd.csd_make_schedule(1, 1.3, 0.5, 4), seed=kw["V"], device=DEV, **kw)
+    n_near, bad = compare_tree(w, run_tree_gpu(w), run_tree_oracle(w))
+    assert not bad, bad[:4]
+    assert n_near <= 2
+
+
+@pytest.mark.parametrize("kw", [dict(B=300, V=4100, dtype=W.F32), dict(B=150, V=2056, dtype=W.BF16, cfg=True, cfg_scale=3.0, top_k=150)])
+def test_statistics_of_the_similarity_relaxation(kw):
+    L = 8
+    w = W.make("t", gamma=L, rho=0.85, schedule=csd.csd_make_schedule(1, 1.2, 0.6, L), seed=9, device=DEV, **kw)
+    nbr = neighbour_table(w.V, 4, seed=4)
+    got = run_similar(w, nbr, 2.0)
+    h, ref = run_oracle(w, neighbours=nbr, nbr_lambda=2.0)
+    rep = compare(ref, got["tokens"], got["accept_len"], h["draft_tokens"], h["uniforms"], status=got["status"], p=got["p"], q=got["q"],
+                  f=got["f"], tol=TOL[w.dtype])
+    assert rep.ok, rep.summary()
